@@ -96,6 +96,11 @@ static RowParams<T> row_params(Geometry* g, const double* in, double* out, const
   rp.io_off = 0;
   rp.trans = 0;
   rp.fsel = 0;
+  int cnt;
+  rp.bands_in = rp.bands_out = touched_bands(g, rp.R, &cnt, &rp.band0_in);
+  rp.band0_out = rp.band0_in;
+  rp.nbands = cnt;
+  rp.on_out = g->row_on;
   rp.grid_in = nullptr;
   rp.jump = g->bc == IBDL_BC_NEUMANN ? -0.5 : 0.5;
   rp.aug = g->naug > 0;
@@ -122,6 +127,7 @@ static ColParams<T> col_params(Geometry* g, const int* stop) {
   cp.tw = static_cast<const cplx<T>*>(Slot2<T>::tw(g));
   cp.stop = stop;
   cp.err = g->err_dev;
+  cp.on_in = cp.on_out = g->row_on;
   return cp;
 }
 
@@ -178,8 +184,9 @@ static ibdl_status launch_for_size(int lg, Geometry* g, const RowParams<T>& rp, 
 }
 
 // run_op mode bits: RUN_LAPLACE solves the plain Laplace problem (λ → 0) without the completed
-// method's terms; RUN_NO_AUG only drops those terms
-enum { RUN_LAPLACE = 1, RUN_NO_AUG = 2 };
+// method's terms; RUN_NO_AUG only drops those terms; RUN_TOUCHED: a grid output is wanted only on
+// the rows that the points' stencils meet (the others are not written)
+enum { RUN_LAPLACE = 1, RUN_NO_AUG = 2, RUN_TOUCHED = 4 };
 
 template <typename T, int OP>
 static ibdl_status run_op(Geometry* g, const double* in, double* out, cudaStream_t s, const int* stop,
@@ -207,26 +214,40 @@ static ibdl_status run_op(Geometry* g, const double* in, double* out, cudaStream
     rp.aug = 0;
     rp.eta_src = 0;
   }
+  // grid input fills every row, and a grid output (unless only its touched rows are wanted) needs them
+  lc.units_in = lc.units_out = rp.nbands;
+  if (grid_in) {
+    rp.bands_in = nullptr;
+    rp.band0_in = 0;
+    cp.on_in = nullptr;
+    lc.units_in = g->n / rp.R;
+  }
+  if (grid && !(mode & RUN_TOUCHED)) {
+    rp.bands_out = nullptr;
+    rp.band0_out = 0;
+    rp.on_out = cp.on_out = nullptr;
+    lc.units_out = g->n / rp.R;
+  }
   return launch_for_size<T, OP, kMinL2d>(log2i(g->n), g, rp, cp, lc, s);
 }
 
 template <typename T>
 static ibdl_status apply_t(Geometry* g, const double* Q, double* Y, cudaStream_t s, const int* stop, double* grid,
-                           const int* idx = nullptr, int vstride = 0, int op = OPK_A) {
+                           const int* idx = nullptr, int vstride = 0, int op = OPK_A, int mode = 0) {
+  auto run = [&](auto opc, int trans) {
+    return run_op<T, decltype(opc)::value>(g, Q, Y, s, stop, grid, idx, vstride, trans, nullptr, mode);
+  };
+  const bool an = g->dipole == IBDL_DIPOLE_ANALYTIC;
   if (op == OPK_AT) {
     if (g->pde == IBDL_PDE_STOKES) {
-      if (g->dipole != IBDL_DIPOLE_ANALYTIC)
-        return fail(IBDL_ERR_UNSUPPORTED, "Stokes transpose: analytic dipole only");
-      return run_op<T, OP_STOKES_T>(g, Q, Y, s, stop, grid, idx, vstride);
+      if (!an) return fail(IBDL_ERR_UNSUPPORTED, "Stokes transpose: analytic dipole only");
+      return run(std::integral_constant<int, OP_STOKES_T>(), 0);
     }
-    return g->dipole == IBDL_DIPOLE_ANALYTIC ? run_op<T, OP_ADJ_AN>(g, Q, Y, s, stop, grid, idx, vstride, 1)
-                                             : run_op<T, OP_ADJ_SD>(g, Q, Y, s, stop, grid, idx, vstride, 1);
+    return an ? run(std::integral_constant<int, OP_ADJ_AN>(), 1) : run(std::integral_constant<int, OP_ADJ_SD>(), 1);
   }
   if (g->pde == IBDL_PDE_STOKES)
-    return g->dipole == IBDL_DIPOLE_ANALYTIC ? run_op<T, OP_STOKES_AN>(g, Q, Y, s, stop, grid, idx, vstride)
-                                             : run_op<T, OP_STOKES_SD>(g, Q, Y, s, stop, grid, idx, vstride);
-  return g->dipole == IBDL_DIPOLE_ANALYTIC ? run_op<T, OP_SCALAR_AN>(g, Q, Y, s, stop, grid, idx, vstride)
-                                           : run_op<T, OP_SCALAR_SD>(g, Q, Y, s, stop, grid, idx, vstride);
+    return an ? run(std::integral_constant<int, OP_STOKES_AN>(), 0) : run(std::integral_constant<int, OP_STOKES_SD>(), 0);
+  return an ? run(std::integral_constant<int, OP_SCALAR_AN>(), 0) : run(std::integral_constant<int, OP_SCALAR_SD>(), 0);
 }
 
 // Y = A Q with Q = V + (*idx)·nd and Y = V + (*idx + 1)·nd read on the device (Krylov basis)
@@ -246,10 +267,11 @@ ibdl_status apply_2d(Geometry* g, int precision, const double* Q, double* Y, cud
 }
 
 // u = K[sources(Q)] (the forward op's grid field: c fields) and v = Kᵀψ, ψ_l = Σ_j λ_{l,j} Φ(x − X_j)
-// (the transpose op's grid field: 1 field scalar, v_s and v_g Stokes), FP64 on [·][n][n]
+// (the transpose op's grid field: 1 field scalar, v_s and v_g Stokes), FP64 on [·][n][n]; only the
+// rows of the points' stencils are written (the boundary derivatives read no others)
 ibdl_status field_pair_2d(Geometry* g, const double* Q, const double* lam, double* u, double* v, cudaStream_t s) {
-  IBDL_TRY(apply_t<double>(g, Q, g->tmp_m, s, nullptr, u));
-  return apply_t<double>(g, lam, g->tmp_m, s, nullptr, v, nullptr, 0, OPK_AT);
+  IBDL_TRY(apply_t<double>(g, Q, g->tmp_m, s, nullptr, u, nullptr, 0, OPK_A, RUN_TOUCHED));
+  return apply_t<double>(g, lam, g->tmp_m, s, nullptr, v, nullptr, 0, OPK_AT, RUN_TOUCHED);
 }
 
 // Z = S*(−L⁻¹)(S V) (scalar PDE)
@@ -537,7 +559,7 @@ static ibdl_status batch_prepare_t(Batch* B, const int* kptr /* device &st[b].k,
     for (int b = 0; b < B->count; ++b) {
       Geometry* g = B->geoms[b];
       if (log2i(g->n) != L) continue;
-      for (int u = 0; u < g->n / g->rows_per_cta[pi]; ++u) ru.push_back(make_int2(b, u));
+      for (int u = 0; u < user[b].nbands; ++u) ru.push_back(make_int2(b, u));
       for (int u = 0; u < (g->n / 2) / g->cols_per_cta[pi]; ++u) cu.push_back(make_int2(b, u));
     }
     z.row_count = (int)ru.size() - z.row_start;

@@ -196,6 +196,13 @@ struct RowParams {
   double hd;              // h^d
   PT eta_src;             // weight of the ηSQ source: η (scalar) or η/μ (Stokes, projected part)
   int fsel;               // one-field launches: the field this launch spreads or interpolates
+  // the bands some stencil meets (NULL: every band), for the spread and for the gather, and the
+  // rows whose spectra the gather needs (see touched rows below; NULL: every row)
+  const int* bands_in;
+  const int* bands_out;
+  int band0_in, band0_out;  // without a list: the first band (the others follow it, wrapped)
+  const unsigned char* on_out;
+  int nbands;  // batched launches: bands this problem's row kernels run
 };
 
 template <typename T>
@@ -221,7 +228,24 @@ struct ColParams {
   const cplx<T>* tw;
   const int* stop;
   int* err;  // the staged column pass sets it to 1 when a bounded wait runs out
+  const unsigned char* on_in;   // rows the spread wrote (NULL: every row; the others are zero)
+  const unsigned char* on_out;  // rows the last kernel reads (NULL: every row)
 };
+
+// Touched rows. A spread field is zero, and an interpolated field unused, on every row that no
+// point's stencil meets: outside the curve's extent in y (40 % of the rows of the Stokes star,
+// half of a circle of radius a quarter of the box). Their row transforms, and the traffic of
+// their spectra, are left out: the row kernels run only the bands that some stencil meets (a list
+// per band height, fullest first so that the slowest CTAs start first; where they are one run of
+// at most 152 bands, which start together anyhow, the run's first band instead: the list's load
+// cost the 64² circle 0.25 µs in each row kernel), the column pass takes the other rows as zeros and stores no others. Rows count in pairs (2i, 2i + 1), the row kernels'
+// packed transforms: bit s of byte j < n/8 says whether the pair of row j + s·n/8 has a
+// touched row, which is the order in which a column lane holds its rows, so a lane reads one byte.
+// (Grid input and grid output take every row.)
+template <typename P>
+__device__ __forceinline__ unsigned rows_on(const unsigned char* on, const P& j) {
+  return on ? (unsigned)on[j] : 0xffu;
+}
 
 // Sorted points whose base row lies in the cell rows [r0 − 3, r0 + R) (mod n): at most two
 // contiguous ranges of the cell-sorted order.
@@ -307,8 +331,10 @@ __device__ __forceinline__ SpreadItem<typename Prec2<T>::PT> spread_item(const R
 // fit shared memory together: the band holds that field only, and the first launch (field 0)
 // also writes the jump term and the completed method's rows.
 template <typename T, int OP, int L, bool PF = true, bool SPLIT = false>
-__device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int unit, int nunits,
+__device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int ord, int nords,
                                                    unsigned char* smem_raw) {
+  // the band (ord of nords in this launch)
+  const int unit = p.bands_in ? p.bands_in[ord] : (ord + p.band0_in) & (p.n / p.R - 1);
   constexpr int NIN = Traits<OP>::NIN;
   constexpr int NB = SPLIT ? 1 : NIN;  // fields held in shared memory
   constexpr int NC = Traits<OP>::C;
@@ -366,10 +392,10 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int un
   const bool first = !SPLIT || p.fsel == 0;
   // jump term: out = ±½·in (the gather kernel adds S*u afterwards); none for grid input
   if (!p.grid_in && first)
-    for (int i = unit * blockDim.x + threadIdx.x; i < NC * M; i += nunits * blockDim.x)
+    for (int i = ord * blockDim.x + threadIdx.x; i < NC * M; i += nords * blockDim.x)
       pout[i] = p.jump * pin[i] + (p.aug ? pin[NC * M + i / M] : 0.0);
   __syncthreads();  // the accumulation buffer is cleared
-  if (p.aug && unit == 0 && first) {
+  if (p.aug && ord == 0 && first) {
     // constraint rows of the completed method: η Σ_i Δs_i Q_{l,i} (Δs = wscale·h^d); the block
     // size is a power of two (a partial warp below 32 threads), the partial sums go to the
     // reduction slots after the sequence buffers
@@ -686,6 +712,12 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
   // only read the same final flag.
   const bool stopped = p.stop && *p.stop;
   if (stopped) return;
+  unsigned oni[V], ono[V];  // the lane's rows to read and to store
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    oni[v] = rows_on(p.on_in, j0 + v * QT);
+    ono[v] = rows_on(p.on_out, j0 + v * QT);
+  }
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
 
@@ -697,7 +729,8 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) x[0][v][s] = p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, R)];
+        for (int s = 0; s < 8; ++s)
+          x[0][v][s] = (oni[v] >> s) & 1u ? p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, R)] : mk(T(0), T(0));
     }
     f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, active);
     if (packed) {
@@ -735,7 +768,8 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, R)] = x[0][v][s];
+        for (int s = 0; s < 8; ++s)
+          if ((ono[v] >> s) & 1u) p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, R)] = x[0][v][s];
     }
   } else {
     // forward transforms of the NIN input fields, results left in shared memory
@@ -749,7 +783,8 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) x[0][v][s] = p.spec[col_at_s<L>(f, j0 + v * QT, s, kx, R)];
+          for (int s = 0; s < 8; ++s)
+            x[0][v][s] = (oni[v] >> s) & 1u ? p.spec[col_at_s<L>(f, j0 + v * QT, s, kx, R)] : mk(T(0), T(0));
       }
       f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, act);
       if (act) {
@@ -832,7 +867,8 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) p.spec[col_at_s<L>(f, j0 + v * QT, s, kx, R)] = x[0][v][s];
+          for (int s = 0; s < 8; ++s)
+            if ((ono[v] >> s) & 1u) p.spec[col_at_s<L>(f, j0 + v * QT, s, kx, R)] = x[0][v][s];
       }
     }
   }
@@ -851,9 +887,12 @@ __device__ __forceinline__ void colpass1_load(const ColParams<T>& p, int unit, i
   const int kx = unit * p.C + c;
   if (active) {
 #pragma unroll
-    for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v) {
+      const unsigned on = rows_on(p.on_in, j0 + v * QT);
 #pragma unroll
-      for (int s = 0; s < 8; ++s) x[0][v][s] = p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, p.R)];
+      for (int s = 0; s < 8; ++s)
+        x[0][v][s] = (on >> s) & 1u ? p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, p.R)] : mk(T(0), T(0));
+    }
   }
 }
 
@@ -926,9 +965,12 @@ __global__ void __launch_bounds__(kMaxThreads2d) kbp_colpass(const ColParams<T>*
       f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, active);
       if (active) {
 #pragma unroll
-        for (int v = 0; v < V; ++v)
+        for (int v = 0; v < V; ++v) {
+          const unsigned on = rows_on(p.on_out, j0 + v * QT);
 #pragma unroll
-          for (int s = 0; s < 8; ++s) p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, p.R)] = x[0][v][s];
+          for (int s = 0; s < 8; ++s)
+            if ((on >> s) & 1u) p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, p.R)] = x[0][v][s];
+        }
       }
     }
     if (!more) break;
@@ -975,17 +1017,24 @@ __global__ void __launch_bounds__(kMaxThreads2d) k_colfft(ColParams<T> p, int fi
   cudaTriggerProgrammaticLaunchCompletion();
   cplx<T> x[1][V][8];
   if (active) {
+    // the forward transform reads the touched rows and writes every ky; the inverse the reverse
 #pragma unroll
-    for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v) {
+      const unsigned on = INV ? 0xffu : rows_on(p.on_in, j0 + v * QT);
 #pragma unroll
-      for (int s8 = 0; s8 < 8; ++s8) x[0][v][s8] = p.spec[col_at_s<L>(field, j0 + v * QT, s8, kx, R)];
+      for (int s8 = 0; s8 < 8; ++s8)
+        x[0][v][s8] = (on >> s8) & 1u ? p.spec[col_at_s<L>(field, j0 + v * QT, s8, kx, R)] : mk(T(0), T(0));
+    }
   }
   f8_fft<T, INV, L, V, 1>(x, sb, 0, j0, tw, active);
   if (active) {
 #pragma unroll
-    for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v) {
+      const unsigned on = INV ? rows_on(p.on_out, j0 + v * QT) : 0xffu;
 #pragma unroll
-      for (int s8 = 0; s8 < 8; ++s8) p.spec[col_at_s<L>(field, j0 + v * QT, s8, kx, R)] = x[0][v][s8];
+      for (int s8 = 0; s8 < 8; ++s8)
+        if ((on >> s8) & 1u) p.spec[col_at_s<L>(field, j0 + v * QT, s8, kx, R)] = x[0][v][s8];
+    }
   }
 }
 
@@ -1169,8 +1218,9 @@ __global__ void __launch_bounds__(kMaxThreads2d)
 #pragma unroll
           for (int v = 0; v < V; ++v) {
             const int b = xb(j0 + v * QT);
+            const unsigned on = rows_on(qv.on_in, j0 + v * QT);
 #pragma unroll
-            for (int s8 = 0; s8 < 8; ++s8) x[0][v][s8] = sx[b + s8 * Q * C];
+            for (int s8 = 0; s8 < 8; ++s8) x[0][v][s8] = (on >> s8) & 1u ? sx[b + s8 * Q * C] : mk(T(0), T(0));
           }
         }
         f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, active);
@@ -1208,9 +1258,12 @@ __global__ void __launch_bounds__(kMaxThreads2d)
         f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, active);
         if (active) {
 #pragma unroll
-          for (int v = 0; v < V; ++v)
+          for (int v = 0; v < V; ++v) {
+            const unsigned on = rows_on(qv.on_out, j0 + v * QT);
 #pragma unroll
-            for (int s8 = 0; s8 < 8; ++s8) qv.spec[col_at_s<L>(0, j0 + v * QT, s8, kx, R)] = x[0][v][s8];
+            for (int s8 = 0; s8 < 8; ++s8)
+              if ((on >> s8) & 1u) qv.spec[col_at_s<L>(0, j0 + v * QT, s8, kx, R)] = x[0][v][s8];
+          }
         }
       }
     } else {
@@ -1225,8 +1278,9 @@ __global__ void __launch_bounds__(kMaxThreads2d)
 #pragma unroll
             for (int v = 0; v < V; ++v) {
               const int b = f * n * C + xb(j0 + v * QT);
+              const unsigned on = rows_on(qv.on_in, j0 + v * QT);
 #pragma unroll
-              for (int s8 = 0; s8 < 8; ++s8) x[0][v][s8] = sx[b + s8 * Q * C];
+              for (int s8 = 0; s8 < 8; ++s8) x[0][v][s8] = (on >> s8) & 1u ? sx[b + s8 * Q * C] : mk(T(0), T(0));
             }
           }
           f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, act);
@@ -1312,9 +1366,12 @@ __global__ void __launch_bounds__(kMaxThreads2d)
           f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, act);
           if (act) {
 #pragma unroll
-            for (int v = 0; v < V; ++v)
+            for (int v = 0; v < V; ++v) {
+              const unsigned on = rows_on(qv.on_out, j0 + v * QT);
 #pragma unroll
-              for (int s8 = 0; s8 < 8; ++s8) qv.spec[col_at_s<L>(f, j0 + v * QT, s8, kx, R)] = x[0][v][s8];
+              for (int s8 = 0; s8 < 8; ++s8)
+                if ((on >> s8) & 1u) qv.spec[col_at_s<L>(f, j0 + v * QT, s8, kx, R)] = x[0][v][s8];
+            }
           }
         }
       }
@@ -1376,7 +1433,8 @@ __device__ __forceinline__ GatherItem<typename Prec2<T>::PT> gather_item(const R
 // SPLIT: one output field (p.fsel) per launch (see the spread kernel); its contribution to every
 // boundary component is added to Y (the operator is linear in the interpolated fields).
 template <typename T, int OP, int GMODE, int L, bool PF = true, bool SPLIT = false>
-__device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int unit, unsigned char* smem_raw) {
+__device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int ord, unsigned char* smem_raw) {
+  const int unit = p.bands_out ? p.bands_out[ord] : (ord + p.band0_out) & (p.n / p.R - 1);
   constexpr int NOUT = Traits<OP>::NOUT;
   constexpr int NB = SPLIT ? 1 : NOUT;  // fields held in shared memory
   using CF = Cfg2<T, L, NB>;
@@ -1395,6 +1453,9 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int u
   typename CF::TW tw[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) tw[v].load(p.tw, j0 + v * QT);
+  // whether this lane's row pair is touched (else its spectra are not read: the transform of zeros)
+  const int prow = r0 + 2 * rp;
+  const bool pair_on = active && ((rows_on(p.on_out, prow & (Q - 1)) >> (prow / Q)) & 1u);
   // the points whose stencil meets the band and this thread's first work item (4 per point),
   // loaded before the wait: the point tables are constant
   const PointRanges pr = band_points(p.cell_start, n, r0, R);
@@ -1423,7 +1484,8 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int u
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) x[0][v][s] = row_z<T, L>(p.spec, fs, r0, rp, R, j0 + v * QT + s * Q);
+        for (int s = 0; s < 8; ++s)
+          x[0][v][s] = pair_on ? row_z<T, L>(p.spec, fs, r0, rp, R, j0 + v * QT + s * Q) : mk(T(0), T(0));
     }
     f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, active);
     if (active) {
@@ -1580,7 +1642,8 @@ __global__ void __launch_bounds__(kMaxThreads2d) k_rowifft_gather1(RowParams<T> 
 // batched launches: one grid per stage covers every problem of a batch; CTA i runs work unit
 // units[i] = (problem, unit) with that problem's parameter block and transform size
 // ------------------------------------------------------------------------------------------
-// One batched kernel per stage and grid size: a CTA runs unit units[i] = (problem, unit) of a
+// One batched kernel per stage and grid size: a CTA runs unit units[i] = (problem, unit; row
+// kernels: the place in the problem's band list) of a
 // problem of this size with that problem's parameter block (the bodies load twiddles, symbol rows
 // and the first gather item where they are used, which keeps registers down and occupancy up).
 template <typename T, int OP, int L>
@@ -1591,7 +1654,7 @@ __global__ void __launch_bounds__(kMaxThreads2d) kb_spread_rowfft(const RowParam
   RowParams<T> p = P[u.x];
   p.in = in_base + p.io_off;
   p.out = out_base + p.io_off;
-  spread_rowfft_body<T, OP, L, false>(p, u.y, p.n / p.R, smem_raw);
+  spread_rowfft_body<T, OP, L, false>(p, u.y, p.nbands, smem_raw);
 }
 
 template <typename T, int OP, int L>
@@ -1636,6 +1699,7 @@ struct Launch2D {
   size_t smem_row, smem_col, smem_gather;
   int threads_row, threads_col, threads_gather;
   bool pdl;
+  int units_in, units_out;  // bands the spread and the gather run
   int grid_mode;            // G_INTERP or G_GRID
   bool split;               // one field per launch (the shapes above are those of one field)
 };

@@ -192,10 +192,10 @@ ibdl_status launch_apply_split_2d(Geometry* g, const RowParams<T>& rp, const Col
     IBDL_CUDA(opt_in_smem(k_spread_rowfft1<T, OP, L>, d1));
     for (int f = 0; f < NIN; ++f) {
       r.fsel = f;
-      IBDL_CUDA(launch_k(k_spread_rowfft1<T, OP, L>, n / lc.R, lc.threads_row, lc.smem_row, s, lc.pdl, r));
+      IBDL_CUDA(launch_k(k_spread_rowfft1<T, OP, L>, lc.units_in, lc.threads_row, lc.smem_row, s, lc.pdl, r));
     }
   } else {
-    IBDL_CUDA(launch_k(k_spread_rowfft<T, OP, L>, n / lc.R, lc.threads_row, lc.smem_row, s, lc.pdl, rp));
+    IBDL_CUDA(launch_k(k_spread_rowfft<T, OP, L>, lc.units_in, lc.threads_row, lc.smem_row, s, lc.pdl, rp));
   }
   if (g->timing) timing_mark(g, s, st0);
   IBDL_CUDA(opt_in_smem(k_colfft<T, L, false>, d2));
@@ -213,7 +213,7 @@ ibdl_status launch_apply_split_2d(Geometry* g, const RowParams<T>& rp, const Col
         IBDL_CUDA(opt_in_smem(k_rowifft_gather1<T, OP, G_GRID, L>, d4));
         for (int f = 0; f < NOUT; ++f) {
           r.fsel = f;
-          IBDL_CUDA(launch_k(k_rowifft_gather1<T, OP, G_GRID, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s,
+          IBDL_CUDA(launch_k(k_rowifft_gather1<T, OP, G_GRID, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s,
                              lc.pdl, r));
         }
       } else {
@@ -223,20 +223,20 @@ ibdl_status launch_apply_split_2d(Geometry* g, const RowParams<T>& rp, const Col
       IBDL_CUDA(opt_in_smem(k_rowifft_gather1<T, OP, G_INTERP, L>, d5));
       for (int f = 0; f < NOUT; ++f) {
         r.fsel = f;
-        IBDL_CUDA(launch_k(k_rowifft_gather1<T, OP, G_INTERP, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s,
+        IBDL_CUDA(launch_k(k_rowifft_gather1<T, OP, G_INTERP, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s,
                            lc.pdl, r));
       }
     }
   } else {
     if constexpr (std::is_same<T, ff>::value) {
       if (lc.grid_mode == G_GRID) return fail(IBDL_ERR_UNSUPPORTED, "float-float grid output");
-      IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s, lc.pdl,
+      IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s, lc.pdl,
                          rp));
     } else if (lc.grid_mode == G_GRID) {
-      IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_GRID, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s, lc.pdl,
+      IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_GRID, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s, lc.pdl,
                          rp));
     } else {
-      IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s, lc.pdl,
+      IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s, lc.pdl,
                          rp));
     }
   }
@@ -257,7 +257,7 @@ ibdl_status launch_apply_2d(Geometry* g, const RowParams<T>& rp, const ColParams
   }
   const int st0 = pi ? IBDL_STAGE_SPREAD_ROWFFT_FP32 : IBDL_STAGE_SPREAD_ROWFFT_FP64;
   if (g->timing) timing_mark(g, s, -1);
-  IBDL_CUDA(launch_k(k_spread_rowfft<T, OP, L>, n / lc.R, lc.threads_row, lc.smem_row, s, lc.pdl, rp));
+  IBDL_CUDA(launch_k(k_spread_rowfft<T, OP, L>, lc.units_in, lc.threads_row, lc.smem_row, s, lc.pdl, rp));
   if (g->timing) timing_mark(g, s, st0);
   bool staged = false;
   if constexpr (std::is_same<T, float>::value) {
@@ -270,13 +270,13 @@ ibdl_status launch_apply_2d(Geometry* g, const RowParams<T>& rp, const ColParams
   if constexpr (std::is_same<T, ff>::value) {
     // float-float serves boundary applications only (the refinement residual)
     if (lc.grid_mode == G_GRID) return fail(IBDL_ERR_UNSUPPORTED, "float-float grid output");
-    IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s, lc.pdl,
+    IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s, lc.pdl,
                        rp));
   } else if (lc.grid_mode == G_GRID) {
-    IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_GRID, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s, lc.pdl,
+    IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_GRID, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s, lc.pdl,
                        rp));
   } else {
-    IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, n / lc.R, lc.threads_gather, lc.smem_gather, s, lc.pdl,
+    IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L>, lc.units_out, lc.threads_gather, lc.smem_gather, s, lc.pdl,
                        rp));
   }
   if (g->timing) timing_mark(g, s, st0 + 2);

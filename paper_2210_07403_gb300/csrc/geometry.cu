@@ -1,7 +1,9 @@
 // Geometry set-up (once per boundary): validation, stencil cells, counting sort of the points
 // by cell, per-point kernel tables in FP64 and FP32, FFT twiddles and per-axis Fourier symbols.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "ff.cuh"
@@ -211,12 +213,52 @@ static ibdl_status dalloc(P** p, size_t bytes) {
   return IBDL_OK;
 }
 
+// The rows some stencil meets (a point of base row b meets rows b … b + 3, wrapped) and the bands
+// that hold such rows, from the cell counts (2-D; read back once per geometry).
+static ibdl_status touched_rows_2d(Geometry* g) {
+  const int n = g->n, Q = n / 8;
+  std::vector<int> start(n + 1);
+  IBDL_CUDA(cudaMemcpy(start.data(), g->cell_start, sizeof(int) * (n + 1), cudaMemcpyDeviceToHost));
+  auto points = [&](int r0, int R) {  // points whose stencils meet the rows [r0, r0 + R)
+    int c = 0;
+    for (int b = r0 - 3; b < r0 + R; ++b) c += start[(b & (n - 1)) + 1] - start[b & (n - 1)];
+    return c;
+  };
+  std::vector<unsigned char> on(Q, 0);
+  for (int m = 0; m < n; ++m)
+    if (points(m & ~1, 2) > 0) on[m & (Q - 1)] |= (unsigned char)(1u << (m / Q));
+  std::vector<int> lists;
+  std::vector<std::pair<int, int>> band;  // (−points, band)
+  for (int r = 1, R = 2; R <= n / 2; ++r, R *= 2) {
+    band.clear();
+    for (int u = 0; u < n / R; ++u)
+      if (const int c = points(u * R, R)) band.push_back({-c, u});
+    // one run (at most one band whose predecessor is off) of at most 152 bands, a CTA per SM
+    int starts = 0, first = 0;
+    for (const auto& b : band)
+      if (points(b.second * R - R, R) == 0) {
+        ++starts;
+        first = b.second;
+      }
+    g->band_first[r] = starts <= 1 && band.size() <= 152 ? first : -1;
+    std::sort(band.begin(), band.end());
+    g->band_off[r] = (int)lists.size();
+    g->band_cnt[r] = (int)band.size();
+    for (const auto& b : band) lists.push_back(b.second);
+  }
+  IBDL_TRY(dalloc(&g->row_on, Q));
+  IBDL_TRY(dalloc(&g->bands, sizeof(int) * lists.size()));
+  IBDL_CUDA(cudaMemcpy(g->row_on, on.data(), Q, cudaMemcpyHostToDevice));
+  IBDL_CUDA(cudaMemcpy(g->bands, lists.data(), sizeof(int) * lists.size(), cudaMemcpyHostToDevice));
+  return IBDL_OK;
+}
+
 static void free_geometry(Geometry* g) {
   if (!g) return;
   void* ptrs[] = {g->perm, g->base, g->cell_start, g->t64.phi, g->t64.dphi, g->t64.wscale, g->t64.nrm,
                   g->t32.phi, g->t32.dphi, g->t32.wscale, g->t32.nrm, g->spec, g->tw64, g->tw32,
                   g->lap64, g->der64, g->lap32, g->der32, g->ubuf, g->tmp_m, g->V, g->gm, g->vec,
-                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff};
+                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->row_on, g->bands};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int i = 0; i < 4; ++i)
@@ -452,6 +494,7 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     GCUDA(cudaHostAlloc((void**)&g->err_host, sizeof(int), cudaHostAllocMapped));
     *g->err_host = 0;
     GCUDA(cudaHostGetDevicePointer((void**)&g->err_dev, g->err_host, 0));
+    if (dim == 2) GTRY(touched_rows_2d(g));
     GTRY(dim == 2 ? plan_2d(g) : plan_3d(g));
   }
   g->X64 = dX;  // kept: the near-boundary interpolation decides on the caller's coordinates

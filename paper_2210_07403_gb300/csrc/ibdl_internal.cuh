@@ -98,6 +98,12 @@ struct Geometry {
   int* base;       // [dim][M] base node per axis (sorted order), already wrapped to [0, n)
   int* cell_start; // [ncell + 1], cells = n^(dim-1) rows of constant (y, z) base
   int ncell;
+  // 2-D: the rows that some stencil meets, as bits in the column lanes' order, and for each band
+  // height 2^r the list of bands holding such rows, fullest first (apply2d_kernels.cuh; NULL: all)
+  unsigned char* row_on;  // [n/8]
+  int* bands;             // the lists of r = 1, 2, …, one after another
+  int band_off[14], band_cnt[14];
+  int band_first[14];     // ≥ 0: the bands are one run from this one on (wrapped), short enough to start at once
   PointTable<double> t64;
   PointTable<float> t32;
   double* ddphi64; // [dim][4][M] φ''(r)/h² in sorted order (boundary derivatives); may be NULL
@@ -302,6 +308,23 @@ inline ibdl_status take_device_error(Geometry* g) {
     return fail(IBDL_ERR_TIMEOUT, "a staged column pass gave up waiting for its shared-memory copies");
   }
   return IBDL_OK;
+}
+
+// the *cnt bands of R rows that some stencil meets: a device list of band numbers, or (NULL) the run
+// of bands that starts with *first
+inline const int* touched_bands(const Geometry* g, int R, int* cnt, int* first) {
+  const int r = __builtin_ctz(R > 0 ? R : 2);
+  *first = 0;
+  if (!g->bands) {
+    *cnt = R > 0 ? g->n / R : 0;
+    return nullptr;
+  }
+  *cnt = g->band_cnt[r];
+  if (g->band_first[r] >= 0) {
+    *first = g->band_first[r];
+    return nullptr;
+  }
+  return g->bands + g->band_off[r];
 }
 
 // length of a boundary vector of the (possibly augmented) system: c·M density values, then ū
