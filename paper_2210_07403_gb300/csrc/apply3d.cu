@@ -22,13 +22,13 @@ IBDL_DECLARE_3D(7)
 IBDL_DECLARE_3D(8)
 
 template <typename T, int OP, int L>
-static ibdl_status launch3_for_size(int lg, Geometry* g, const Row3Params& rp, const Col3Params& cp, int R, int C,
-                                    int Cz, bool grid, cudaStream_t s) {
+static ibdl_status launch3_for_size(int lg, Geometry* g, const Row3Params& rp, const Col3Params& cp,
+                                    const Launch3D& lc, cudaStream_t s) {
   if constexpr (L > 8) {
     return fail(IBDL_ERR_UNSUPPORTED, "3-D grid size outside 16 … 256");
   } else {
-    if (lg == L) return launch_apply_3d<T, OP, L>(g, rp, cp, R, C, Cz, grid, s);
-    return launch3_for_size<T, OP, L + 1>(lg, g, rp, cp, R, C, Cz, grid, s);
+    if (lg == L) return launch_apply_3d<T, OP, L>(g, rp, cp, lc, s);
+    return launch3_for_size<T, OP, L + 1>(lg, g, rp, cp, lc, s);
   }
 }
 
@@ -76,7 +76,7 @@ ibdl_status plan_3d(Geometry* g) {
 template <typename T, int OP>
 static ibdl_status run_op3(Geometry* g, const double* in, double* out, cudaStream_t s, const int* stop, double* grid,
                            const int* idx = nullptr, int vstride = 0, int trans = 0, bool laplace = false,
-                           const double* grid_in = nullptr) {
+                           const double* grid_in = nullptr, bool touched = false) {
   constexpr bool is_ff = std::is_same<T, ff>::value;
   const int pi = std::is_same<T, float>::value ? 1 : (is_ff ? 2 : 0);
   const int R = g->rows_per_cta[pi], C = g->cols_per_cta[pi], Cz = g->zcols_per_cta[pi];
@@ -123,19 +123,43 @@ static ibdl_status run_op3(Geometry* g, const double* in, double* out, cudaStrea
   cp.spec = g->spec;
   cp.tw = rp.tw;
   cp.stop = stop;
-  cp.nf = 1;  // (the launch sets the fields of each y pass)
-  return launch3_for_size<T, OP, 4>(rp.log2n, g, rp, cp, R, C, Cz, grid != nullptr, s);
+  cp.nf = 1;  // (the launch sets the fields and planes of each y pass)
+  // the touched bands, rows and planes; a grid input fills every row, and a grid output (unless only
+  // its touched rows are wanted) needs them
+  Launch3D lc = {R, C, Cz, n * (n / R), n * (n / R), n, n, grid != nullptr};
+  int cnt, first;
+  const int* bands = touched_bands(g, R, &cnt, &first);
+  rp.bands_in = rp.bands_out = nullptr;
+  rp.rows_out = cp.rows_in = cp.rows_out = cp.planes_in = cp.planes_out = nullptr;
+  cp.planes = g->planes;
+  if (!grid_in) {
+    rp.bands_in = bands;
+    cp.rows_in = g->row_on;
+    cp.planes_in = g->plane_on;
+    lc.bands_in = cnt;
+    lc.planes_in = g->nplanes;
+  }
+  if (!grid || touched) {
+    rp.bands_out = bands;
+    rp.rows_out = cp.rows_out = g->row_on;
+    cp.planes_out = g->plane_on;
+    lc.bands_out = cnt;
+    lc.planes_out = g->nplanes;
+  }
+  return launch3_for_size<T, OP, 4>(rp.log2n, g, rp, cp, lc, s);
 }
 
 template <typename T>
 static ibdl_status apply3_t(Geometry* g, const double* Q, double* Y, cudaStream_t s, const int* stop, double* grid,
-                            const int* idx = nullptr, int vstride = 0, int op = OPK_A) {
+                            const int* idx = nullptr, int vstride = 0, int op = OPK_A, bool touched = false) {
   if (g->pde != IBDL_PDE_SCALAR) return fail(IBDL_ERR_UNSUPPORTED, "3-D: scalar PDE only");
   if (op == OPK_AT)
-    return g->dipole == IBDL_DIPOLE_ANALYTIC ? run_op3<T, OP3_ADJ_AN>(g, Q, Y, s, stop, grid, idx, vstride, 1)
-                                             : run_op3<T, OP3_ADJ_SD>(g, Q, Y, s, stop, grid, idx, vstride, 1);
-  return g->dipole == IBDL_DIPOLE_ANALYTIC ? run_op3<T, OP3_SCALAR_AN>(g, Q, Y, s, stop, grid, idx, vstride)
-                                           : run_op3<T, OP3_SCALAR_SD>(g, Q, Y, s, stop, grid, idx, vstride);
+    return g->dipole == IBDL_DIPOLE_ANALYTIC
+               ? run_op3<T, OP3_ADJ_AN>(g, Q, Y, s, stop, grid, idx, vstride, 1, false, nullptr, touched)
+               : run_op3<T, OP3_ADJ_SD>(g, Q, Y, s, stop, grid, idx, vstride, 1, false, nullptr, touched);
+  return g->dipole == IBDL_DIPOLE_ANALYTIC
+             ? run_op3<T, OP3_SCALAR_AN>(g, Q, Y, s, stop, grid, idx, vstride, 0, false, nullptr, touched)
+             : run_op3<T, OP3_SCALAR_SD>(g, Q, Y, s, stop, grid, idx, vstride, 0, false, nullptr, touched);
 }
 
 ibdl_status apply_3d(Geometry* g, int precision, const double* Q, double* Y, cudaStream_t s, const int* stop,
@@ -152,10 +176,11 @@ ibdl_status apply_3d_indexed(Geometry* g, int precision, double* V, const int* i
                                 : apply3_t<double>(g, V, V, s, stop, nullptr, idx, nd, op);
 }
 
-// u = −L⁻¹S̃Q and v = −L⁻¹(Σ_j λ_j Φ(x − X_j)), FP64 on [n][n][n]
+// u = −L⁻¹S̃Q and v = −L⁻¹(Σ_j λ_j Φ(x − X_j)), FP64 on [n][n][n]; only the rows of the points' stencils
+// are written (the boundary derivatives read no others)
 ibdl_status field_pair_3d(Geometry* g, const double* Q, const double* lam, double* u, double* v, cudaStream_t s) {
-  IBDL_TRY(apply3_t<double>(g, Q, g->tmp_m, s, nullptr, u));
-  return apply3_t<double>(g, lam, g->tmp_m, s, nullptr, v, nullptr, 0, OPK_AT);
+  IBDL_TRY(apply3_t<double>(g, Q, g->tmp_m, s, nullptr, u, nullptr, 0, OPK_A, true));
+  return apply3_t<double>(g, lam, g->tmp_m, s, nullptr, v, nullptr, 0, OPK_AT, true);
 }
 
 // u = −Δ₀⁻¹S̃Q (mean-zero), the geometry's λ ignored

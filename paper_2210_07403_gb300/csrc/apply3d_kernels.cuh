@@ -179,6 +179,11 @@ struct Row3Params {
   // values multiplied by Δs/h³ in place of the spread's Δs/h³ · W⁻¹)
   int trans;
   double jump;  // jump term coefficient: ½ (Dirichlet) or −½ (Neumann)
+  // the bands some stencil meets, numbered z·(n/R) + band (NULL: every band), for the spread and for
+  // the gather, and the touched rows (NULL: every row; see touched rows below)
+  const int* bands_in;
+  const int* bands_out;
+  const unsigned char* rows_out;
   const double* grid_in;  // optional [NIN][n][n][n]: the row bands are read from it instead of spread
 };
 
@@ -191,7 +196,24 @@ struct Col3Params {
   void* spec;
   const void* tw;
   const int* stop;
+  // touched rows of each plane and touched planes, on entry and on exit (NULL: all), and the list of
+  // planes a y pass runs (NULL: all)
+  const unsigned char* rows_in;
+  const unsigned char* rows_out;
+  const unsigned char* planes_in;
+  const unsigned char* planes_out;
+  const int* planes;
 };
+
+// Touched rows. The spread field is zero, and the interpolated field unused, outside the rows (z, y)
+// that some point's stencil meets: a sphere of radius a quarter of the box meets a quarter of
+// the rows, in half of the planes. The row kernels run only the bands that hold such rows (fullest
+// first), the y passes only the planes that do, the column passes take the other rows and planes
+// as zeros and store no others. On the 128³ sphere that leaves 25 % of the row transforms and 54 %
+// of the y transforms. Bit s of byte j < n/8 of a mask is row (or plane) j + s·n/8, the order in
+// which a lane of a column transform holds them; rows count in the pairs (2i, 2i + 1) of the
+// row kernels' packed transforms.
+__device__ __forceinline__ unsigned mask3(const unsigned char* m, size_t j) { return m ? (unsigned)m[j] : 0xffu; }
 
 __device__ __forceinline__ void resolve_io3(const Row3Params& p, const double*& in, double*& out) {
   in = p.in;
@@ -273,7 +295,8 @@ __global__ void __launch_bounds__(kThreads3) k3_spread_rowfft(Row3Params p) {
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);  // the padded sequences (field, row pair)
   PT* acc = reinterpret_cast<PT*>(bufA);  // (the same bytes per complex element as cplx<T>)
   const int bands = n / R;
-  const int z = blockIdx.x / bands, y0 = (blockIdx.x - z * bands) * R;
+  const int unit = p.bands_in ? p.bands_in[blockIdx.x] : (int)blockIdx.x;
+  const int z = unit / bands, y0 = (unit - z * bands) * R;
   const double* pin;
   double* pout;
   resolve_io3(p, pin, pout);
@@ -383,12 +406,24 @@ template <typename T>
 struct YColumnIO {
   cplx<T>* spec;
   int n, nh, z, k0, lc, C;
+  int lq;             // log2(n/8): row m is bit m >> lq of the lane's masks
+  unsigned in, out;   // the lane's rows to read and to store
   __device__ __forceinline__ size_t at(int bi, int m) const {
     return (((size_t)(bi >> lc) * n + z) * n + m) * nh + k0 + (bi & (C - 1));
   }
-  __device__ __forceinline__ cplx<T> load(int bi, int m) const { return spec[at(bi, m)]; }
-  __device__ __forceinline__ void store(int bi, int m, cplx<T> v) const { spec[at(bi, m)] = v; }
+  __device__ __forceinline__ cplx<T> load(int bi, int m) const {
+    return (in >> (m >> lq)) & 1u ? spec[at(bi, m)] : mk(T(0), T(0));
+  }
+  __device__ __forceinline__ void store(int bi, int m, cplx<T> v) const {
+    if ((out >> (m >> lq)) & 1u) spec[at(bi, m)] = v;
+  }
 };
+
+// the lane of an interleaved column transform that this thread runs (fft3_run with IL)
+template <typename T, int L>
+__device__ __forceinline__ int lane3() {
+  return (int)threadIdx.x / (kThreads3 / Cfg3<T, L>::QT);
+}
 
 template <typename T, bool INV, int L>
 __global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
@@ -401,9 +436,14 @@ __global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
   constexpr int n = 1 << L, nh = n >> 1;
   const int C = p.C;
   const int groups = nh / C;
-  const int z = blockIdx.x / groups, k0 = (blockIdx.x - z * groups) * C;
+  const int zi = blockIdx.x / groups, k0 = (blockIdx.x - zi * groups) * C;
+  const int z = p.planes ? p.planes[zi] : zi;
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
-  const YColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, z, k0, p.lc, C};
+  // the forward pass reads the touched rows of its plane and writes every ky; the inverse the reverse
+  constexpr int Q = n / 8;
+  const int j0 = lane3<T, L>();
+  const unsigned in = INV ? 0xffu : mask3(p.rows_in, z * Q + j0), out = INV ? mask3(p.rows_out, z * Q + j0) : 0xffu;
+  const YColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, z, k0, p.lc, C, L - 3, in, out};
   fft3_run<T, INV, L, true>(bufA, p.nf * C, static_cast<const cplx<T>*>(p.tw), GlobLd3<YColumnIO<T>>{io},
                             GlobSt3<YColumnIO<T>>{io});
 }
@@ -416,16 +456,20 @@ template <typename T>
 struct ZColumnIO {
   cplx<T>* spec;
   int n, nh, ky1, ky2, k0, lc, C;
+  int lq;             // log2(n/8)
+  unsigned in, out;   // the lane's planes to read and to store
   __device__ __forceinline__ size_t at(int bi, int m) const {
     const int c = bi & (C - 1), fq = bi >> lc;
     const int f = fq >> 1, ky = (fq & 1) ? ky2 : ky1;
     return (((size_t)f * n + m) * n + ky) * nh + k0 + c;
   }
-  __device__ __forceinline__ cplx<T> load(int bi, int m) const { return spec[at(bi, m)]; }
+  __device__ __forceinline__ cplx<T> load(int bi, int m) const {
+    return (in >> (m >> lq)) & 1u ? spec[at(bi, m)] : mk(T(0), T(0));
+  }
   // with ky1 = ky2 the q = 1 slots alias the q = 0 column and carry no symbol: never stored
   __device__ __forceinline__ void store(int bi, int m, cplx<T> v) const {
     if (ky1 == ky2 && ((bi >> lc) & 1)) return;
-    spec[at(bi, m)] = v;
+    if ((out >> (m >> lq)) & 1u) spec[at(bi, m)] = v;
   }
 };
 
@@ -475,7 +519,9 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
     der1[i] = static_cast<const T*>(p.der1)[i];
   }
   __syncthreads();
-  const ZColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, ky1, ky2, k0, lc, C};
+  const int j0 = lane3<T, L>();
+  const ZColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, ky1, ky2, k0, lc, C, L - 3,
+                        mask3(p.planes_in, j0), mask3(p.planes_out, j0)};
   // with one column (ky = −ky) only the q = 0 sequences exist: sequence index bi maps to
   // (f·2 + 0)·C + c, so transform all 2·C slots per field and ignore q = 1 (it aliases q = 0)
   fft3_run<T, false, L, true>(bufA, NIN * 2 * C, twg, GlobLd3<ZColumnIO<T>>{io}, SmemSt3<T>());
@@ -542,8 +588,12 @@ template <typename T>
 struct RowZLoad3 {
   const cplx<T>* spec;
   int n, nh, row0, half, nrows;  // row0 = z·n + y0; field stride nrows rows
+  const unsigned char* rows;     // touched rows of this plane (NULL: all); the others' spectra are not read
+  int y0, lq;
   __device__ __forceinline__ cplx<T> load(int sq, int m) const {
     const int f = sq / half, j = sq - f * half;
+    const int y = y0 + 2 * j;
+    if (!((mask3(rows, y & ((1 << lq) - 1)) >> (y >> lq)) & 1u)) return mk(T(0), T(0));
     const size_t ra = ((size_t)f * nrows + row0 + 2 * j) * nh;
     const size_t rb = ra + nh;
     if (m == 0 || m == nh) {
@@ -577,8 +627,10 @@ __global__ void __launch_bounds__(kThreads3) k3_rowifft_gather(Row3Params p) {
   const PT* nrm = static_cast<const PT*>(p.nrm);
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
   const int bands = n / R;
-  const int z = blockIdx.x / bands, y0 = (blockIdx.x - z * bands) * R;
-  const RowZLoad3<T> zl{static_cast<const cplx<T>*>(p.spec), n, nh, z * n + y0, half, n * n};
+  const int unit = p.bands_out ? p.bands_out[blockIdx.x] : (int)blockIdx.x;
+  const int z = unit / bands, y0 = (unit - z * bands) * R;
+  const RowZLoad3<T> zl{static_cast<const cplx<T>*>(p.spec), n, nh, z * n + y0, half, n * n,
+                        p.rows_out ? p.rows_out + (size_t)z * (n / 8) : nullptr, y0, L - 3};
   fft3_run<T, true, L>(bufA, seqs, static_cast<const cplx<T>*>(p.tw), GlobLd3<RowZLoad3<T>>{zl}, SmemSt3<T>());
   __syncthreads();
   const T* u = reinterpret_cast<const T*>(bufA);
@@ -671,8 +723,14 @@ inline cudaError_t opt_in_smem3(K kernel, std::atomic<unsigned long long>& done)
   return e;
 }
 
-// The five kernels of one application at n = 2^L: rows R per band, C kx columns per y pass, Cz per
-// z pass; `grid` selects the grid output of the last kernel.
+// Launch of one application: rows R per band, C kx columns per y pass, Cz per z pass, the bands and
+// planes the row kernels and y passes run on the way in and out, and whether the last kernel writes
+// the grid.
+struct Launch3D {
+  int R, C, Cz;
+  int bands_in, bands_out, planes_in, planes_out;
+  bool grid;
+};
 // Programmatic dependent launch of an application's kernels (IBDL_NO_PDL=1 turns it off): a kernel
 // may launch once every CTA of the previous one has passed its wait, and it waits in turn before
 // it reads anything; the launch latency is taken while the previous kernel drains.
@@ -701,8 +759,9 @@ inline cudaError_t launch3(void (*kernel)(KArgs...), int grid, size_t smem, cuda
 }
 
 template <typename T, int OP, int L>
-ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp, const Col3Params& cp, int R, int C, int Cz,
-                            bool grid, cudaStream_t s) {
+ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp, const Col3Params& cp, const Launch3D& lc,
+                            cudaStream_t s) {
+  const int R = lc.R, C = lc.C, Cz = lc.Cz;
   constexpr int NIN = Traits3<OP>::NIN, NOUT = Traits3<OP>::NOUT, NMAX = NIN > NOUT ? NIN : NOUT;
   constexpr int n = 1 << L;
   constexpr bool f32 = std::is_same<T, float>::value;
@@ -713,25 +772,27 @@ ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp, const Col3Params&
   IBDL_CUDA(opt_in_smem3(k3_ypass<T, true, L>, d[3]));
   IBDL_CUDA(opt_in_smem3(k3_rowifft_gather<T, OP, G3_GRID, L>, d[4]));
   IBDL_CUDA(opt_in_smem3(k3_rowifft_gather<T, OP, G3_INTERP, L>, d[5]));
-  const int rows_grid = n * (n / R), col_grid = n * ((n / 2) / C), z_grid = (n / 2 + 1) * ((n / 2) / Cz);
+  const int groups = (n / 2) / C, z_grid = (n / 2 + 1) * ((n / 2) / Cz);
   const int st0 = f32 ? IBDL_STAGE_SPREAD_ROWFFT_FP32 : IBDL_STAGE_SPREAD_ROWFFT_FP64;
   if (g->timing) timing_mark(g, s, -1);
-  IBDL_CUDA(launch3(k3_spread_rowfft<T, OP, L>, rows_grid, smem_rows3<T>(n, NIN, R), s, rp));
+  IBDL_CUDA(launch3(k3_spread_rowfft<T, OP, L>, lc.bands_in, smem_rows3<T>(n, NIN, R), s, rp));
   if (g->timing) timing_mark(g, s, st0);
   Col3Params yp = cp;
   yp.nf = NIN;
-  IBDL_CUDA(launch3(k3_ypass<T, false, L>, col_grid, smem_y3<T>(n, NIN, C), s, yp));
+  yp.planes = cp.planes_in ? cp.planes : nullptr;
+  IBDL_CUDA(launch3(k3_ypass<T, false, L>, lc.planes_in * groups, smem_y3<T>(n, NIN, C), s, yp));
   Col3Params zp = cp;
   zp.C = Cz;
   zp.lc = __builtin_ctz(Cz);
   IBDL_CUDA(launch3(k3_zpass<T, OP, L>, z_grid, smem_z3<T>(n, NMAX, Cz), s, zp));
   yp.nf = NOUT;
-  IBDL_CUDA(launch3(k3_ypass<T, true, L>, col_grid, smem_y3<T>(n, NOUT, C), s, yp));
+  yp.planes = cp.planes_out ? cp.planes : nullptr;
+  IBDL_CUDA(launch3(k3_ypass<T, true, L>, lc.planes_out * groups, smem_y3<T>(n, NOUT, C), s, yp));
   if (g->timing) timing_mark(g, s, st0 + 1);
-  if (grid)
-    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_GRID, L>, rows_grid, smem_rows3<T>(n, NOUT, R), s, rp));
+  if (lc.grid)
+    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_GRID, L>, lc.bands_out, smem_rows3<T>(n, NOUT, R), s, rp));
   else
-    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_INTERP, L>, rows_grid, smem_rows3<T>(n, NOUT, R), s, rp));
+    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_INTERP, L>, lc.bands_out, smem_rows3<T>(n, NOUT, R), s, rp));
   if (g->timing) timing_mark(g, s, st0 + 2);
   g->launches += 5;
   IBDL_CUDA(cudaGetLastError());
@@ -741,11 +802,11 @@ ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp, const Col3Params&
 // every operator and grid arithmetic at one size (instantiated by apply3d_n<n>.cu)
 #define IBDL_3D_OPS(X, T, L) X(T, OP3_SCALAR_AN, L) X(T, OP3_SCALAR_SD, L) X(T, OP3_ADJ_AN, L) X(T, OP3_ADJ_SD, L)
 #define IBDL_3D_INST1(T, OP, L)                                                                          \
-  template ibdl_status launch_apply_3d<T, OP, L>(Geometry*, const Row3Params&, const Col3Params&, int, int, int, \
-                                                 bool, cudaStream_t);
+  template ibdl_status launch_apply_3d<T, OP, L>(Geometry*, const Row3Params&, const Col3Params&,        \
+                                                 const Launch3D&, cudaStream_t);
 #define IBDL_3D_DECL1(T, OP, L)                                                                                 \
-  extern template ibdl_status launch_apply_3d<T, OP, L>(Geometry*, const Row3Params&, const Col3Params&, int, int, \
-                                                        int, bool, cudaStream_t);
+  extern template ibdl_status launch_apply_3d<T, OP, L>(Geometry*, const Row3Params&, const Col3Params&,        \
+                                                        const Launch3D&, cudaStream_t);
 #define IBDL_INSTANTIATE_3D(L) IBDL_3D_OPS(IBDL_3D_INST1, double, L) IBDL_3D_OPS(IBDL_3D_INST1, float, L) IBDL_3D_OPS(IBDL_3D_INST1, ff, L)
 #define IBDL_DECLARE_3D(L) IBDL_3D_OPS(IBDL_3D_DECL1, double, L) IBDL_3D_OPS(IBDL_3D_DECL1, float, L) IBDL_3D_OPS(IBDL_3D_DECL1, ff, L)
 

@@ -213,43 +213,71 @@ static ibdl_status dalloc(P** p, size_t bytes) {
   return IBDL_OK;
 }
 
-// The rows some stencil meets (a point of base row b meets rows b … b + 3, wrapped) and the bands
-// that hold such rows, from the cell counts (2-D; read back once per geometry).
-static ibdl_status touched_rows_2d(Geometry* g) {
-  const int n = g->n, Q = n / 8;
-  std::vector<int> start(n + 1);
-  IBDL_CUDA(cudaMemcpy(start.data(), g->cell_start, sizeof(int) * (n + 1), cudaMemcpyDeviceToHost));
-  auto points = [&](int r0, int R) {  // points whose stencils meet the rows [r0, r0 + R)
+// The rows some stencil meets (a point of base row b meets rows b … b + 3, wrapped; in 3-D likewise
+// planes) and the bands that hold such rows, from the cell counts, read back once per geometry.
+static ibdl_status touched_rows(Geometry* g) {
+  const int n = g->n, Q = n / 8, planes = g->dim == 3 ? n : 1;
+  std::vector<int> start(g->ncell + 1);
+  IBDL_CUDA(cudaMemcpy(start.data(), g->cell_start, sizeof(int) * (g->ncell + 1), cudaMemcpyDeviceToHost));
+  // points whose stencils meet the rows [r0, r0 + R) (wrapped) of plane z
+  auto points = [&](int z, int r0, int R) {
     int c = 0;
-    for (int b = r0 - 3; b < r0 + R; ++b) c += start[(b & (n - 1)) + 1] - start[b & (n - 1)];
+    for (int dz = g->dim == 3 ? -3 : 0; dz <= 0; ++dz) {
+      const int* st = start.data() + (size_t)((z + dz) & (planes - 1)) * n;
+      const int lo = std::max(r0 - 3, 0);
+      c += st[r0 + R] - st[lo];
+      if (r0 < 3) c += st[n] - st[n + r0 - 3];
+    }
     return c;
   };
-  std::vector<unsigned char> on(Q, 0);
-  for (int m = 0; m < n; ++m)
-    if (points(m & ~1, 2) > 0) on[m & (Q - 1)] |= (unsigned char)(1u << (m / Q));
-  std::vector<int> lists;
+  std::vector<unsigned char> on((size_t)planes * Q, 0), pl(Q, 0);
+  std::vector<int> lists, zs;
+  for (int z = 0; z < planes; ++z) {
+    bool any = false;
+    for (int m = 0; m < n; m += 2)
+      if (points(z, m, 2) > 0) {
+        any = true;
+        for (int k = m; k < m + 2; ++k) on[(size_t)z * Q + (k & (Q - 1))] |= (unsigned char)(1u << (k / Q));
+      }
+    if (any) {
+      pl[z & (Q - 1)] |= (unsigned char)(1u << (z / Q));
+      zs.push_back(z);
+    }
+  }
   std::vector<std::pair<int, int>> band;  // (−points, band)
   for (int r = 1, R = 2; R <= n / 2; ++r, R *= 2) {
+    const int nb = n / R;
     band.clear();
-    for (int u = 0; u < n / R; ++u)
-      if (const int c = points(u * R, R)) band.push_back({-c, u});
-    // one run (at most one band whose predecessor is off) of at most 152 bands, a CTA per SM
-    int starts = 0, first = 0;
-    for (const auto& b : band)
-      if (points(b.second * R - R, R) == 0) {
-        ++starts;
-        first = b.second;
-      }
-    g->band_first[r] = starts <= 1 && band.size() <= 152 ? first : -1;
+    for (int z = 0; z < planes; ++z)
+      for (int u = 0; u < nb; ++u)
+        if (const int c = points(z, u * R, R)) band.push_back({-c, z * nb + u});
+    g->band_first[r] = -1;
+    if (g->dim == 2 && band.size() <= 152) {
+      // one run (at most one band whose predecessor is off) of at most a CTA per SM
+      int starts = 0, first = 0;
+      for (const auto& b : band)
+        if (points(0, ((b.second + nb - 1) & (nb - 1)) * R, R) == 0) {
+          ++starts;
+          first = b.second;
+        }
+      if (starts <= 1) g->band_first[r] = first;
+    }
     std::sort(band.begin(), band.end());
     g->band_off[r] = (int)lists.size();
     g->band_cnt[r] = (int)band.size();
     for (const auto& b : band) lists.push_back(b.second);
   }
-  IBDL_TRY(dalloc(&g->row_on, Q));
+  IBDL_TRY(dalloc(&g->row_on, on.size()));
   IBDL_TRY(dalloc(&g->bands, sizeof(int) * lists.size()));
-  IBDL_CUDA(cudaMemcpy(g->row_on, on.data(), Q, cudaMemcpyHostToDevice));
+  IBDL_CUDA(cudaMemcpy(g->row_on, on.data(), on.size(), cudaMemcpyHostToDevice));
   IBDL_CUDA(cudaMemcpy(g->bands, lists.data(), sizeof(int) * lists.size(), cudaMemcpyHostToDevice));
+  if (g->dim == 3) {
+    g->nplanes = (int)zs.size();
+    IBDL_TRY(dalloc(&g->plane_on, Q));
+    IBDL_TRY(dalloc(&g->planes, sizeof(int) * zs.size()));
+    IBDL_CUDA(cudaMemcpy(g->plane_on, pl.data(), Q, cudaMemcpyHostToDevice));
+    IBDL_CUDA(cudaMemcpy(g->planes, zs.data(), sizeof(int) * zs.size(), cudaMemcpyHostToDevice));
+  }
   return IBDL_OK;
 }
 
@@ -258,7 +286,8 @@ static void free_geometry(Geometry* g) {
   void* ptrs[] = {g->perm, g->base, g->cell_start, g->t64.phi, g->t64.dphi, g->t64.wscale, g->t64.nrm,
                   g->t32.phi, g->t32.dphi, g->t32.wscale, g->t32.nrm, g->spec, g->tw64, g->tw32,
                   g->lap64, g->der64, g->lap32, g->der32, g->ubuf, g->tmp_m, g->V, g->gm, g->vec,
-                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->row_on, g->bands};
+                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->row_on, g->bands,
+                  g->plane_on, g->planes};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int i = 0; i < 4; ++i)
@@ -494,7 +523,7 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     GCUDA(cudaHostAlloc((void**)&g->err_host, sizeof(int), cudaHostAllocMapped));
     *g->err_host = 0;
     GCUDA(cudaHostGetDevicePointer((void**)&g->err_dev, g->err_host, 0));
-    if (dim == 2) GTRY(touched_rows_2d(g));
+    GTRY(touched_rows(g));
     GTRY(dim == 2 ? plan_2d(g) : plan_3d(g));
   }
   g->X64 = dX;  // kept: the near-boundary interpolation decides on the caller's coordinates

@@ -98,9 +98,13 @@ struct Geometry {
   int* base;       // [dim][M] base node per axis (sorted order), already wrapped to [0, n)
   int* cell_start; // [ncell + 1], cells = n^(dim-1) rows of constant (y, z) base
   int ncell;
-  // 2-D: the rows that some stencil meets, as bits in the column lanes' order, and for each band
-  // height 2^r the list of bands holding such rows, fullest first (apply2d_kernels.cuh; NULL: all)
-  unsigned char* row_on;  // [n/8]
+  // the rows that some stencil meets, as bits in the column lanes' order, and for each band
+  // height 2^r the list of bands holding such rows, fullest first (apply2d_kernels.cuh,
+  // apply3d_kernels.cuh; NULL: all)
+  unsigned char* row_on;    // 2-D [n/8], 3-D [n][n/8]
+  unsigned char* plane_on;  // 3-D: planes with such rows [n/8], and their list
+  int* planes;
+  int nplanes;
   int* bands;             // the lists of r = 1, 2, …, one after another
   int band_off[14], band_cnt[14];
   int band_first[14];     // ≥ 0: the bands are one run from this one on (wrapped), short enough to start at once

@@ -86,3 +86,40 @@ def test_touched_rows_2d(N, pde, dipole, split, kind, rows, monkeypatch):
     field = O.grid_field(og, q)
     assert _rel(g.evaluate_field(qd).cpu().numpy(), field) < 1e-12
     g.close()
+
+
+def _surface(kind, N):
+    h = 1.0 / N
+    if kind == "one_point":
+        return np.array([[0.3], [0.6], [0.9]]), np.array([[0.6], [0.8], [0.0]]), np.array([h * h])
+    if kind == "edge":  # across y = 0 and z = 0
+        b = I.fibonacci_sphere(60, 2.0 * h, (0.4, 1.0 - 0.3 * h, 0.2 * h))
+    elif kind == "gaps":
+        return _join(I.fibonacci_sphere(50, 1.6 * h, (0.5, 0.2, 0.2)), I.fibonacci_sphere(70, 2.2 * h, (0.5, 0.75, 0.7)))
+    else:  # every plane
+        b = I.fibonacci_sphere(6 * N * N, 0.499)
+    return b.X, b.n, b.w
+
+
+@pytest.mark.parametrize("rows", [2, 8])
+@pytest.mark.parametrize("kind", ["one_point", "edge", "gaps", "tall"])
+@pytest.mark.parametrize("N,dipole", [(16, "analytic"), (32, "spectral_div"), (64, "analytic")])
+def test_touched_rows_3d(N, dipole, kind, rows, monkeypatch):
+    from paper_2210_07403_gb300 import Geometry
+
+    monkeypatch.setenv("IBDL_PLAN3_R", str(rows))
+    X, n, w = _surface(kind, N)
+    og = O.Geometry(O.Grid(3, N), X, n, w, "cos", dipole, "spectral", "scalar", 0.0, 1.0, "dirichlet")
+    g = Geometry(X, n, w, N, dipole=dipole)
+    rng = np.random.default_rng(N + rows)
+    q = rng.standard_normal(og.M)
+    qd = torch.from_numpy(q).cuda()
+    bad = torch.full_like(qd, float("nan"))
+    want, wantT = O.apply(og, q), O.transpose_apply(og, q)
+    for precision in ("fp64", "fp32", "fp32x2"):
+        assert torch.isnan(g.evaluate_field(bad)).all()
+        assert _rel(g.apply(qd, precision=precision).cpu().numpy(), want) < TOL[precision]
+        assert torch.isnan(g.apply(bad, precision=precision)).all()
+        assert _rel(g.apply_transpose(qd, precision=precision).cpu().numpy(), wantT) < TOL[precision]
+    assert _rel(g.evaluate_field(qd).cpu().numpy(), O.grid_field(og, q)) < 1e-12
+    g.close()
