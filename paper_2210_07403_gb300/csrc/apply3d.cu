@@ -40,11 +40,17 @@ ibdl_status plan_3d(Geometry* g) {
   auto clampp2 = [](int v, int lo, int hi) { v = v < lo ? lo : (v > hi ? hi : v); int r = 1; while (r * 2 <= v) r *= 2; return r; };
   for (int pi = 0; pi < 3; ++pi) {
     const bool f32 = pi == 1;
-    // FP32 CTAs take about 2048 complex elements, FP64 (and float-float, the same element size)
-    // about 1024 (measured on the 128³ sphere); R ≤ n/2 keeps the wrapped band rows
-    // [y0 − 3, y0 + R) distinct (no point counted twice)
+    // FP32 column CTAs take about 2048 complex elements, FP64 (and float-float, the same element
+    // size) about 1024 (measured on the 128³ sphere).
     const int target = f32 ? 2048 : 1024;
-    int R = clampp2(2 * (target / (n * nf)), 2, n / 2);
+    // Row bands: tall ones transform untouched rows along with the touched ones and make the
+    // fullest band (a pole of the sphere) the kernel's tail, short ones spread a point in more
+    // bands and leave threads idle. Applications of the scalar operator on spheres at R = 8 / 16 / 32
+    // (µs): 64³ FP32 25.4 / 26.4 / 26.2, FP64 103 / 90 / 92, float-float 55.5 / 56.0 / 56.2; 128³
+    // FP32 42.0 / 47.1 / 47.3, FP64 263 / 260 / 293, float-float 114 / 131 / 135; 256³ FP32 150 / 139
+    // / 146, FP64 1740 / 1712 / 1742, float-float 497 / 474 / 501. R ≤ n/2 keeps the wrapped band
+    // rows [y0 − 3, y0 + R) distinct (no point counted twice).
+    int R = clampp2((pi == 0 || n > 128 ? 16 : 8) / nf, 2, n / 2);
     int C = clampp2(target / (n * nf), 1, n / 2);
     int Cz = clampp2(target / 2 / (n * nf), 1, n / 2);
     // the column passes interleave a pass's kThreads3/(n/8) sequences across the threads of each
