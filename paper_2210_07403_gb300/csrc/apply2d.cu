@@ -768,6 +768,36 @@ void shape_for_target_2d(Geometry* g, int pi, int row_target, int col_target, in
   }
 }
 
+// Default shapes of a batch. The default shapes of a geometry favour one problem's latency (many
+// small CTAs); where a batch has so many problems of one size that those would make more than two
+// CTAs per SM, throughput decides: CTAs of about 2048 row elements and 1024 column elements (FP64: 1024
+// and 512; never smaller than the geometry's own), 256 threads in the row kernels. Scalar ellipses,
+// a third each of n, n/2 and n/4, geometry's own / these / autotuned shapes (µs): 256 to 512² FP32
+// 353 / 176 / 174, FP64 3177 / 2670 / 2650, float-float 1235 / 749 / 714; 64 to 512² FP32 109 / 69 / 69;
+// 64 to 256² FP32 59 / 46 / 43; 4 to 512² (the geometry's own are kept) FP32 36 / 41 / 37.
+void batch_shapes_2d(Batch* B) {
+  for (int pi = 0; pi < 3; ++pi) {
+    const int row_target = pi == 0 ? 1024 : 2048, col_target = pi == 0 ? 512 : 1024;
+    int units[14] = {};
+    for (int b = 0; b < B->count; ++b) {
+      const Geometry* g = B->geoms[b];
+      int cnt, first;
+      if (g->rows_per_cta[pi]) touched_bands(g, g->rows_per_cta[pi], &cnt, &first), units[log2i(g->n)] += cnt;
+    }
+    for (int b = 0; b < B->count; ++b) {
+      Geometry* g = B->geoms[b];
+      if (units[log2i(g->n)] <= 2 * 152 || g->split[pi]) continue;
+      int R = std::max(g->rows_per_cta[pi], 2 * pow2_in(row_target / g->n, 1, g->n / 4));
+      while (R > g->rows_per_cta[pi] && !row_fits(g, pi, R)) R /= 2;
+      int C = std::max(g->cols_per_cta[pi], pow2_in(col_target / (g->n * nf_row_max(g)), 1, g->n / 2));
+      while (C > g->cols_per_cta[pi] && !col_fits(g, pi, C)) C /= 2;
+      g->rows_per_cta[pi] = R;
+      g->cols_per_cta[pi] = C;
+      g->threads[pi] = 256;
+    }
+  }
+}
+
 // Default shapes: about 256 FFT lanes per CTA, but at least 2·152 CTAs per kernel where the grid
 // allows (one GB300 has 152 SMs), and at least 256 threads in the row kernels; the autotuner
 // refines them. IBDL_PLAN_R and IBDL_PLAN_C override (for tuning experiments).

@@ -106,6 +106,7 @@ ibdl_status ibdl_create_batch(const ibdl_geometry_desc* descs, int count, void* 
     B->max_log2n = std::max(B->max_log2n, __builtin_ctz(B->geoms[i]->n));
   }
   B->total = B->off[count];
+  batch_shapes_2d(B);
   ibdl_status st = batch_prepare_2d(B);
   if (st != IBDL_OK) {
     free_batch(B);

@@ -229,6 +229,7 @@ struct Batch {
 };
 
 ibdl_status batch_prepare_2d(Batch* B);
+void batch_shapes_2d(Batch* B);  // default launch shapes of the batched kernels
 // tensor map of FP32 half spectra [nf][n][n/2] in band-major order for the staged column pass:
 // dimensions (R·n floats of a band, n/R bands, nf fields), box (2·C·R, min(n/R, 256), 1)
 ibdl_status encode_col_map(void* spec, int n, int R, int C, int nf, CUtensorMap* out);
