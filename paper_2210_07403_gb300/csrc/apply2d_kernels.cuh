@@ -111,7 +111,7 @@ struct Cfg2 {
   static constexpr int V = lanes_per_thread_2d(L, F32);
   static constexpr int QT = threads_per_seq_2d(L, F32);
   static constexpr int NGRP = field_groups_2d(NF, L, F32);
-  static constexpr int NTW = F8<L, V>::NTW;
+  static constexpr int NTW = twiddles8<T, L>();
   // register budget for twiddles: 42 FP32 registers; 56 in FP64; 28 in float-float, whose
   // arithmetic needs the most temporaries
   static constexpr bool TWR =

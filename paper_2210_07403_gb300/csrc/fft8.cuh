@@ -18,6 +18,19 @@
 //
 // Twiddles come from the table tw[m] = e^{−2πi m/N}: held in registers per lane (read once,
 // before a kernel's dependency wait) or read from the table at each use.
+//
+// FP64 transforms are bound by the FP64 pipe (one warp instruction per 64 cycles and SM
+// sub-partition), so their stages are written for the least number of FP64 instructions: a twiddled
+// radix-8 stage is three levels of radix-2 butterflies a ± w·b, and with w = c(1 + i·t), t = tan of its
+// angle, p = b·(1 + i·t) and a ± c·p take six fused multiply-adds (Linzer and Feig, IEEE Trans. Signal
+// Process. 41 (1993) 93–107, and Goedecker, SIAM J. Sci. Comput. 18 (1997) 1605–1611, describe such
+// forms): 72 instructions instead of 84 for seven complex products and the 8-point DFT; the first
+// stage's √½ factors go into its last additions (52 instead of 56). The error of c·(b_x − t·b_y)
+// is that of c·b_x − s·b_y, however large t is. The table then holds (c, t) of e^{−2πi m/N}, and a
+// lane needs four entries per radix-8 stage instead of seven. FP64 applications before / after: 512²
+// Stokes star 131 / 118 µs, 2048² (finite differences, divergence dipole) 791 / 671 µs, 128³ sphere 261 /
+// 249 µs; the error against an 80-bit reference is unchanged (64² circle 4.2e−15 of S*u, 1024² 3.7e−14 /
+// 3.6e−14, 128³ 2.4e−15), which the kernel tables' rounding sets.
 #pragma once
 
 #include <type_traits>
@@ -47,19 +60,30 @@ struct F8 {
   static constexpr int V = V_;                           // lanes per thread
   static_assert(Q % V == 0, "lanes per thread must divide Q");
   static constexpr int QT = Q / V;                       // threads per sequence
-  // twiddles per lane: 7 per radix-8 stage after the first, (RT − 1) per tail butterfly
-  static constexpr int NTW = (S8 - 1) * 7 + (LT ? (RT - 1) * (8 / RT) : 0);
   static constexpr int PN = N + N / 8;                   // padded sequence length in shared memory
 };
 
+// T transforms in the fused form (table entries (cos, tan)); twiddles per lane: 7 per radix-8 stage
+// after the first and (RT − 1) per tail butterfly, in the fused form 4 (w, w², w⁴ and w·e^{−iπ/4})
+// and log2(RT) (w, w²)
+template <typename T>
+constexpr bool kFused8 = std::is_same<T, double>::value;
+template <typename T, int L>
+constexpr int twiddles8() {
+  constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT;
+  return kFused8<T> ? (S8 - 1) * 4 + (LT ? LT * (8 / RT) : 0) : (S8 - 1) * 7 + (LT ? (RT - 1) * (8 / RT) : 0);
+}
+
 __host__ __device__ constexpr int ipow8(int s) { return s == 0 ? 1 : 8 * ipow8(s - 1); }
 
-// table index of the twiddle of stage S, tail butterfly m (0 for radix-8 stages), input r, lane j
+// table index of the twiddle of stage S, tail butterfly m (0 for radix-8 stages), input r, lane j;
+// r = 9 (fused form): that of r = 1 times e^{−iπ/4}
 template <int L, int S>
 __device__ __forceinline__ int tw_index(int j, int m, int r) {
   constexpr int S8 = L / 3, N = 1 << L, Q = N / 8;
   if constexpr (S < S8) {
     constexpr int p = ipow8(S);
+    if (r == 9) return (j & (p - 1)) * (N / (8 * p)) + N / 8;
     return r * (j & (p - 1)) * (N / (8 * p));
   } else {
     return r * (j + m * Q);
@@ -70,23 +94,29 @@ __device__ __forceinline__ int tw_index(int j, int m, int r) {
 template <typename T, int L>
 struct TwRegs {
   static constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT;
-  static constexpr int NTW = (S8 - 1) * 7 + (LT ? (RT - 1) * (8 / RT) : 0);
+  static constexpr int NTW = twiddles8<T, L>();
+  static constexpr int N8 = kFused8<T> ? 4 : 7;       // per radix-8 stage
+  static constexpr int NT = kFused8<T> ? LT : RT - 1;  // per tail butterfly
   cplx<T> w[NTW > 0 ? NTW : 1];
   template <int S>
   __host__ __device__ static constexpr int off(int m, int r) {
-    return S < S8 ? (S - 1) * 7 + (r - 1) : (S8 - 1) * 7 + m * (RT - 1) + (r - 1);
+    // fused form: slots 0 … 3 for r = 1, 2, 4, 9
+    const int k = !kFused8<T> ? r - 1 : (r == 9 ? 3 : (r == 4 ? 2 : r - 1));
+    return S < S8 ? (S - 1) * N8 + k : (S8 - 1) * N8 + m * NT + k;
   }
   __device__ __forceinline__ void load(const cplx<T>* __restrict__ tab, int j) {
     static_for<1, S8>([&](auto st) {
       constexpr int S = decltype(st)::value;
 #pragma unroll
-      for (int r = 1; r < 8; ++r) w[off<S>(0, r)] = tab[tw_index<L, S>(j, 0, r)];
+      for (int r = 1; r < 10; ++r)
+        if (kFused8<T> ? (r == 1 || r == 2 || r == 4 || r == 9) : r < 8)
+          w[off<S>(0, r)] = tab[tw_index<L, S>(j, 0, r)];
     });
     if constexpr (LT > 0) {
 #pragma unroll
       for (int m = 0; m < 8 / RT; ++m)
 #pragma unroll
-        for (int r = 1; r < RT; ++r) w[off<S8>(m, r)] = tab[tw_index<L, S8>(j, m, r)];
+        for (int r = 1; r <= NT; ++r) w[off<S8>(m, r)] = tab[tw_index<L, S8>(j, m, r)];
     }
   }
   template <int S>
@@ -112,11 +142,86 @@ __device__ __forceinline__ cplx<T> cmul_tw(cplx<T> a, cplx<T> w) {
   return INV ? mk(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y) : mk(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
 }
 
+// (a, b) ← (a + w·b, a − w·b) with w = c(1 + i·t) given as (c, t) (INV: conj w; ROT: times −i, INV i)
+template <typename T, bool INV, bool ROT>
+__device__ __forceinline__ void bfly_tan(cplx<T>& a, cplx<T>& b, cplx<T> w) {
+  const T t = INV ? -w.y : w.y;
+  cplx<T> p = mk(fma(-t, b.y, b.x), fma(t, b.x, b.y));
+  if (ROT) p = rot90<T, INV>(p);
+  b = mk(fma(-w.x, p.x, a.x), fma(-w.x, p.y, a.y));
+  a = mk(fma(w.x, p.x, a.x), fma(w.x, p.y, a.y));
+}
+
+// 8-point DFT of w^r·x_r, r < 8, from w, w², w⁴ and w·e^{−iπ/4} as (cos, tan): 72 fused multiply-adds
+template <typename T, bool INV>
+__device__ __forceinline__ void dft8_tan(cplx<T> (&x)[8], cplx<T> w1, cplx<T> w2, cplx<T> w4, cplx<T> w1e) {
+  // t mod 2 from the pairs (r, r + 4): x[r], x[r + 4]
+#pragma unroll
+  for (int r = 0; r < 4; ++r) bfly_tan<T, INV, false>(x[r], x[r + 4], w4);
+  // t mod 4 from the pairs (r, r + 2): t = 0, 2 in (x0, x2), (x1, x3); 1, 3 in (x4, x6), (x5, x7)
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    bfly_tan<T, INV, false>(x[r], x[r + 2], w2);
+    bfly_tan<T, INV, true>(x[r + 4], x[r + 6], w2);
+  }
+  bfly_tan<T, INV, false>(x[0], x[1], w1);  // outputs 0, 4
+  bfly_tan<T, INV, true>(x[2], x[3], w1);   // 2, 6
+  bfly_tan<T, INV, false>(x[4], x[5], w1e);  // 1, 5
+  bfly_tan<T, INV, true>(x[6], x[7], w1e);   // 3, 7
+  const cplx<T> y[8] = {x[0], x[4], x[2], x[6], x[1], x[5], x[3], x[7]};
+#pragma unroll
+  for (int t = 0; t < 8; ++t) x[t] = y[t];
+}
+
+// 8-point DFT as dft8, the odd half's √½ factors inside its last additions: 52 FP64 instructions
+template <typename T, bool INV>
+__device__ __forceinline__ void dft8_fma(cplx<T>* u) {
+  const T c = T(0.70710678118654752440);
+  cplx<T> a0 = cadd(u[0], u[4]), a1 = cadd(u[1], u[5]), a2 = cadd(u[2], u[6]), a3 = cadd(u[3], u[7]);
+  const cplx<T> b0 = csub(u[0], u[4]), b1 = csub(u[1], u[5]), b2 = rot90<T, INV>(csub(u[2], u[6])), b3 = csub(u[3], u[7]);
+  // √2·ω₈·b1 and √2·ω₈³·b3
+  const cplx<T> p1 = INV ? mk(b1.x - b1.y, b1.x + b1.y) : mk(b1.x + b1.y, b1.y - b1.x);
+  const cplx<T> p3 = INV ? mk(-(b3.x + b3.y), b3.x - b3.y) : mk(b3.y - b3.x, -(b3.x + b3.y));
+  dft4<T, INV>(a0, a1, a2, a3);
+  const cplx<T> t0 = cadd(b0, b2), t1 = csub(b0, b2), t2 = cadd(p1, p3), t3 = rot90<T, INV>(csub(p1, p3));
+  u[0] = a0;
+  u[1] = mk(fma(c, t2.x, t0.x), fma(c, t2.y, t0.y));
+  u[2] = a1;
+  u[3] = mk(fma(c, t3.x, t1.x), fma(c, t3.y, t1.y));
+  u[4] = a2;
+  u[5] = mk(fma(-c, t2.x, t0.x), fma(-c, t2.y, t0.y));
+  u[6] = a3;
+  u[7] = mk(fma(-c, t3.x, t1.x), fma(-c, t3.y, t1.y));
+}
+
 // stage S on one lane's registers
 template <typename T, bool INV, int L, int S, class TW>
 __device__ __forceinline__ void f8_stage(cplx<T> (&x)[8], const TW& tw) {
   constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT;
-  if constexpr (S < S8) {
+  if constexpr (kFused8<T>) {
+    if constexpr (S == 0) {
+      dft8_fma<T, INV>(x);
+    } else if constexpr (S < S8) {
+      dft8_tan<T, INV>(x, tw.template get<S>(0, 1), tw.template get<S>(0, 2), tw.template get<S>(0, 4),
+                       tw.template get<S>(0, 9));
+    } else if constexpr (LT == 1) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) bfly_tan<T, INV, false>(x[m], x[m + 4], tw.template get<S>(m, 1));
+    } else {
+      // radix 4: inputs and outputs of butterfly m at x[m + 2r], r = 0 … 3
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const cplx<T> w1 = tw.template get<S>(m, 1), w2 = tw.template get<S>(m, 2);
+        bfly_tan<T, INV, false>(x[m], x[m + 4], w2);
+        bfly_tan<T, INV, false>(x[m + 2], x[m + 6], w2);
+        bfly_tan<T, INV, false>(x[m], x[m + 2], w1);     // outputs 0, 2
+        bfly_tan<T, INV, true>(x[m + 4], x[m + 6], w1);  // outputs 1, 3
+        const cplx<T> y1 = x[m + 4], y2 = x[m + 2];
+        x[m + 2] = y1;
+        x[m + 4] = y2;
+      }
+    }
+  } else if constexpr (S < S8) {
     if constexpr (S > 0) {
 #pragma unroll
       for (int r = 1; r < 8; ++r) x[r] = cmul_tw<T, INV>(x[r], tw.template get<S>(0, r));

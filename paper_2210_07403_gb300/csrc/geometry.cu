@@ -112,23 +112,27 @@ __global__ void k_tables(int dim, int n, int M, int delta, const double* __restr
   t32.wscale[s] = (float)(w[i] / hd);
 }
 
-// tw[j] = e^{−2πi j/n}
+// tw[j] = e^{−2πi j/n} = (c, s) in FP32; (c, t) with t = s/c for the FP64 transforms' fused form. At a
+// quarter turn, where c = 0, c = 2^−60 stands for it: c·(b_x − t·b_y) with t = −2^60 is then −s·b_y to
+// rounding (the term 2^−60·b_x lies below it).
 __global__ void k_twiddles(int n, double2* tw64, float2* tw32) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   double s, c;
   sincospi(-2.0 * (double)j / (double)n, &s, &c);
-  tw64[j] = make_double2(c, s);
+  const double cc = c == 0.0 ? 0x1p-60 : c;
+  tw64[j] = make_double2(cc, s / cc);
   tw32[j] = make_float2((float)c, (float)s);
 }
 
 // float-float copies of the FP64 twiddles and symbols (hi = fl32(x), lo = fl32(x − hi))
-__global__ void k_ff_tables(int n, const double2* tw64, const double* lap64, const double* der64, ff* twff, ff* lapff,
-                            ff* derff) {
+__global__ void k_ff_tables(int n, const double* lap64, const double* der64, ff* twff, ff* lapff, ff* derff) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  twff[2 * j] = ff(tw64[j].x);
-  twff[2 * j + 1] = ff(tw64[j].y);
+  double s, c;
+  sincospi(-2.0 * (double)j / (double)n, &s, &c);
+  twff[2 * j] = ff(c);
+  twff[2 * j + 1] = ff(s);
   lapff[j] = ff(lap64[j]);
   derff[j] = ff(der64[j]);
 }
@@ -173,7 +177,7 @@ ibdl_status fill_geometry_tables(Geometry* g, const double* dX, const double* dN
   k_twiddles<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->tw64, g->tw32);
   k_symbols<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->box, g->symbol, g->lap64, g->der64, g->lap32, g->der32);
   if (g->twff)
-    k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->tw64, g->lap64, g->der64, static_cast<ff*>(g->twff),
+    k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->lap64, g->der64, static_cast<ff*>(g->twff),
                                                   static_cast<ff*>(g->lapff), static_cast<ff*>(g->derff));
   IBDL_CUDA(cudaGetLastError());
   return IBDL_OK;
@@ -514,7 +518,7 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     k_twiddles<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->tw64, g->tw32);
     k_symbols<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->box, g->symbol, g->lap64, g->der64, g->lap32, g->der32);
     if (g->twff)
-      k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->tw64, g->lap64, g->der64, static_cast<ff*>(g->twff),
+      k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->lap64, g->der64, static_cast<ff*>(g->twff),
                                                     static_cast<ff*>(g->lapff), static_cast<ff*>(g->derff));
     GCUDA(cudaGetLastError());
     GCUDA(cudaStreamSynchronize(s));

@@ -118,8 +118,8 @@ struct Geometry {
   // workspace: half spectra, packed format (see apply kernels): [nf][rows][n/2] complex
   void* spec;      // sized for nf_in fields in FP64
   size_t spec_bytes;
-  double2* tw64;   // [n] e^{-2πi j/n}
-  float2* tw32;
+  double2* tw64;   // [n] (cos, tan) of e^{-2πi j/n} (fft8.cuh)
+  float2* tw32;    // [n] e^{-2πi j/n}
   // per-axis Fourier symbols indexed by FFT index j (wavenumber 2π m/box, m = j or j − n):
   // lap = symbol of −∂² along one axis, der = k̃ with ∂ ↦ i k̃ (0 at Nyquist)
   double *lap64, *der64;
