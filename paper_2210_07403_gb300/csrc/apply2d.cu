@@ -120,7 +120,7 @@ static ColParams<T> col_params(Geometry* g, const int* stop) {
   cp.R = g->rows_per_cta[pi];
   cp.lam = T(g->lambda);
   cp.mu = T(g->mu);
-  cp.scale = T(1.0 / ((double)g->n * (double)g->n));
+  cp.scale = T(0.5 / ((double)g->n * (double)g->n));  // the transforms' 1/n², and ½: the spread's spectra are doubled
   cp.lap1 = static_cast<const T*>(Slot2<T>::lap(g));
   cp.der1 = static_cast<const T*>(Slot2<T>::der(g));
   cp.spec = reinterpret_cast<cplx<T>*>(g->spec);

@@ -520,7 +520,8 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // unpack Z = FFT(a + i b) of the row pair (2j, 2j + 1) into A = FFT(a) (even row) and
   // B = FFT(b) (odd row), k = 0..n/2, packed format: thread t takes wavenumber k = t mod n/2 of
   // one (field, row pair), reads Z_k and Z_{n−k} once and writes A_k and B_k, adjacent in the
-  // band-major block (offset k·R + 2j), with one store
+  // band-major block (offset k·R + 2j), with one store. Both are left doubled (the ½ is in the
+  // symbol's scale: half the arithmetic of this step)
   const cplx<T>* res = buf;
   constexpr int nh = n >> 1, lnh = L - 1;
   for (int t = threadIdx.x; t < NB * half * nh; t += blockDim.x) {
@@ -531,12 +532,12 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
     cplx<T> a, b;
     if (k == 0) {
       const cplx<T> z0 = res[zb], zh = res[zb + ppos(nh)];
-      a = mk(z0.x, zh.x);
-      b = mk(z0.y, zh.y);
+      a = mk(z0.x + z0.x, zh.x + zh.x);
+      b = mk(z0.y + z0.y, zh.y + zh.y);
     } else {
       const cplx<T> zk = res[zb + ppos(k)], zc = res[zb + ppos(n - k)];
-      a = mk(T(0.5) * (zk.x + zc.x), T(0.5) * (zk.y - zc.y));
-      b = mk(T(0.5) * (zk.y + zc.y), T(0.5) * (zc.x - zk.x));
+      a = mk(zk.x + zc.x, zk.y - zc.y);
+      b = mk(zk.y + zc.y, zc.x - zk.x);
     }
     store_pair(p.spec + ((fo * n + r0) * nh + k * R + 2 * jj), a, b);
   }
@@ -558,12 +559,6 @@ __global__ void __launch_bounds__(kMaxThreads2d) k_spread_rowfft1(RowParams<T> p
 // Fourier symbols: NIN transformed fields in → NOUT out; lap = |k̃|² (sum of the per-axis
 // Laplacian symbols), dkx, dky the per-axis derivative symbols
 // ------------------------------------------------------------------------------------------
-// a/b: the hardware reciprocal estimate in FP32 (within 2 ulp, well inside the FP32 application's
-// rounding), IEEE division in FP64, a corrected quotient in float-float
-__device__ __forceinline__ float sym_div(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double sym_div(double a, double b) { return a / b; }
-__device__ __forceinline__ ff sym_div(ff a, ff b) { return a / b; }
-
 template <typename T, int OP>
 __device__ __forceinline__ void apply_symbol(const ColParams<T>& p, T lap, T dkx, T dky, const cplx<T>* in,
                                              cplx<T>* out) {

@@ -123,7 +123,7 @@ static ibdl_status run_op3(Geometry* g, const double* in, double* out, cudaStrea
   cp.C = C;
   cp.lc = __builtin_ctz(C);
   cp.lam = laplace ? 0.0 : g->lambda;
-  cp.scale = 1.0 / ((double)n * n * n);
+  cp.scale = 0.5 / ((double)n * n * n);  // the transforms' 1/n³, and ½: the spread's spectra are doubled
   cp.lap1 = pi == 1 ? (const void*)g->lap32 : (pi == 2 ? (const void*)g->lapff : (const void*)g->lap64);
   cp.der1 = pi == 1 ? (const void*)g->der32 : (pi == 2 ? (const void*)g->derff : (const void*)g->der64);
   cp.spec = g->spec;

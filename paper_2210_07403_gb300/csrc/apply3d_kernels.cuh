@@ -385,12 +385,12 @@ __global__ void __launch_bounds__(kThreads3) k3_spread_rowfft(Row3Params p) {
     cplx<T> A, B;
     if (k == 0) {
       const cplx<T> z0 = res[pidx(zb)], zh = res[pidx(zb + nh)];
-      A = mk(z0.x, zh.x);
-      B = mk(z0.y, zh.y);
-    } else {
+      A = mk(z0.x + z0.x, zh.x + zh.x);
+      B = mk(z0.y + z0.y, zh.y + zh.y);
+    } else {  // both left doubled: the ½ is in the symbol's scale
       const cplx<T> zk = res[pidx(zb + k)], zc = res[pidx(zb + n - k)];
-      A = mk(T(0.5) * (zk.x + zc.x), T(0.5) * (zk.y - zc.y));
-      B = mk(T(0.5) * (zk.y + zc.y), T(0.5) * (zc.x - zk.x));
+      A = mk(zk.x + zc.x, zk.y - zc.y);
+      B = mk(zk.y + zc.y, zc.x - zk.x);
     }
     const size_t row = (size_t)z * n + y0 + 2 * j;
     spec[((size_t)f * n * n + row) * nh + k] = A;
@@ -478,7 +478,7 @@ __device__ __forceinline__ void symbol3(const T* lap1, const T* der1, T lam, T s
                                         const cplx<T>* in, cplx<T>* out) {
   const T lap = lap1[kx] + lap1[ky] + lap1[kz];
   const T den = lap + lam;
-  const T sig = den != T(0) ? scale / den : T(0);
+  const T sig = den != T(0) ? sym_div(scale, den) : T(0);
   if (OP == OP3_SCALAR_AN || OP == OP3_ADJ_AN) {
     out[0] = cscale(in[0], sig);
   } else if (OP == OP3_SCALAR_SD) {
