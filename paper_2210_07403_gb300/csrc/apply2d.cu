@@ -95,6 +95,7 @@ static RowParams<T> row_params(Geometry* g, const double* in, double* out, const
   rp.vstride = 0;
   rp.io_off = 0;
   rp.trans = 0;
+  rp.late = 0;
   rp.fsel = 0;
   int cnt;
   rp.bands_in = rp.bands_out = touched_bands(g, rp.R, &cnt, &rp.band0_in);
@@ -126,6 +127,7 @@ static ColParams<T> col_params(Geometry* g, const int* stop) {
   cp.spec = reinterpret_cast<cplx<T>*>(g->spec);
   cp.tw = static_cast<const cplx<T>*>(Slot2<T>::tw(g));
   cp.stop = stop;
+  cp.late = 0;
   cp.err = g->err_dev;
   cp.on_in = cp.on_out = g->row_on;
   return cp;
@@ -135,11 +137,13 @@ static ColParams<T> col_params(Geometry* g, const int* stop) {
 // for band height R, column group C and the row kernels' least thread count `floor`, or an error
 // if they do not fit.
 static int row_threads(int nf, int R, int L, bool f32, int floor) {
-  const int need = field_groups_2d(nf, L, f32) * (R / 2) * threads_per_seq_2d(L, f32);
+  const int ng = field_groups_2d(nf, L, f32);
+  const int need = ng * group_threads_2d(ng, (R / 2) * threads_per_seq_2d(L, f32));
   return need > floor ? need : (floor < kMaxThreads2d ? floor : kMaxThreads2d);
 }
 static int col_threads(int nf, int C, int L, bool f32) {
-  return field_groups_2d(nf, L, f32) * C * threads_per_seq_2d(L, f32);
+  const int ng = field_groups_2d(nf, L, f32);
+  return ng * group_threads_2d(ng, C * threads_per_seq_2d(L, f32));
 }
 
 template <typename T, int OP>
@@ -181,6 +185,18 @@ static ibdl_status launch_for_size(int lg, Geometry* g, const RowParams<T>& rp, 
     if (lg == L) return launch_apply_2d<T, OP, L>(g, rp, cp, lc, s);
     return launch_for_size<T, OP, L + 1>(lg, g, rp, cp, lc, s);
   }
+}
+
+// When the row kernels of a single problem let the next kernel launch (programmatic launch): before
+// their transforms, or (late) after them. Early hides the launch, which is what counts in FP32. But
+// the next kernel's CTAs then settle beside the running ones, and where about as many CTAs as SMs are
+// running they leave some SMs with two CTAs and others with none: FP64 kernels of 64 (several
+// fields) or 128 to 200 bands trigger late (scalar 512² 92 → 47 µs, Stokes 256² 54.1 → 51.1). Float-float
+// kernels always do: their code is large, and the next kernel's prologue evicts it from the
+// instruction cache (scalar 64² 31 → 24 µs, 512² 43 → 31; its column pass as well with several
+// fields, Stokes 64² 33.6 → 31.8).
+static int late_rows_2d(int pi, int nin, int units) {
+  return pi == 2 || (pi == 0 && units >= (nin > 1 ? 64 : 128) && units <= 200);
 }
 
 // run_op mode bits: RUN_LAPLACE solves the plain Laplace problem (λ → 0) without the completed
@@ -228,6 +244,8 @@ static ibdl_status run_op(Geometry* g, const double* in, double* out, cudaStream
     rp.on_out = cp.on_out = nullptr;
     lc.units_out = g->n / rp.R;
   }
+  rp.late = late_rows_2d(pi, Traits<OP>::NIN, lc.units_in);
+  cp.late = pi == 2 && Traits<OP>::NIN > 1;
   return launch_for_size<T, OP, kMinL2d>(log2i(g->n), g, rp, cp, lc, s);
 }
 
@@ -619,13 +637,17 @@ static bool row_fits(const Geometry* g, int pi, int R) {
   const int L = log2i(g->n), nf = nf_held(g, pi);
   const size_t bytes = pi == 1 ? smem_rows_2d<float>(nf, R, L) : smem_rows_2d<double>(nf, R, L);
   // R ≤ n/8 (the column pass's lanes then address their rows with one stride per band)
-  return R >= 2 && R <= std::max(2, g->n / 8) && bytes <= kSmemLimit2d &&
-         row_threads(nf, R, L, pi == 1, 0) <= kMaxThreads2d;
+  // (fewer fields may need more threads: as many groups as fields that fit)
+  int threads = 0;
+  for (int f = 1; f <= nf; ++f) threads = std::max(threads, row_threads(f, R, L, pi == 1, 0));
+  return R >= 2 && R <= std::max(2, g->n / 8) && bytes <= kSmemLimit2d && threads <= kMaxThreads2d;
 }
 static bool col_fits(const Geometry* g, int pi, int C) {
   const int L = log2i(g->n), nf = nf_held(g, pi);
   const size_t bytes = pi == 1 ? smem_cols_2d<float>(nf, C, L) : smem_cols_2d<double>(nf, C, L);
-  return C >= 1 && C <= g->n / 2 && bytes <= kSmemLimit2d && col_threads(nf, C, L, pi == 1) <= kMaxThreads2d;
+  int threads = 0;
+  for (int f = 1; f <= nf; ++f) threads = std::max(threads, col_threads(f, C, L, pi == 1));
+  return C >= 1 && C <= g->n / 2 && bytes <= kSmemLimit2d && threads <= kMaxThreads2d;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -786,6 +808,7 @@ void batch_shapes_2d(Batch* B) {
     }
     for (int b = 0; b < B->count; ++b) {
       Geometry* g = B->geoms[b];
+      g->threads[pi] = 256;
       if (units[log2i(g->n)] <= 2 * 152 || g->split[pi]) continue;
       int R = std::max(g->rows_per_cta[pi], 2 * pow2_in(row_target / g->n, 1, g->n / 4));
       while (R > g->rows_per_cta[pi] && !row_fits(g, pi, R)) R /= 2;
@@ -793,33 +816,38 @@ void batch_shapes_2d(Batch* B) {
       while (C > g->cols_per_cta[pi] && !col_fits(g, pi, C)) C /= 2;
       g->rows_per_cta[pi] = R;
       g->cols_per_cta[pi] = C;
-      g->threads[pi] = 256;
     }
   }
 }
 
-// Default shapes: about 256 FFT lanes per CTA, but at least 2·152 CTAs per kernel where the grid
-// allows (one GB300 has 152 SMs), and at least 256 threads in the row kernels; the autotuner
-// refines them. IBDL_PLAN_R and IBDL_PLAN_C override (for tuning experiments).
+// Default shapes, from sweeps of every shape over n = 16 … 8192 and one to three fields, applications
+// back to back; the autotuner refines them. FP64 and float-float: two-row bands and single columns (the
+// FP64 pipe wants as many CTAs as possible: scalar 64² with C = 2 / 1 34.7 / 32.1 µs, 1024² 130 / 120,
+// Stokes 512² 117 / 105), 512 threads in the row kernels where there are about as many bands as SMs,
+// so that no SM takes two (Stokes 512² 92 → 85 µs), else 256. FP32: two columns (8192² with C = 1 / 2
+// 705 / 625 µs, Stokes 4096² 509 / 431), bands of four rows from 512² to 4096² (4096² R = 2 / 4 170 / 149
+// µs), and 512 threads in the row kernels' loops where the transforms need at most 256 (512² 11.1 →
+// 10.0 µs, 2048² 47 → 39; with 384 lanes they only add barriers' width, Stokes 1024² 39.9 → 43.5).
+// Shapes that do not fit give way to smaller ones. IBDL_PLAN_R and IBDL_PLAN_C override (for tuning
+// experiments).
 ibdl_status plan_2d(Geometry* g) {
   const int n = g->n, L = log2i(n);
-  const int min_ctas = 2 * 152;
   int tuned_stage = 0;
   const char* se = getenv("IBDL_SPLIT_FIELDS");
   const bool force_split = se && atoi(se) != 0 && nf_row_max(g) > 1;
   for (int pi = 0; pi < 3; ++pi) {
-    const int qt = threads_per_seq_2d(L, pi == 1);
+    const bool f32 = pi == 1;
     int R = 0, C = 0;
     // all fields of a band or column group at once where they fit shared memory, else one field
     // per launch (multi-field operators only)
     for (int split = force_split ? 1 : 0; split < 2; ++split) {
       if (split && nf_row_max(g) == 1) break;
       g->split[pi] = split;
-      R = 2 * pow2_in(256 / qt, 1, n / 4 > 1 ? n / 4 : 1);
-      while (R > 2 && (n / R < std::min(min_ctas, n / 2) || !row_fits(g, pi, R))) R /= 2;
+      R = f32 && n >= 512 && n <= 4096 ? 4 : 2;
+      while (R > 2 && !row_fits(g, pi, R)) R /= 2;
       if (!row_fits(g, pi, R)) R = 0;
-      C = pow2_in(256 / qt, 1, n / 2);
-      while (C > 1 && ((n / 2) / C < std::min(min_ctas, n / 4) || !col_fits(g, pi, C))) C /= 2;
+      C = f32 ? 2 : 1;
+      while (C > 1 && !col_fits(g, pi, C)) C /= 2;
       if (!col_fits(g, pi, C)) C = 0;
       if (R && C) break;
     }
@@ -834,7 +862,12 @@ ibdl_status plan_2d(Geometry* g) {
     if (R == 0 || C == 0) R = C = 0;
     g->rows_per_cta[pi] = R;
     g->cols_per_cta[pi] = C;
-    g->threads[pi] = 256;  // the row kernels' loops (clearing, spreading, unpacking) get 256 threads
+    // the row kernels' loops (clearing, spreading, unpacking) get at least 256 threads
+    int cnt = 0, first;
+    if (R) touched_bands(g, R, &cnt, &first);
+    const bool more = f32 ? n <= 4096 && R && row_threads(nf_held(g, pi), R, L, true, 0) <= 256
+                          : cnt >= (g->nf_in > 1 ? 64 : 128) && cnt <= 200;
+    g->threads[pi] = more ? 512 : 256;
     TuneVal tv;
     if (R && tuned_lookup(tune_key(g, pi), &tv) && row_fits(g, pi, tv.R) && col_fits(g, pi, tv.C)) {
       g->rows_per_cta[pi] = tv.R;

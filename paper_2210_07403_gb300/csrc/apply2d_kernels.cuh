@@ -135,11 +135,19 @@ __host__ __device__ constexpr int col_stride_2d(int L, int C, int esize) {
   const int t = (w / C > 1 ? w / C : 1) % w;
   return C < 2 ? pn : pn + (((t - pn) % w) + w) % w;
 }
-template <int QT>
-__device__ __forceinline__ void col_lane_2d(int C, int& g, int& c, int& j0) {
-  const int per = C * QT;
-  g = (int)threadIdx.x / per;
-  const int t = (int)threadIdx.x - g * per;
+// With several thread groups (one per field) a group starts on a warp: groups of fewer than 32 lanes
+// would share a warp and run one after another.
+__host__ __device__ constexpr int group_threads_2d(int ngrp, int per) { return ngrp > 1 && per < 32 ? 32 : per; }
+template <int QT, int NGRP>
+__device__ __forceinline__ void col_lane_2d(int C, int& g, int& c, int& j0, bool& active) {
+  const int per = C * QT, st = group_threads_2d(NGRP, per);
+  g = (int)threadIdx.x / st;
+  int t = (int)threadIdx.x - g * st;
+  active = g < NGRP;
+  if (NGRP > 1 && t >= per) {  // the rest of a short group's warp
+    active = false;
+    t = 0;
+  }
   c = t & (C - 1);
   j0 = t >> (__ffs(C) - 1);
 }
@@ -151,15 +159,16 @@ __host__ __device__ constexpr bool row_interleave_2d(int L, bool f32) { return l
 __host__ __device__ constexpr int row_stride_2d(int L, int half, int esize) {
   return row_interleave_2d(L, esize == 8) ? col_stride_2d(L, half, esize) : (1 << L) + (1 << L) / 8;
 }
-template <int QT, bool IL>
-__device__ __forceinline__ void row_lane_2d(int half, int& g, int& rp, int& j0) {
+template <int QT, int NGRP, bool IL>
+__device__ __forceinline__ void row_lane_2d(int half, int& g, int& rp, int& j0, bool& active) {
   if constexpr (IL) {
-    col_lane_2d<QT>(half, g, rp, j0);
+    col_lane_2d<QT, NGRP>(half, g, rp, j0, active);
   } else {
     const int q = (int)threadIdx.x / QT;
     j0 = (int)threadIdx.x - q * QT;
     g = q / half;
     rp = q - g * half;
+    active = g < NGRP;
   }
 }
 
@@ -195,6 +204,7 @@ struct RowParams {
   double eta;             // η
   double hd;              // h^d
   PT eta_src;             // weight of the ηSQ source: η (scalar) or η/μ (Stokes, projected part)
+  int late;               // single problems: let the next kernel launch after the transforms, not before
   int fsel;               // one-field launches: the field this launch spreads or interpolates
   // the bands some stencil meets (NULL: every band), for the spread and for the gather, and the
   // rows whose spectra the gather needs (see touched rows below; NULL: every row)
@@ -228,6 +238,7 @@ struct ColParams {
   const cplx<T>* tw;
   const int* stop;
   int* err;  // the staged column pass sets it to 1 when a bounded wait runs out
+  int late;  // as in RowParams
   const unsigned char* on_in;   // rows the spread wrote (NULL: every row; the others are zero)
   const unsigned char* on_out;  // rows the last kernel reads (NULL: every row)
 };
@@ -356,8 +367,8 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // FFT lanes: thread (group g, row pair rp, lane j0); threads past NGRP·half·QT only help with
   // the loops (clearing, spreading, unpacking)
   int g, rp, j0;
-  row_lane_2d<QT, row_interleave_2d(L, sizeof(T) == 4)>(half, g, rp, j0);
-  const bool active = g < NGRP;
+  bool active;
+  row_lane_2d<QT, NGRP, row_interleave_2d(L, sizeof(T) == 4)>(half, g, rp, j0, active);
   // prologue independent of the previous kernel, then wait for it (programmatic launch)
   {
     // clear the accumulation buffer (NIN·half padded sequences, a multiple of 16 bytes) with
@@ -380,7 +391,7 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // Let the next kernel launch and run its prologue. Triggered only after this kernel's own
   // wait, so every kernel before the previous one has completed by then: a prologue overlaps
   // its direct predecessor only (its wait still covers this grid's completion and writes).
-  cudaTriggerProgrammaticLaunchCompletion();
+  if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();
   // In a GMRES cycle the step just before this kernel writes the stop flag and the Krylov index:
   // both loads go out together, then the branch
   const int stopped = p.stop ? *p.stop : 0;
@@ -522,6 +533,7 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // one (field, row pair), reads Z_k and Z_{n−k} once and writes A_k and B_k, adjacent in the
   // band-major block (offset k·R + 2j), with one store. Both are left doubled (the ½ is in the
   // symbol's scale: half the arithmetic of this step)
+  if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
   const cplx<T>* res = buf;
   constexpr int nh = n >> 1, lnh = L - 1;
   for (int t = threadIdx.x; t < NB * half * nh; t += blockDim.x) {
@@ -669,8 +681,8 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
   const int k0 = unit * C;
   // thread (group g, column c, lane j0), the group's C columns interleaved across threads
   int g, c, j0;
-  col_lane_2d<QT>(C, g, c, j0);
-  const bool active = g < NGRP;
+  bool active;
+  col_lane_2d<QT, NGRP>(C, g, c, j0, active);
   const int kx = k0 + c;
   // sequence (field f, column c) at buf + (f·C + c)·PN
   const int PN = col_stride_2d(L, C, (int)sizeof(cplx<T>));
@@ -714,7 +726,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
     ono[v] = rows_on(p.on_out, j0 + v * QT);
   }
   cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
+  if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
 
   if constexpr (NIN == 1 && NOUT == 1) {
     // one field in and out: the symbol is applied to the registers between the transforms
@@ -759,6 +771,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
     }
     // (the inverse transform's first exchange barrier orders the partner reads before its writes)
     f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, active);
+    if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
@@ -858,6 +871,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
           for (int s = 0; s < 8; ++s) x[0][v][s] = sb[ppos_strided<Q>(j0 + v * QT, s)];
       }
       f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, act);
+      if (PF && p.late && k + 1 == (NOUT + NGRP - 1) / NGRP) cudaTriggerProgrammaticLaunchCompletion();
       if (act) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
@@ -999,8 +1013,8 @@ __global__ void __launch_bounds__(kMaxThreads2d) k_colfft(ColParams<T> p, int fi
   constexpr int V = CF::V, QT = CF::QT;
   const int C = p.C, R = p.R, kx0 = blockIdx.x * C;
   int g, c, j0;
-  col_lane_2d<QT>(C, g, c, j0);
-  const bool active = g < 1;
+  bool active;
+  col_lane_2d<QT, 1>(C, g, c, j0, active);
   const int kx = kx0 + c;
   cplx<T>* sb = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)c * col_stride_2d(L, C, (int)sizeof(cplx<T>));
   typename CF::TW tw[V];
@@ -1163,7 +1177,8 @@ __global__ void __launch_bounds__(kMaxThreads2d)
     unit_of(0, q0, m0, c0);
     // (every unit of a launch has the same column group C, so a lane keeps its twiddles)
     int gg, cc, jj;
-    col_lane_2d<QT>(q0->C, gg, cc, jj);
+    bool aa;
+    col_lane_2d<QT, NGRP>(q0->C, gg, cc, jj, aa);
     const cplx<T>* twp = q0->tw;
 #pragma unroll
     for (int v = 0; v < V; ++v) tw[v].load(twp, jj + v * QT);
@@ -1192,8 +1207,8 @@ __global__ void __launch_bounds__(kMaxThreads2d)
     const ColParams<T> qv = *q;
     const int C = qv.C, R = qv.R, k0 = cu * C;
     int g, c, j0;
-    col_lane_2d<QT>(C, g, c, j0);
-    const bool active = g < NGRP;
+    bool active;
+    col_lane_2d<QT, NGRP>(C, g, c, j0, active);
     const int kx = k0 + c;
     const int PN = col_stride_2d(L, C, (int)sizeof(cplx<T>));
     const bool packed = k0 == 0;
@@ -1443,8 +1458,8 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   const int r0 = unit * R;
   // FFT lanes: thread (group g, row pair rp, lane j0); threads past NGRP·half·QT only gather
   int g, rp, j0;
-  row_lane_2d<QT, row_interleave_2d(L, sizeof(T) == 4)>(half, g, rp, j0);
-  const bool active = g < NGRP;
+  bool active;
+  row_lane_2d<QT, NGRP, row_interleave_2d(L, sizeof(T) == 4)>(half, g, rp, j0, active);
   typename CF::TW tw[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) tw[v].load(p.tw, j0 + v * QT);
@@ -1466,7 +1481,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   double* pout;
   resolve_io(p, pin, pout);
   cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
+  if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
 
   // inverse FFT of every (field, row pair) sequence, its first stage fed from the half spectra
 #pragma unroll
@@ -1491,6 +1506,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
     }
   }
   __syncthreads();
+  if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
   // real values: field f, local row lr, column x at element e = (f·half + lr/2)·n + x, part lr & 1
   const T* u = reinterpret_cast<const T*>(buf);
 

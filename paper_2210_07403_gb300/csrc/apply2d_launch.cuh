@@ -142,7 +142,8 @@ ibdl_status launch_col_staged(Geometry* g, const ColParams<float>& cp, cudaStrea
     return fail(IBDL_ERR_UNSUPPORTED, "staged column pass: the column group does not fit shared memory");
   static std::atomic<unsigned long long> d{0};
   IBDL_CUDA(opt_in_smem(kt_colpass<OP, L>, d));
-  const int threads = field_groups_2d(NMAX, L, true) * cp.C * threads_per_seq_2d(L, true);
+  constexpr int NG = field_groups_2d(NMAX, L, true);
+  const int threads = NG * group_threads_2d(NG, cp.C * threads_per_seq_2d(L, true));
   const int units = (n / 2) / cp.C;
   const int grid = persistent_grid(kt_colpass<OP, L>, threads, sh.smem, units);
   ColStageArgs a;
