@@ -128,9 +128,16 @@ static ColParams<T> col_params(Geometry* g, const int* stop) {
   cp.tw = static_cast<const cplx<T>*>(Slot2<T>::tw(g));
   cp.stop = stop;
   cp.late = 0;
+  cp.drop0 = g->lambda == 0.0;
   cp.err = g->err_dev;
   cp.on_in = cp.on_out = g->row_on;
   return cp;
+}
+
+// whether the geometry's spread field has no mean (the analytic dipole without a single layer); in
+// huge boxes other FP32 wavenumbers underflow too, and the symbol could not tell them from k = 0
+static bool no_mean_2d(const Geometry* g) {
+  return g->dipole == IBDL_DIPOLE_ANALYTIC && g->naug == 0 && g->box < 1e12;
 }
 
 // Launch shape of one operator at one precision: threads and shared memory of the three kernels
@@ -225,7 +232,8 @@ static ibdl_status run_op(Geometry* g, const double* in, double* out, cudaStream
     rp.eta_src = 0;
   }
   ColParams<T> cp = col_params<T>(g, stop);
-  if (mode & RUN_LAPLACE) cp.lam = T(0);  // the plain Laplace problem (indicator)
+  if ((OP == OP_SCALAR_AN || OP == OP_STOKES_AN) && !grid_in && no_mean_2d(g)) cp.drop0 = 1;
+  if (mode & RUN_LAPLACE) cp.lam = T(0), cp.drop0 = 1;  // the plain Laplace problem (indicator)
   if (mode & (RUN_LAPLACE | RUN_NO_AUG)) {  // no completed-method terms
     rp.aug = 0;
     rp.eta_src = 0;
@@ -561,6 +569,7 @@ static ibdl_status batch_prepare_t(Batch* B, const int* kptr /* device &st[b].k,
     user[b].io_off = B->off[b];
     kry[b] = user[b];
     col[b] = col_params<T>(g, nullptr);
+    if (no_mean_2d(g)) col[b].drop0 = 1;
     if (kptr) {
       const int* kb = reinterpret_cast<const int*>(reinterpret_cast<const char*>(kptr) + kstride * b);
       kry[b].idx = kb;                               // &st[b].k

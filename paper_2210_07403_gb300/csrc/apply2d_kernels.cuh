@@ -239,6 +239,7 @@ struct ColParams {
   const int* stop;
   int* err;  // the staged column pass sets it to 1 when a bounded wait runs out
   int late;  // as in RowParams
+  int drop0;  // the k = 0 mode is dropped: λ = 0, or a spread whose field has no mean (apply_symbol)
   const unsigned char* on_in;   // rows the spread wrote (NULL: every row; the others are zero)
   const unsigned char* on_out;  // rows the last kernel reads (NULL: every row)
 };
@@ -575,9 +576,10 @@ template <typename T, int OP>
 __device__ __forceinline__ void apply_symbol(const ColParams<T>& p, T lap, T dkx, T dky, const cplx<T>* in,
                                              cplx<T>* out) {
   if (OP == OP_SCALAR_AN || OP == OP_SCALAR_SD || OP == OP_ADJ_AN || OP == OP_ADJ_SD || OP == OP_SL) {
-    // −L⁻¹ ↦ 1/(|k|² + λ), zero mode dropped when λ = 0 (Δ₀⁻¹)
-    const T den = lap + p.lam;
-    const T sig = den != T(0) ? sym_div(p.scale, den) : T(0);
+    // −L⁻¹ ↦ 1/(|k|² + λ), zero mode dropped when λ = 0 (Δ₀⁻¹), and for the analytic dipole spread, which
+    // sums to zero (Σ_a φ'(r + a) = 0 for both kernels): its zero mode holds only rounding, which a
+    // small λ > 0 would amplify by 1/λ
+    const T sig = p.drop0 && sym_zero(lap) ? T(0) : sym_div(p.scale, lap + p.lam);
     if (OP == OP_SCALAR_AN || OP == OP_ADJ_AN || OP == OP_SL) {
       out[0] = cscale(in[0], sig);
     } else if (OP == OP_SCALAR_SD) {
@@ -591,7 +593,7 @@ __device__ __forceinline__ void apply_symbol(const ColParams<T>& p, T lap, T dkx
     }
   } else if (OP == OP_STOKES_T) {
     // transpose of the Stokes multiplier (conjugate symbol): v̂_s = −i k̃·ψ̂/|k|², v̂_g = P̂ψ̂/|k|²
-    const T inv = lap != T(0) ? sym_div(T(1), lap) : T(0);
+    const T inv = sym_zero(lap) ? T(0) : sym_div(T(1), lap);
     const cplx<T> kp = cadd(cscale(in[0], dkx), cscale(in[1], dky));
     const T sc = inv * p.scale;
     // Brinkman (λ > 0): the projected part carries μ/(μ|k|² + λ) in place of 1/|k|²
@@ -601,7 +603,7 @@ __device__ __forceinline__ void apply_symbol(const ColParams<T>& p, T lap, T dkx
     out[2] = cscale(csub(in[1], cscale(kp, dky * inv)), sg);
   } else {
     // Stokes, interior, η = 0: û = (i k̃ ŝ + P̂ ĝ)/|k|², P̂ = I − k̃k̃ᵀ/|k|²
-    const T inv = lap != T(0) ? sym_div(T(1), lap) : T(0);
+    const T inv = sym_zero(lap) ? T(0) : sym_div(T(1), lap);
     cplx<T> gx, gy;
     if (OP == OP_STOKES_AN) {
       gx = in[1];
@@ -615,7 +617,9 @@ __device__ __forceinline__ void apply_symbol(const ColParams<T>& p, T lap, T dkx
     const T sc = inv * p.scale;
     if (p.lam > T(0)) {
       // Brinkman (Sec. 6.3.2): û = i k̃ ŝ/|k|² + μ P̂ ĝ/(μ|k|² + λ), defined at k = 0 as well
-      const T sg = sym_div(p.mu, p.mu * lap + p.lam) * p.scale;
+      // (the analytic dipole's ĝ has no mean: see the scalar symbol)
+      const bool none = OP == OP_STOKES_AN && p.drop0 && sym_zero(lap);
+      const T sg = none ? T(0) : sym_div(p.mu, p.mu * lap + p.lam) * p.scale;
       out[0] = cadd(cscale(is, dkx * sc), cscale(csub(gx, cscale(kg, dkx * inv)), sg));
       out[1] = cadd(cscale(is, dky * sc), cscale(csub(gy, cscale(kg, dky * inv)), sg));
     } else {

@@ -191,6 +191,7 @@ struct Col3Params {
   int n, log2n, C, lc;
   int nf;        // fields transformed (y passes)
   double lam, scale;
+  int drop0;     // the zero mode is dropped: λ = 0, or the spread field has no mean (symbol3)
   const void* lap1;
   const void* der1;
   void* spec;
@@ -474,11 +475,11 @@ struct ZColumnIO {
 };
 
 template <typename T, int OP>
-__device__ __forceinline__ void symbol3(const T* lap1, const T* der1, T lam, T scale, int kx, int ky, int kz,
+__device__ __forceinline__ void symbol3(const T* lap1, const T* der1, T lam, T scale, int drop0, int kx, int ky, int kz,
                                         const cplx<T>* in, cplx<T>* out) {
   const T lap = lap1[kx] + lap1[ky] + lap1[kz];
-  const T den = lap + lam;
-  const T sig = den != T(0) ? sym_div(scale, den) : T(0);
+  // (the analytic dipole spread sums to zero: a small λ > 0 would amplify its zero mode's rounding)
+  const T sig = drop0 && sym_zero(lap) ? T(0) : sym_div(scale, lap + lam);
   if (OP == OP3_SCALAR_AN || OP == OP3_ADJ_AN) {
     out[0] = cscale(in[0], sig);
   } else if (OP == OP3_SCALAR_SD) {
@@ -539,7 +540,7 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
     if (kx != 0) {
 #pragma unroll
       for (int f = 0; f < NIN; ++f) in[f] = res[at(f, q, c, kz)];
-      symbol3<T, OP>(lap1, der1, lam, scale, kx, ky, kz, in, out);
+      symbol3<T, OP>(lap1, der1, lam, scale, p.drop0, kx, ky, kz, in, out);
 #pragma unroll
       for (int f = 0; f < NOUT; ++f) res[at(f, q, c, kz)] = out[f];
       continue;
@@ -566,10 +567,10 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
       Bb[f] = mk(T(0.5) * (Pp.y + P.y), T(0.5) * (P.x - Pp.x));
     }
     cplx<T> oA[NOUT], oB[NOUT], oAp[NOUT], oBp[NOUT];
-    symbol3<T, OP>(lap1, der1, lam, scale, 0, ky, kz, Aa, oA);
-    symbol3<T, OP>(lap1, der1, lam, scale, nh, ky, kz, Ba, oB);
-    symbol3<T, OP>(lap1, der1, lam, scale, 0, kyp, kzp, Ab, oAp);
-    symbol3<T, OP>(lap1, der1, lam, scale, nh, kyp, kzp, Bb, oBp);
+    symbol3<T, OP>(lap1, der1, lam, scale, p.drop0, 0, ky, kz, Aa, oA);
+    symbol3<T, OP>(lap1, der1, lam, scale, p.drop0, nh, ky, kz, Ba, oB);
+    symbol3<T, OP>(lap1, der1, lam, scale, p.drop0, 0, kyp, kzp, Ab, oAp);
+    symbol3<T, OP>(lap1, der1, lam, scale, p.drop0, nh, kyp, kzp, Bb, oBp);
     const bool self = (qp == q) && (kzp == kz);
 #pragma unroll
     for (int f = 0; f < NOUT; ++f) {

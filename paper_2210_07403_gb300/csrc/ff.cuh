@@ -61,6 +61,7 @@ __device__ __forceinline__ ff operator/(ff a, ff b) {
   return ff_fast_two_sum(q1, q2);
 }
 __device__ __forceinline__ ff sym_div(ff a, ff b) { return a / b; }
+__device__ __forceinline__ bool sym_zero(ff a) { return a.hi == 0.0f; }
 __device__ __forceinline__ ff& operator+=(ff& a, ff b) { return a = a + b; }
 
 // The float-float value of a double by integer arithmetic on its bits, so the conversion does not

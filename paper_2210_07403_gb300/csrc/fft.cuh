@@ -65,6 +65,10 @@ __device__ __forceinline__ void dft8(cplx<T>* u) {
   u[7] = b3;
 }
 
+// whether a sum of squares is zero; in FP64 by its bits, which keeps the comparison off the FP64 pipe
+__device__ __forceinline__ bool sym_zero(float a) { return a == 0.0f; }
+__device__ __forceinline__ bool sym_zero(double a) { return __double_as_longlong(a) == 0; }
+
 // a/b of a Fourier symbol: the hardware reciprocal estimate in FP32 (within 2 ulp, well inside the
 // FP32 application's rounding), a corrected quotient in float-float. In FP64 the hardware estimate r
 // (about 20 bits; no FP64-pipe instruction) with one third-order step for the reciprocal,

@@ -271,17 +271,21 @@ static ibdl_status touched_rows(Geometry* g) {
     g->band_cnt[r] = (int)band.size();
     for (const auto& b : band) lists.push_back(b.second);
   }
-  IBDL_TRY(dalloc(&g->row_on, on.size()));
-  IBDL_TRY(dalloc(&g->bands, sizeof(int) * lists.size()));
-  IBDL_CUDA(cudaMemcpy(g->row_on, on.data(), on.size(), cudaMemcpyHostToDevice));
-  IBDL_CUDA(cudaMemcpy(g->bands, lists.data(), sizeof(int) * lists.size(), cudaMemcpyHostToDevice));
-  if (g->dim == 3) {
-    g->nplanes = (int)zs.size();
-    IBDL_TRY(dalloc(&g->plane_on, Q));
-    IBDL_TRY(dalloc(&g->planes, sizeof(int) * zs.size()));
-    IBDL_CUDA(cudaMemcpy(g->plane_on, pl.data(), Q, cudaMemcpyHostToDevice));
-    IBDL_CUDA(cudaMemcpy(g->planes, zs.data(), sizeof(int) * zs.size(), cudaMemcpyHostToDevice));
-  }
+  // one allocation and copy: the lists, the planes, then the masks
+  const size_t ints = lists.size() + zs.size(), bytes = ints * sizeof(int);
+  std::vector<unsigned char> all(bytes + on.size() + pl.size());
+  std::memcpy(all.data(), lists.data(), lists.size() * sizeof(int));
+  std::memcpy(all.data() + lists.size() * sizeof(int), zs.data(), zs.size() * sizeof(int));
+  std::memcpy(all.data() + bytes, on.data(), on.size());
+  std::memcpy(all.data() + bytes + on.size(), pl.data(), pl.size());
+  unsigned char* d = nullptr;
+  IBDL_TRY(dalloc(&d, all.size()));
+  g->bands = reinterpret_cast<int*>(d);
+  g->planes = g->bands + lists.size();
+  g->row_on = d + bytes;
+  g->plane_on = g->row_on + on.size();
+  g->nplanes = (int)zs.size();
+  IBDL_CUDA(cudaMemcpy(d, all.data(), all.size(), cudaMemcpyHostToDevice));
   return IBDL_OK;
 }
 
@@ -290,8 +294,7 @@ static void free_geometry(Geometry* g) {
   void* ptrs[] = {g->perm, g->base, g->cell_start, g->t64.phi, g->t64.dphi, g->t64.wscale, g->t64.nrm,
                   g->t32.phi, g->t32.dphi, g->t32.wscale, g->t32.nrm, g->spec, g->tw64, g->tw32,
                   g->lap64, g->der64, g->lap32, g->der32, g->ubuf, g->tmp_m, g->V, g->gm, g->vec,
-                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->row_on, g->bands,
-                  g->plane_on, g->planes};
+                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->bands};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int i = 0; i < 4; ++i)

@@ -105,7 +105,7 @@ struct Geometry {
   unsigned char* plane_on;  // 3-D: planes with such rows [n/8], and their list
   int* planes;
   int nplanes;
-  int* bands;             // the lists of r = 1, 2, …, one after another
+  int* bands;             // the lists of r = 1, 2, …, one after another (the allocation of all these)
   int band_off[14], band_cnt[14];
   int band_first[14];     // ≥ 0: the bands are one run from this one on (wrapped), short enough to start at once
   PointTable<double> t64;
