@@ -277,11 +277,6 @@ __device__ __forceinline__ Ranges3 band_points3(const int* cell_start, int n, in
 // ------------------------------------------------------------------------------------------
 template <typename T, int OP, int L>
 __global__ void __launch_bounds__(kThreads3) k3_spread_rowfft(Row3Params p) {
-  // programmatic launch: wait for the previous kernel, then let the next one launch; a GMRES
-  // cycle's stop flag is read after the wait (the step just before may have written it)
-  cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
-  if (p.stop && *p.stop) return;
   constexpr int NIN = Traits3<OP>::NIN;
   constexpr int n = 1 << L;
   using PT = typename Prec3<T>::PT;
@@ -298,12 +293,22 @@ __global__ void __launch_bounds__(kThreads3) k3_spread_rowfft(Row3Params p) {
   const int bands = n / R;
   const int unit = p.bands_in ? p.bands_in[blockIdx.x] : (int)blockIdx.x;
   const int z = unit / bands, y0 = (unit - z * bands) * R;
+  // prologue independent of the previous kernel: the band, its points' ranges and the cleared buffer
+  const Ranges3 rg = band_points3(p.cell_start, n, z, y0, R);
+  for (int i = threadIdx.x; i < (int)padded((size_t)seqs * n) * 2; i += blockDim.x) acc[i] = PT(0);
+  // programmatic launch: wait for the previous kernel, then let the next one launch; a GMRES
+  // cycle's stop flag is read after the wait (the step just before may have written it). The later
+  // kernels read it first: they launch once this one has passed its wait, when the step that wrote
+  // it has completed; so a slot after the stop returns without waiting, as in 2-D. What a kernel
+  // does before its wait reads constant tables only.
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  if (p.stop && *p.stop) return;
   const double* pin;
   double* pout;
   resolve_io3(p, pin, pout);
   if (!p.grid_in)  // jump term: out = ±½·in (the gather adds S*u afterwards); none for grid input
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) pout[i] = p.jump * pin[i];
-  for (int i = threadIdx.x; i < (int)padded((size_t)seqs * n) * 2; i += blockDim.x) acc[i] = PT(0);
   __syncthreads();
 
   if (p.grid_in) {  // rows of a grid field ([NIN][z][y][x]) in place of the spread
@@ -315,7 +320,6 @@ __global__ void __launch_bounds__(kThreads3) k3_spread_rowfft(Row3Params p) {
           PT(p.grid_in[(((size_t)f * n + z) * n + y0 + lr) * n + x]);
     }
   }
-  const Ranges3 rg = band_points3(p.cell_start, n, z, y0, R);
   // one thread per (point, stencil row ay): the point's plane and row weights and its density are
   // read once, then the four nodes along x of that row are added
   for (int t = threadIdx.x; t < (p.grid_in ? 0 : rg.total * 4); t += blockDim.x) {
@@ -428,11 +432,7 @@ __device__ __forceinline__ int lane3() {
 
 template <typename T, bool INV, int L>
 __global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
-  // programmatic launch: wait for the previous kernel, then let the next one launch; a GMRES
-  // cycle's stop flag is read after the wait (the step just before may have written it)
-  cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
-  if (p.stop && *p.stop) return;
+  if (p.stop && *p.stop) return;  // final before the wait (see the spread kernel)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int n = 1 << L, nh = n >> 1;
   const int C = p.C;
@@ -445,6 +445,8 @@ __global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
   const int j0 = lane3<T, L>();
   const unsigned in = INV ? 0xffu : mask3(p.rows_in, z * Q + j0), out = INV ? mask3(p.rows_out, z * Q + j0) : 0xffu;
   const YColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, z, k0, p.lc, C, L - 3, in, out};
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   fft3_run<T, INV, L, true>(bufA, p.nf * C, static_cast<const cplx<T>*>(p.tw), GlobLd3<YColumnIO<T>>{io},
                             GlobSt3<YColumnIO<T>>{io});
 }
@@ -495,11 +497,7 @@ __device__ __forceinline__ void symbol3(const T* lap1, const T* der1, T lam, T s
 
 template <typename T, int OP, int L>
 __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
-  // programmatic launch: wait for the previous kernel, then let the next one launch; a GMRES
-  // cycle's stop flag is read after the wait (the step just before may have written it)
-  cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
-  if (p.stop && *p.stop) return;
+  if (p.stop && *p.stop) return;  // final before the wait (see the spread kernel)
   constexpr int NIN = Traits3<OP>::NIN;
   constexpr int NOUT = Traits3<OP>::NOUT;
   constexpr int NMAX = NIN > NOUT ? NIN : NOUT;
@@ -519,10 +517,12 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
     lap1[i] = static_cast<const T*>(p.lap1)[i];
     der1[i] = static_cast<const T*>(p.der1)[i];
   }
-  __syncthreads();
   const int j0 = lane3<T, L>();
   const ZColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, ky1, ky2, k0, lc, C, L - 3,
                         mask3(p.planes_in, j0), mask3(p.planes_out, j0)};
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  __syncthreads();
   // with one column (ky = −ky) only the q = 0 sequences exist: sequence index bi maps to
   // (f·2 + 0)·C + c, so transform all 2·C slots per field and ignore q = 1 (it aliases q = 0)
   fft3_run<T, false, L, true>(bufA, NIN * 2 * C, twg, GlobLd3<ZColumnIO<T>>{io}, SmemSt3<T>());
@@ -612,11 +612,7 @@ struct RowZLoad3 {
 
 template <typename T, int OP, int GMODE, int L>
 __global__ void __launch_bounds__(kThreads3) k3_rowifft_gather(Row3Params p) {
-  // programmatic launch: wait for the previous kernel, then let the next one launch; a GMRES
-  // cycle's stop flag is read after the wait (the step just before may have written it)
-  cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
-  if (p.stop && *p.stop) return;
+  if (p.stop && *p.stop) return;  // final before the wait (see the spread kernel)
   constexpr int NOUT = Traits3<OP>::NOUT;
   using PT = typename Prec3<T>::PT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -632,6 +628,9 @@ __global__ void __launch_bounds__(kThreads3) k3_rowifft_gather(Row3Params p) {
   const int z = unit / bands, y0 = (unit - z * bands) * R;
   const RowZLoad3<T> zl{static_cast<const cplx<T>*>(p.spec), n, nh, z * n + y0, half, n * n,
                         p.rows_out ? p.rows_out + (size_t)z * (n / 8) : nullptr, y0, L - 3};
+  const Ranges3 rg = band_points3(p.cell_start, n, z, y0, R);
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   fft3_run<T, true, L>(bufA, seqs, static_cast<const cplx<T>*>(p.tw), GlobLd3<RowZLoad3<T>>{zl}, SmemSt3<T>());
   __syncthreads();
   const T* u = reinterpret_cast<const T*>(bufA);
@@ -648,7 +647,6 @@ __global__ void __launch_bounds__(kThreads3) k3_rowifft_gather(Row3Params p) {
   const double* pin;
   double* pout;
   resolve_io3(p, pin, pout);
-  const Ranges3 rg = band_points3(p.cell_start, n, z, y0, R);
   for (int t = threadIdx.x; t < rg.total * 4; t += blockDim.x) {
     const int s = rg.at(t >> 2);
     const int ay = t & 3;
