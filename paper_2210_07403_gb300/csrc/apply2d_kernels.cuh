@@ -111,7 +111,7 @@ struct Cfg2 {
   static constexpr int V = lanes_per_thread_2d(L, F32);
   static constexpr int QT = threads_per_seq_2d(L, F32);
   static constexpr int NGRP = field_groups_2d(NF, L, F32);
-  static constexpr int NTW = twiddles8<T, L>();
+  static constexpr int NTW = TwLayout<T, L>::NTW;
   // register budget for twiddles: 42 FP32 registers; 56 in FP64; 28 in float-float, whose
   // arithmetic needs the most temporaries
   static constexpr bool TWR =
@@ -187,7 +187,7 @@ struct RowParams {
   const double* in;   // [c][M] density
   double* out;        // [c][M] result (first kernel stores ½·in, last kernel adds S*u)
   cplx<T>* spec;      // [nf][n][n/2]
-  const cplx<T>* tw;  // [n] e^{−2πi j/n}
+  const cplx<T>* tw;  // the twiddle table (TwLayout)
   const int* stop;    // optional: skip all work when *stop != 0
   double* grid;       // G_GRID: [nf][n][n]
   const int* idx;     // optional: in += (*idx)·vstride, out += (*idx + 1)·vstride (Krylov basis)

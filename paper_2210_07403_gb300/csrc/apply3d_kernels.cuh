@@ -99,7 +99,7 @@ template <typename T, int L>
 struct Cfg3 {
   static constexpr int V = 1;
   static constexpr int QT = (1 << L) / 8;
-  static constexpr int NTW = twiddles8<T, L>();
+  static constexpr int NTW = TwLayout<T, L>::NTW;
   static constexpr bool TWR =
       sizeof(T) == 4 ? NTW <= 21 : (std::is_same<T, ff>::value ? NTW <= 7 : NTW <= 14);
   using TW = std::conditional_t<TWR, TwRegs<T, L>, TwTable<T, L>>;

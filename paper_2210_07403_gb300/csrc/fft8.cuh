@@ -16,8 +16,8 @@
 // buffer per sequence (N + N/8 elements: one pad after every eight keeps the stride-8 writes of the
 // first stage free of bank conflicts).
 //
-// Twiddles come from the table tw[m] = e^{−2πi m/N}: held in registers per lane (read once,
-// before a kernel's dependency wait) or read from the table at each use.
+// Twiddles come from a table (TwLayout): held in registers per lane (read once, before a kernel's
+// dependency wait) or read from the table at each use.
 //
 // FP64 transforms are bound by the FP64 pipe (one warp instruction per 64 cycles and SM
 // sub-partition), so their stages are written for the least number of FP64 instructions: a twiddled
@@ -26,7 +26,7 @@
 // Process. 41 (1993) 93–107, and Goedecker, SIAM J. Sci. Comput. 18 (1997) 1605–1611, describe such
 // forms): 72 instructions instead of 84 for seven complex products and the 8-point DFT; the first
 // stage's √½ factors go into its last additions (52 instead of 56). The error of c·(b_x − t·b_y)
-// is that of c·b_x − s·b_y, however large t is. The table then holds (c, t) of e^{−2πi m/N}, and a
+// is that of c·b_x − s·b_y, however large t is. The table then holds (c, t), and a
 // lane needs four entries per radix-8 stage instead of seven. FP64 applications before / after: 512²
 // Stokes star 131 / 118 µs, 2048² (finite differences, divergence dipole) 791 / 671 µs, 128³ sphere 261 /
 // 249 µs; the error against an 80-bit reference is unchanged (64² circle 4.2e−15 of S*u, 1024² 3.7e−14 /
@@ -63,64 +63,68 @@ struct F8 {
   static constexpr int PN = N + N / 8;                   // padded sequence length in shared memory
 };
 
-// T transforms in the fused form (table entries (cos, tan)); twiddles per lane: 7 per radix-8 stage
-// after the first and (RT − 1) per tail butterfly, in the fused form 4 (w, w², w⁴ and w·e^{−iπ/4})
-// and log2(RT) (w, w²)
+// T transforms in the fused form (table entries (cos, tan)).
 template <typename T>
 constexpr bool kFused8 = std::is_same<T, double>::value;
-template <typename T, int L>
-constexpr int twiddles8() {
-  constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT;
-  return kFused8<T> ? (S8 - 1) * 4 + (LT ? LT * (8 / RT) : 0) : (S8 - 1) * 7 + (LT ? (RT - 1) * (8 / RT) : 0);
-}
 
 __host__ __device__ constexpr int ipow8(int s) { return s == 0 ? 1 : 8 * ipow8(s - 1); }
 
-// table index of the twiddle of stage S, tail butterfly m (0 for radix-8 stages), input r, lane j;
-// r = 9 (fused form): that of r = 1 times e^{−iπ/4}
-template <int L, int S>
-__device__ __forceinline__ int tw_index(int j, int m, int r) {
-  constexpr int S8 = L / 3, N = 1 << L, Q = N / 8;
-  if constexpr (S < S8) {
-    constexpr int p = ipow8(S);
-    if (r == 9) return (j & (p - 1)) * (N / (8 * p)) + N / 8;
-    return r * (j & (p - 1)) * (N / (8 * p));
-  } else {
-    return r * (j + m * Q);
+// The twiddle table, per stage in the order the lanes read it. A radix-8 stage S ≥ 1 with sub-length
+// p = 8^S has NV = 7 values per k = j mod p (w^r, r = 1 … 7), in the fused form 4 (w, w², w⁴ and w·e^{−iπ/4});
+// a tail stage has 8/RT butterflies m of RT − 1 values per lane j (w^r of i = j + m·Q), in the fused
+// form log2(RT) (w, w²). The values of one k form 16-byte chunks (two FP32 values, or one of 16 bytes);
+// chunk c of k lies at (offset of the stage) + c·p + k, so that the lanes of a warp read adjacent
+// chunks. (Read from one table of e^{−2πi m/N} at m = r·k·N/(8p), a warp's loads touched up to 32 cache
+// lines each; the L1 cache was 84 % busy in the 8192² row kernels. Applications before / after: FP32
+// 8192² circle 584 / 499 µs, scalar 4096² 141 / 113, 2048² 41 / 34, Stokes 2048² 124 / 102; FP64 8192² 7774 /
+// 7619, 2048² 420 / 411; float-float Stokes 2048² 424 / 373.)
+template <typename T, int L>
+struct TwLayout {
+  static constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT, Q = (1 << L) / 8;
+  static constexpr int PER = sizeof(T) == 4 ? 2 : 1;      // values per chunk
+  static constexpr int N8 = kFused8<T> ? 4 : 7;           // values of a radix-8 stage
+  static constexpr int NT = kFused8<T> ? LT : RT - 1;     // values of a tail butterfly
+  static constexpr int NTAIL = LT ? NT * (8 / RT) : 0;
+  static constexpr int C8 = (N8 + PER - 1) / PER, CT = (NTAIL + PER - 1) / PER;
+  static constexpr int NTW = (S8 - 1) * N8 + NTAIL;       // values per lane
+  static constexpr int CHUNKS = C8 * ((ipow8(S8) - 8) / 7) + CT * Q;
+  template <int S>
+  static constexpr int NV = S < S8 ? N8 : NTAIL;
+  // the values of stage S on lane j
+  template <int S>
+  __device__ static __forceinline__ void read(const cplx<T>* __restrict__ tab, int j, cplx<T>* w) {
+    constexpr int p = S < S8 ? ipow8(S) : Q, NC = S < S8 ? C8 : CT;
+    const int k = S < S8 ? j & (p - 1) : j;
+    const cplx<T>* t = tab + PER * (C8 * ((ipow8(S < S8 ? S : S8) - 8) / 7) + k);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if constexpr (PER == 2) {
+        const float4 v = reinterpret_cast<const float4*>(t)[c * p];
+        w[2 * c] = mk(T(v.x), T(v.y));
+        if (2 * c + 1 < NV<S>) w[2 * c + 1] = mk(T(v.z), T(v.w));
+      } else {
+        w[c] = t[c * p];
+      }
+    }
   }
-}
+};
 
 // the twiddles of one lane, in registers
 template <typename T, int L>
 struct TwRegs {
-  static constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT;
-  static constexpr int NTW = twiddles8<T, L>();
-  static constexpr int N8 = kFused8<T> ? 4 : 7;       // per radix-8 stage
-  static constexpr int NT = kFused8<T> ? LT : RT - 1;  // per tail butterfly
-  cplx<T> w[NTW > 0 ? NTW : 1];
-  template <int S>
-  __host__ __device__ static constexpr int off(int m, int r) {
-    // fused form: slots 0 … 3 for r = 1, 2, 4, 9
-    const int k = !kFused8<T> ? r - 1 : (r == 9 ? 3 : (r == 4 ? 2 : r - 1));
-    return S < S8 ? (S - 1) * N8 + k : (S8 - 1) * N8 + m * NT + k;
-  }
+  using Y = TwLayout<T, L>;
+  cplx<T> w[Y::NTW > 0 ? Y::NTW : 1];
   __device__ __forceinline__ void load(const cplx<T>* __restrict__ tab, int j) {
-    static_for<1, S8>([&](auto st) {
+    static_for<1, Y::S8 + (Y::LT ? 1 : 0)>([&](auto st) {
       constexpr int S = decltype(st)::value;
-#pragma unroll
-      for (int r = 1; r < 10; ++r)
-        if (kFused8<T> ? (r == 1 || r == 2 || r == 4 || r == 9) : r < 8)
-          w[off<S>(0, r)] = tab[tw_index<L, S>(j, 0, r)];
+      Y::template read<S>(tab, j, w + (S - 1) * Y::N8);
     });
-    if constexpr (LT > 0) {
-#pragma unroll
-      for (int m = 0; m < 8 / RT; ++m)
-#pragma unroll
-        for (int r = 1; r <= NT; ++r) w[off<S8>(m, r)] = tab[tw_index<L, S8>(j, m, r)];
-    }
   }
   template <int S>
-  __device__ __forceinline__ cplx<T> get(int m, int r) const { return w[off<S>(m, r)]; }
+  __device__ __forceinline__ void get(cplx<T>* v) const {
+#pragma unroll
+    for (int i = 0; i < Y::template NV<S>; ++i) v[i] = w[(S - 1) * Y::N8 + i];
+  }
 };
 
 // the twiddles of one lane, read from the table (global memory, L1-cached) at each use
@@ -133,7 +137,7 @@ struct TwTable {
     j = lane;
   }
   template <int S>
-  __device__ __forceinline__ cplx<T> get(int m, int r) const { return tab[tw_index<L, S>(j, m, r)]; }
+  __device__ __forceinline__ void get(cplx<T>* v) const { TwLayout<T, L>::template read<S>(tab, j, v); }
 };
 
 // a·w (forward) or a·conj(w) (inverse)
@@ -198,24 +202,24 @@ __device__ __forceinline__ void dft8_fma(cplx<T>* u) {
 template <typename T, bool INV, int L, int S, class TW>
 __device__ __forceinline__ void f8_stage(cplx<T> (&x)[8], const TW& tw) {
   constexpr int S8 = L / 3, LT = L % 3, RT = 1 << LT;
+  cplx<T> w[8];
+  if constexpr (S > 0) tw.template get<S>(w);
   if constexpr (kFused8<T>) {
     if constexpr (S == 0) {
       dft8_fma<T, INV>(x);
     } else if constexpr (S < S8) {
-      dft8_tan<T, INV>(x, tw.template get<S>(0, 1), tw.template get<S>(0, 2), tw.template get<S>(0, 4),
-                       tw.template get<S>(0, 9));
+      dft8_tan<T, INV>(x, w[0], w[1], w[2], w[3]);
     } else if constexpr (LT == 1) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) bfly_tan<T, INV, false>(x[m], x[m + 4], tw.template get<S>(m, 1));
+      for (int m = 0; m < 4; ++m) bfly_tan<T, INV, false>(x[m], x[m + 4], w[m]);
     } else {
       // radix 4: inputs and outputs of butterfly m at x[m + 2r], r = 0 … 3
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        const cplx<T> w1 = tw.template get<S>(m, 1), w2 = tw.template get<S>(m, 2);
-        bfly_tan<T, INV, false>(x[m], x[m + 4], w2);
-        bfly_tan<T, INV, false>(x[m + 2], x[m + 6], w2);
-        bfly_tan<T, INV, false>(x[m], x[m + 2], w1);     // outputs 0, 2
-        bfly_tan<T, INV, true>(x[m + 4], x[m + 6], w1);  // outputs 1, 3
+        bfly_tan<T, INV, false>(x[m], x[m + 4], w[2 * m + 1]);
+        bfly_tan<T, INV, false>(x[m + 2], x[m + 6], w[2 * m + 1]);
+        bfly_tan<T, INV, false>(x[m], x[m + 2], w[2 * m]);     // outputs 0, 2
+        bfly_tan<T, INV, true>(x[m + 4], x[m + 6], w[2 * m]);  // outputs 1, 3
         const cplx<T> y1 = x[m + 4], y2 = x[m + 2];
         x[m + 2] = y1;
         x[m + 4] = y2;
@@ -224,7 +228,7 @@ __device__ __forceinline__ void f8_stage(cplx<T> (&x)[8], const TW& tw) {
   } else if constexpr (S < S8) {
     if constexpr (S > 0) {
 #pragma unroll
-      for (int r = 1; r < 8; ++r) x[r] = cmul_tw<T, INV>(x[r], tw.template get<S>(0, r));
+      for (int r = 1; r < 8; ++r) x[r] = cmul_tw<T, INV>(x[r], w[r - 1]);
     }
     dft8<T, INV>(x);
   } else {
@@ -235,7 +239,7 @@ __device__ __forceinline__ void f8_stage(cplx<T> (&x)[8], const TW& tw) {
 #pragma unroll
       for (int r = 0; r < RT; ++r) u[r] = x[m + r * MB];
 #pragma unroll
-      for (int r = 1; r < RT; ++r) u[r] = cmul_tw<T, INV>(u[r], tw.template get<S>(m, r));
+      for (int r = 1; r < RT; ++r) u[r] = cmul_tw<T, INV>(u[r], w[m * (RT - 1) + r - 1]);
       if constexpr (RT == 4)
         dft4<T, INV>(u[0], u[1], u[2], u[3]);
       else
@@ -258,7 +262,7 @@ __device__ __forceinline__ int ppos_strided(int j, int s) {
 }
 
 // The same transform for one sequence with the radix-8 stages as a loop over a runtime
-// sub-length p and the twiddles read from the table (index r·k·n/(8p), k = j mod p): one copy of
+// sub-length p and the twiddles read from the table: one copy of
 // the stage code instead of one per stage. For float-float, whose unrolled stages would not fit
 // the instruction cache.
 template <typename T, bool INV, int L, int V>
@@ -272,9 +276,10 @@ __device__ __forceinline__ void f8_fft_rolled(cplx<T> (&x)[1][V][8], cplx<T>* bu
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         if (S > 0) {
-          const int step = ((j0 + v * F::QT) & (p - 1)) << (L - 3 - 3 * S);
+          // (seven 16-byte chunks per k; 8 + … + 8^(S−1) = (p − 8)/7 values of k before this stage)
+          const cplx<T>* t = tab + (p - 8) + ((j0 + v * F::QT) & (p - 1));
 #pragma unroll
-          for (int r = 1; r < 8; ++r) x[0][v][r] = cmul_tw<T, INV>(x[0][v][r], tab[r * step]);
+          for (int r = 1; r < 8; ++r) x[0][v][r] = cmul_tw<T, INV>(x[0][v][r], t[(r - 1) * p]);
         }
         dft8<T, INV>(x[0][v]);
       }

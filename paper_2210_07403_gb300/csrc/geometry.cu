@@ -8,6 +8,7 @@
 
 #include "ff.cuh"
 #include "fft.cuh"
+#include "fft8.cuh"
 
 namespace ibdl {
 
@@ -112,27 +113,74 @@ __global__ void k_tables(int dim, int n, int M, int delta, const double* __restr
   t32.wscale[s] = (float)(w[i] / hd);
 }
 
-// tw[j] = e^{−2πi j/n} = (c, s) in FP32; (c, t) with t = s/c for the FP64 transforms' fused form. At a
-// quarter turn, where c = 0, c = 2^−60 stands for it: c·(b_x − t·b_y) with t = −2^60 is then −s·b_y to
-// rounding (the term 2^−60·b_x lies below it).
-__global__ void k_twiddles(int n, double2* tw64, float2* tw32) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  double s, c;
-  sincospi(-2.0 * (double)j / (double)n, &s, &c);
-  const double cc = c == 0.0 ? 0x1p-60 : c;
-  tw64[j] = make_double2(cc, s / cc);
-  tw32[j] = make_float2((float)c, (float)s);
+// The twiddle table of n-point transforms (TwLayout in fft8.cuh, here for a runtime n): thread e
+// writes the values of chunk e. A value is e^{−2πi m/n} = (c, s), or (c, t) with t = s/c for the FP64
+// transforms' fused form. There, at a quarter turn, where c = 0, c = 2^−60 stands for it:
+// c·(b_x − t·b_y) with t = −2^60 is then −s·b_y to rounding (the term 2^−60·b_x lies below it).
+static __host__ __device__ int tw_chunks8(bool fused, int per) { return ((fused ? 4 : 7) + per - 1) / per; }
+static __host__ __device__ int tw_values_tail(int lt, bool fused) {
+  return lt == 0 ? 0 : (fused ? lt : (1 << lt) - 1) * (8 >> lt);
 }
+template <typename T>
+static int tw_chunks(int n) {
+  constexpr bool fused = kFused8<T>;
+  constexpr int per = sizeof(T) == 4 ? 2 : 1;
+  const int L = __builtin_ctz(n);
+  return tw_chunks8(fused, per) * ((ipow8(L / 3) - 8) / 7) + (tw_values_tail(L % 3, fused) + per - 1) / per * (n / 8);
+}
+template <typename T>
+__device__ void tw_put(cplx<T>* p, double c, double s) { *p = mk(T(c), T(s)); }
+template <>
+__device__ void tw_put<double>(cplx<double>* p, double c, double s) {
+  const double cc = c == 0.0 ? 0x1p-60 : c;
+  *p = mk(cc, s / cc);
+}
+template <typename T>
+__global__ void k_twiddles(int L, int chunks, cplx<T>* tw) {
+  constexpr bool fused = kFused8<T>;
+  constexpr int per = sizeof(T) == 4 ? 2 : 1;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= chunks) return;
+  const int n = 1 << L, Q = n / 8, S8 = L / 3, lt = L % 3, c8 = tw_chunks8(fused, per);
+  // stage S (sub-length p), or the tail (S = S8): chunk c of lane (k) k
+  int S = 1, p = 8, off = 0;
+  while (S < S8 && e >= off + c8 * p) {
+    off += c8 * p;
+    p *= 8;
+    ++S;
+  }
+  if (S == S8) p = Q;
+  const int c = (e - off) / p, k = (e - off) - c * p;
+  for (int i = 0; i < per; ++i) {
+    const int v = c * per + i;
+    long long m = 0;  // (values that pad the last chunk: 1)
+    if (S < S8) {
+      const int step = n / (8 * p), r = !fused ? v + 1 : (v == 2 ? 4 : v + 1);
+      if (fused && v == 3)
+        m = (long long)k * step + n / 8;
+      else if (v < (fused ? 4 : 7))
+        m = (long long)r * k * step;
+    } else if (v < tw_values_tail(lt, fused)) {
+      const int nt = fused ? lt : (1 << lt) - 1;
+      m = (long long)(v % nt + 1) * (k + (v / nt) * Q);
+    }
+    double s, co;
+    sincospi(-2.0 * (double)m / (double)n, &s, &co);
+    tw_put<T>(tw + (size_t)e * per + i, co, s);
+  }
+}
+template <typename T>
+static void launch_twiddles(int n, void* tw, cudaStream_t s) {
+  const int ch = tw_chunks<T>(n);
+  k_twiddles<T><<<(ch + 127) / 128, 128, 0, s>>>(__builtin_ctz(n), ch, static_cast<cplx<T>*>(tw));
+}
+size_t twiddle_bytes_fp64(int n) { return 16 * (size_t)tw_chunks<double>(n); }
+size_t twiddle_bytes_fp32(int n) { return 16 * (size_t)tw_chunks<float>(n); }
 
-// float-float copies of the FP64 twiddles and symbols (hi = fl32(x), lo = fl32(x − hi))
-__global__ void k_ff_tables(int n, const double* lap64, const double* der64, ff* twff, ff* lapff, ff* derff) {
+// float-float copies of the FP64 symbols (hi = fl32(x), lo = fl32(x − hi))
+__global__ void k_ff_tables(int n, const double* lap64, const double* der64, ff* lapff, ff* derff) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  double s, c;
-  sincospi(-2.0 * (double)j / (double)n, &s, &c);
-  twff[2 * j] = ff(c);
-  twff[2 * j + 1] = ff(s);
   lapff[j] = ff(lap64[j]);
   derff[j] = ff(der64[j]);
 }
@@ -174,11 +222,14 @@ ibdl_status fill_geometry_tables(Geometry* g, const double* dX, const double* dN
   k_sort_cells<<<(g->ncell + tb - 1) / tb, tb, 0, s>>>(g->ncell, g->cell_start, g->perm);
   k_tables<<<(M + tb - 1) / tb, tb, 0, s>>>(dim, n, M, g->delta, dX, dN, dW, g->origin[0], g->origin[1], g->origin[2],
                                              g->h, g->perm, g->base, g->t64, g->t32, g->ddphi64);
-  k_twiddles<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->tw64, g->tw32);
+  launch_twiddles<double>(n, g->tw64, s);
+  launch_twiddles<float>(n, g->tw32, s);
   k_symbols<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->box, g->symbol, g->lap64, g->der64, g->lap32, g->der32);
-  if (g->twff)
-    k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->lap64, g->der64, static_cast<ff*>(g->twff),
-                                                  static_cast<ff*>(g->lapff), static_cast<ff*>(g->derff));
+  if (g->twff) {
+    launch_twiddles<ff>(n, g->twff, s);
+    k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->lap64, g->der64, static_cast<ff*>(g->lapff),
+                                                  static_cast<ff*>(g->derff));
+  }
   IBDL_CUDA(cudaGetLastError());
   return IBDL_OK;
 }
@@ -497,14 +548,14 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     const int nf = g->nf_in > g->nf_out ? g->nf_in : g->nf_out;
     g->spec_bytes = (size_t)nf * rows * (n / 2) * sizeof(double2);
     GTRY(dalloc(&g->spec, g->spec_bytes));
-    GTRY(dalloc(&g->tw64, sizeof(double2) * n));
-    GTRY(dalloc(&g->tw32, sizeof(float2) * n));
+    GTRY(dalloc(&g->tw64, twiddle_bytes_fp64(n)));
+    GTRY(dalloc(&g->tw32, twiddle_bytes_fp32(n)));
     GTRY(dalloc(&g->lap64, sizeof(double) * n));
     GTRY(dalloc(&g->der64, sizeof(double) * n));
     GTRY(dalloc(&g->lap32, sizeof(float) * n));
     GTRY(dalloc(&g->der32, sizeof(float) * n));
     // float-float twiddles and symbols (2-D and 3-D)
-    GTRY(dalloc(&g->twff, 2 * sizeof(ff) * n));
+    GTRY(dalloc(&g->twff, 16 * (size_t)tw_chunks<ff>(n)));
     GTRY(dalloc(&g->lapff, sizeof(ff) * n));
     GTRY(dalloc(&g->derff, sizeof(ff) * n));
     GTRY(dalloc(&g->tmp_m, sizeof(double) * (g->ncomp * M + g->ncomp)));  // room for ū / constraint rows
@@ -518,11 +569,14 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     k_sort_cells<<<(g->ncell + tb - 1) / tb, tb, 0, s>>>(g->ncell, g->cell_start, g->perm);
     k_tables<<<(M + tb - 1) / tb, tb, 0, s>>>(dim, n, M, g->delta, dX, dN, dW, g->origin[0], g->origin[1],
                                                g->origin[2], h, g->perm, g->base, g->t64, g->t32, g->ddphi64);
-    k_twiddles<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->tw64, g->tw32);
+    launch_twiddles<double>(n, g->tw64, s);
+    launch_twiddles<float>(n, g->tw32, s);
     k_symbols<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->box, g->symbol, g->lap64, g->der64, g->lap32, g->der32);
-    if (g->twff)
-      k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->lap64, g->der64, static_cast<ff*>(g->twff),
-                                                    static_cast<ff*>(g->lapff), static_cast<ff*>(g->derff));
+    if (g->twff) {
+      launch_twiddles<ff>(n, g->twff, s);
+      k_ff_tables<<<(n + tb - 1) / tb, tb, 0, s>>>(n, g->lap64, g->der64, static_cast<ff*>(g->lapff),
+                                                    static_cast<ff*>(g->derff));
+    }
     GCUDA(cudaGetLastError());
     GCUDA(cudaStreamSynchronize(s));
     GCUDA(cudaEventCreateWithFlags(&g->ev, cudaEventDisableTiming));

@@ -118,13 +118,13 @@ struct Geometry {
   // workspace: half spectra, packed format (see apply kernels): [nf][rows][n/2] complex
   void* spec;      // sized for nf_in fields in FP64
   size_t spec_bytes;
-  double2* tw64;   // [n] (cos, tan) of e^{-2πi j/n} (fft8.cuh)
-  float2* tw32;    // [n] e^{-2πi j/n}
+  void* tw64;      // twiddle tables of the transforms (TwLayout in fft8.cuh)
+  void* tw32;
   // per-axis Fourier symbols indexed by FFT index j (wavenumber 2π m/box, m = j or j − n):
   // lap = symbol of −∂² along one axis, der = k̃ with ∂ ↦ i k̃ (0 at Nyquist)
   double *lap64, *der64;
   float *lap32, *der32;
-  // float-float copies of the twiddles and symbols (2-D): [n] complex pairs and [n] pairs
+  // float-float twiddle table and copies of the symbols
   void* twff;
   void* lapff;
   void* derff;
@@ -273,6 +273,9 @@ ibdl_status field_3d(Geometry* g, const double* Q, double* u, cudaStream_t s);
 ibdl_status adjoint_2d(Geometry* g, int precision, const double* W, double* Z, cudaStream_t s);
 ibdl_status adjoint_3d(Geometry* g, int precision, const double* W, double* Z, cudaStream_t s);
 ibdl_status plan_2d(Geometry* g);
+// bytes of the twiddle tables of n-point transforms (together at most 24·n)
+size_t twiddle_bytes_fp64(int n);
+size_t twiddle_bytes_fp32(int n);
 ibdl_status plan_3d(Geometry* g);
 ibdl_status solve_impl(Geometry* g, const double* Ub, double* Q, const ibdl_solve_opts* o,
                        ibdl_solve_info* info, cudaStream_t s, int op = OPK_A, const double* gsrc = nullptr);

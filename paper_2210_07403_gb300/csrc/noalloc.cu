@@ -156,8 +156,8 @@ extern "C" ibdl_status ibdl_apply_noalloc(const ibdl_geometry_desc* d, int preci
   const int nf = g.nf_in > g.nf_out ? g.nf_in : g.nf_out;
   g.spec_bytes = (size_t)nf * n * (n / 2) * sizeof(double2);
   g.spec = c.take<unsigned char>(g.spec_bytes);
-  g.tw64 = c.take<double2>(n);
-  g.tw32 = c.take<float2>(n);
+  g.tw64 = c.take<unsigned char>(twiddle_bytes_fp64((int)n));
+  g.tw32 = c.take<unsigned char>(twiddle_bytes_fp32((int)n));
   g.lap64 = c.take<double>(n);
   g.der64 = c.take<double>(n);
   g.lap32 = c.take<float>(n);
