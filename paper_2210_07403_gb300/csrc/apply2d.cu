@@ -835,7 +835,7 @@ void batch_shapes_2d(Batch* B) {
 // Stokes 512² 117 / 105), 512 threads in the row kernels where there are about as many bands as SMs,
 // so that no SM takes two (Stokes 512² 92 → 85 µs), else 256. FP32: two columns (8192² with C = 1 / 2
 // 705 / 625 µs, Stokes 4096² 509 / 431), bands of four rows from 512² to 4096² (4096² R = 2 / 4 170 / 149
-// µs), and from 128² 512 threads in the row kernels' loops where the transforms need at most 256 (512² 11.1 →
+// µs), and 512 threads in the row kernels' loops where the transforms need at most 256 (512² 11.1 →
 // 10.0 µs, 2048² 47 → 39; with 384 lanes they only add barriers' width, Stokes 1024² 39.9 → 43.5).
 // Shapes that do not fit give way to smaller ones. IBDL_PLAN_R and IBDL_PLAN_C override (for tuning
 // experiments).
@@ -874,7 +874,7 @@ ibdl_status plan_2d(Geometry* g) {
     // the row kernels' loops (clearing, spreading, unpacking) get at least 256 threads
     int cnt = 0, first;
     if (R) touched_bands(g, R, &cnt, &first);
-    const bool more = f32 ? n >= 128 && n <= 4096 && R && row_threads(nf_held(g, pi), R, L, true, 0) <= 256
+    const bool more = f32 ? n <= 4096 && R && row_threads(nf_held(g, pi), R, L, true, 0) <= 256
                           : cnt >= (g->nf_in > 1 ? 64 : 128) && cnt <= 200;
     g->threads[pi] = more ? 512 : 256;
     TuneVal tv;
