@@ -792,6 +792,20 @@ namespace ibdl {
 // ------------------------------------------------------------------------------------------
 // batched solve driver
 // ------------------------------------------------------------------------------------------
+// CTAs per problem of the batched Arnoldi step (`most`: a single problem's cluster, 16 or 8). A batch
+// runs one cluster per problem, so small clusters leave fewer CTAs and waves, and a slice of a few
+// hundred rows costs little more than one of sixty: the smallest of 4 (2 above 32 problems) whose
+// basis slices fit shared memory. Mixed solves to 1e−10 with 2 / 4 / 16 CTAs: 256 ellipses to 512² 5318 /
+// 5694 / 6095 µs, 64 of them 2014 / 2061 / 2190, 256 to 128² 1757 / 1826 / 2469; 16 Stokes problems to 256²
+// 2092 / 2061 / 2098, 8 to 512² in FP64 5493 / 5427 / 5457.
+static int batch_cluster(const Batch* B, int m, int most) {
+  int nd = 0;
+  for (int b = 0; b < B->count; ++b) nd = std::max(nd, (int)(B->off[b + 1] - B->off[b]));
+  int cl = B->count > 32 ? 2 : 4;
+  while (cl < most && arnoldi_dyn_doubles(m, (nd + cl - 1) / cl, true) * sizeof(double) > 200 * 1024) cl *= 2;
+  return std::min(cl, most);
+}
+
 // Workspace for restart length m: per-problem Krylov bases (offsets voff), states, control
 // block, work vectors, targets, activity flags, and the parameter blocks of the batched apply
 // in Krylov-basis mode (which point at the states).
@@ -801,12 +815,13 @@ static ibdl_status batch_workspace(Batch* B, int m, const ArnoldiCfg& c) {
   B->V = nullptr;
   std::vector<int64_t> voff(B->count);
   std::vector<int> nd(B->count), slice(B->count);
+  const int cl = batch_cluster(B, m, c.cl);
   int64_t vtot = 0;
   for (int b = 0; b < B->count; ++b) {
     nd[b] = (int)(B->off[b + 1] - B->off[b]);
     voff[b] = vtot;
     vtot += (int64_t)(m + 1) * nd[b];
-    slice[b] = (nd[b] + c.cl - 1) / c.cl;
+    slice[b] = (nd[b] + cl - 1) / cl;
   }
   for (int b = 0; b < B->count; ++b) B->voff[b] = voff[b];
   IBDL_CUDA(cudaMalloc((void**)&B->V, sizeof(double) * vtot));
@@ -829,7 +844,7 @@ static ibdl_status batch_workspace(Batch* B, int m, const ArnoldiCfg& c) {
   IBDL_TRY(up(reinterpret_cast<void**>(&B->d_nd), nd.data(), sizeof(int) * B->count));
   IBDL_TRY(up(reinterpret_cast<void**>(&B->d_slice), slice.data(), sizeof(int) * B->count));
   B->m = m;
-  B->cl = c.cl;
+  B->cl = cl;
   for (int i = 0; i < 2; ++i) {
     if (B->exec[i]) cudaGraphExecDestroy(B->exec[i]);
     B->exec[i] = nullptr;
@@ -866,6 +881,14 @@ static cudaError_t kb_arnoldi_attrs() {
   return e;
 }
 
+template <int CL>
+static cudaError_t launch_kb_arnoldi_cl(Batch* B, bool staged, size_t dyn, cudaGraphConditionalHandle cond,
+                                        cudaStream_t s) {
+  cudaError_t e = staged ? kb_arnoldi_attrs<true, CL>() : kb_arnoldi_attrs<false, CL>();
+  if (e != cudaSuccess) return e;
+  return staged ? launch_kb_arnoldi<true, CL>(B, dyn, cond, s) : launch_kb_arnoldi<false, CL>(B, dyn, cond, s);
+}
+
 // the batched cycle graph: while (any problem running) { batched apply on V_b,k ; batched Arnoldi }
 static ibdl_status build_batch_graph(Batch* B, int prec, cudaGraphExec_t* out) {
   *out = nullptr;
@@ -878,16 +901,6 @@ static ibdl_status build_batch_graph(Batch* B, int prec, cudaGraphExec_t* out) {
   const bool staged = staged_bytes <= 200 * 1024;
   const size_t dyn = staged ? staged_bytes : arnoldi_dyn_doubles(B->m, maxslice, false) * sizeof(double);
   if (dyn > 200 * 1024) return fail(IBDL_ERR_UNSUPPORTED, "too many boundary unknowns for the Arnoldi kernel");
-  static bool attrs = false;
-  if (!attrs) {
-    IBDL_CUDA((kb_arnoldi_attrs<true, 8>()));
-    IBDL_CUDA((kb_arnoldi_attrs<false, 8>()));
-    if (B->cl == 16) {
-      IBDL_CUDA((kb_arnoldi_attrs<true, 16>()));
-      IBDL_CUDA((kb_arnoldi_attrs<false, 16>()));
-    }
-    attrs = true;
-  }
   cudaGraph_t graph = nullptr;
   cudaStream_t cs = nullptr;
   IBDL_CUDA(cudaGraphCreate(&graph, 0));
@@ -913,10 +926,12 @@ static ibdl_status build_batch_graph(Batch* B, int prec, cudaGraphExec_t* out) {
     ret = batch_apply_2d(B, prec, 1, B->V, B->V, cs);
     if (ret == IBDL_OK) {
       cudaError_t le;
-      if (B->cl == 16)
-        le = staged ? launch_kb_arnoldi<true, 16>(B, dyn, h, cs) : launch_kb_arnoldi<false, 16>(B, dyn, h, cs);
-      else
-        le = staged ? launch_kb_arnoldi<true, 8>(B, dyn, h, cs) : launch_kb_arnoldi<false, 8>(B, dyn, h, cs);
+      switch (B->cl) {
+        case 16: le = launch_kb_arnoldi_cl<16>(B, staged, dyn, h, cs); break;
+        case 8: le = launch_kb_arnoldi_cl<8>(B, staged, dyn, h, cs); break;
+        case 4: le = launch_kb_arnoldi_cl<4>(B, staged, dyn, h, cs); break;
+        default: le = launch_kb_arnoldi_cl<2>(B, staged, dyn, h, cs);
+      }
       if (le != cudaSuccess) ret = cuda_fail(le, "batched Arnoldi launch");
     }
     cudaGraph_t captured = nullptr;
