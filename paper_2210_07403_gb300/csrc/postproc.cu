@@ -18,15 +18,17 @@
 // operation rounded on its own (no contraction), equal distances ordered by point index.
 //
 // Kernels (the interpolation): k_mark flags the nodes within ceil(m1) + 2 cells of some point
-// (a superset of the nodes to replace), k_compact lists the flagged nodes of Ω, and k_near
-// takes the listed nodes in batches of kNearBatch per warp. For each node in turn the warp scans
-// the points whose cell row lies within K rows of the node (rows of the geometry's cell-sorted
-// order), keeps the three nearest per lane, merges them across the warp, and rescans all M
-// points when the row slab cannot guarantee the result (the third distance not below
-// W = (K − 1)·h); lane k keeps node k's result and finally interpolates it. Within the slab a point
-// whose |dx| is not below W is dropped after one FP64 subtraction and an integer comparison; the
-// distance comparisons run on the integer pipe (non-negative doubles order as their bits), so the
-// FP64 unit only forms the distances.
+// (a superset of the nodes to replace), k_compact lists the row segments of 32 nodes that hold a
+// flagged node of Ω, and k_near takes a segment per warp, a node per lane. The points whose cell lies
+// within K rows and K + 1 columns of the segment (rows of the geometry's cell-sorted order, an integer
+// test of the cell column) are collected in shared memory with their squared y distance, which the
+// whole segment shares; every lane then runs through them and keeps its three nearest: three FP64
+// instructions per point for 32 nodes. A node whose third distance is not below W = (K − 1)·h is scanned
+// again over all M points by the whole warp. The distance comparisons run on the integer pipe
+// (non-negative doubles order as their bits), so the FP64 unit only forms the distances. (With a
+// warp scanning the points of one node after another, five FP64 instructions per 32 points and node,
+// and 16 nodes per warp, some SMs held twice the warps of others: the 1024² circle, 19 000 nodes, took
+// 141 µs.)
 #include <climits>
 #include <cmath>
 #include <cstring>
@@ -72,20 +74,18 @@ __global__ void k_mark(int n, int M, int k1, const int* __restrict__ base, uint8
   }
 }
 
-// list the marked nodes of Ω (warp-aggregated append; the list order is irrelevant)
-__global__ void k_compact(int64_t cells, const uint8_t* __restrict__ marks, const uint8_t* __restrict__ omega,
+// nodes of a row segment
+__host__ __device__ constexpr int segment_width(int n) { return n < 32 ? n : 32; }
+
+// list the row segments that hold a marked node of Ω (the list order is irrelevant)
+__global__ void k_compact(int n, int64_t cells, const uint8_t* __restrict__ marks, const uint8_t* __restrict__ omega,
                           int* __restrict__ list, int* __restrict__ count) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, sw = segment_width(n);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) - lane; b < cells; b += stride) {
     const int64_t i = b + lane;
-    const bool take = i < cells && marks[i] && omega[i];
-    const unsigned m = __ballot_sync(0xffffffffu, take);
-    if (!m) continue;
-    int at = 0;
-    if (lane == 0) at = atomicAdd(count, __popc(m));
-    at = __shfl_sync(0xffffffffu, at, 0);
-    if (take) list[at + __popc(m & ((1u << lane) - 1u))] = (int)i;
+    const unsigned m = __ballot_sync(0xffffffffu, i < cells && marks[i] && omega[i]);
+    if (lane % sw == 0 && ((m >> lane) & (0xffffffffu >> (32 - sw)))) list[atomicAdd(count, 1)] = (int)(i / sw);
   }
 }
 
@@ -95,16 +95,19 @@ struct NearParams {
   unsigned long long r1key;    // bits of (m1·h)²
   unsigned long long slabkey;  // bits of W², W = (K − 1)·h: a slab result is exact when its third
                                // distance is below W
-  unsigned long long slabbits, halfbits;  // bits of W and of L/2
+  unsigned long long halfbits; // bits of L/2
   double halfL;
   double m2h;                  // m2·h
   const double* X;             // [2][M] original order
+  const int* base;             // [2][M] first stencil nodes, sorted order
   const int* perm;             // sorted position → original index
   const int* cell_start;       // [n + 1] rows of constant base y
   const double* Ub;            // [c][M]
   const double* u;             // [c][n][n]
   double* out;                 // [c][n][n]
-  const int* list;
+  const uint8_t* marks;
+  const uint8_t* omega;
+  const int* list;             // segments
   const int* count;
 };
 
@@ -161,15 +164,10 @@ struct Top3 {
   }
 };
 
-// lanes scan sorted positions [a, b) into their own three nearest. With WINDOW a point whose |dx| is
-// not below W is skipped: it is no nearer than W, and a slab result is kept only when its third
-// distance is below W (otherwise every point is rescanned without the window)
-template <bool WINDOW>
-__device__ __forceinline__ void scan_range(const NearParams& p, int a, int b, int lane, double px, double py, Top3& t) {
-  for (int s = a + lane; s < b; s += 32) {
-    const int i = p.perm[s];
+// lanes scan every point into their own three nearest
+__device__ __forceinline__ void scan_all(const NearParams& p, int lane, double px, double py, Top3& t) {
+  for (int i = lane; i < p.M; i += 32) {
     const double dx = mimg_fast(__dsub_rn(p.X[i], px), p);
-    if (WINDOW && absbits(dx) >= p.slabbits) continue;
     const double dy = mimg_fast(__dsub_rn(p.X[p.M + i], py), p);
     t.insert(dbits(sqdist(dx, dy)), i);
   }
@@ -269,60 +267,86 @@ __device__ void near_tail(const NearParams& p, int node, const int* i3) {
   }
 }
 
-// Each warp takes kNearBatch listed nodes at a time: for each in turn all lanes scan its candidate
-// points and merge; lane k keeps node k's three nearest. Then lanes 0..kNearBatch−1 each finish
-// their own node, so the FP64 arithmetic of the interpolation runs on many lanes instead of one.
-// The warp's nodes are scanned one after another (a latency-bound chain), so the batch trades the
-// chain's length against the lanes the interpolation keeps busy; adjacent batches stay in one block
-// (they share slab points in L1).
-constexpr int kNearBatch = 16;
-__global__ void __launch_bounds__(kPPThreads, 2) k_near(NearParams p) {
-  const int lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int warps = gridDim.x * (blockDim.x >> 5);
+// One warp per block: the segments (about 1 000 at 1024²) then spread evenly over the SMs.
+constexpr int kNearCap = 128;  // points collected before the lanes run through them
+__global__ void __launch_bounds__(32) k_near(NearParams p) {
+  __shared__ double cx[kNearCap], cy2[kNearCap];
+  __shared__ int ci[kNearCap];
+  const int lane = threadIdx.x;
   const int count = *p.count;
-  const int n = p.n;
+  const int n = p.n, sw = segment_width(n);
   const bool whole = 2 * p.K + 3 >= n;
-  for (int base = gw * kNearBatch; base < count; base += warps * kNearBatch) {
-    const int nb = min(kNearBatch, count - base);
-    int mine[3] = {-1, -1, -1};
-    for (int k = 0; k < nb; ++k) {
-      const int node = p.list[base + k];
-      const int ix = node % n, iy = node / n;
-      const double px = node_x(p, ix), py = node_y(p, iy);
-      Top3 t;
-      t.init();
-      if (whole) {
-        scan_range<false>(p, 0, p.M, lane, px, py, t);
-      } else {
-        const int lo = iy - p.K - 2, hi = iy + p.K + 1;  // cell rows [lo, hi), wrapped
-        if (lo < 0) {
-          scan_range<true>(p, p.cell_start[lo + n], p.cell_start[n], lane, px, py, t);
-          scan_range<true>(p, p.cell_start[0], p.cell_start[hi], lane, px, py, t);
-        } else if (hi > n) {
-          scan_range<true>(p, p.cell_start[lo], p.cell_start[n], lane, px, py, t);
-          scan_range<true>(p, p.cell_start[0], p.cell_start[hi - n], lane, px, py, t);
-        } else {
-          scan_range<true>(p, p.cell_start[lo], p.cell_start[hi], lane, px, py, t);
+  for (int q = blockIdx.x; q < count; q += gridDim.x) {
+    const int cell0 = p.list[q] * sw;
+    const int iy = cell0 / n, x0 = cell0 - iy * n;
+    const bool take = lane < sw && p.marks[cell0 + lane] && p.omega[cell0 + lane];
+    const double px = node_x(p, x0 + lane), py = node_y(p, iy);
+    Top3 t;
+    t.init();
+    int cnt = 0;
+    auto flush = [&]() {
+      __syncwarp();
+#pragma unroll 4
+      for (int c = 0; c < cnt; ++c) {
+        const double dx = mimg_fast(__dsub_rn(cx[c], px), p);
+        t.insert(dbits(__dadd_rn(__dmul_rn(dx, dx), cy2[c])), ci[c]);
+      }
+      __syncwarp();
+      cnt = 0;
+    };
+    // sorted positions [a, b): the points whose cell column is within K + 1 of the segment
+    auto collect = [&](int a, int b) {
+      for (int s0 = a; s0 < b; s0 += 32) {
+        const int s = s0 + lane;
+        bool in = s < b;
+        if (in && !whole) in = ((p.base[s] + 1 - (x0 - p.K - 1)) & (n - 1)) <= sw + 2 * p.K + 1;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) {
+          const int i = p.perm[s], at = cnt + __popc(m & ((1u << lane) - 1u));
+          const double dy = mimg_fast(__dsub_rn(p.X[p.M + i], py), p);
+          cx[at] = p.X[i];
+          cy2[at] = __dmul_rn(dy, dy);
+          ci[at] = i;
         }
+        cnt += __popc(m);
+        if (cnt > kNearCap - 32) flush();
       }
-      unsigned long long key[3];
-      int idx[3];
-      warp_top3(t, key, idx);
-      // not within m1·h of Γ (a point beyond the slab or the window is farther still)
-      if (!(key[0] < p.r1key)) continue;
-      if (!whole && !(key[2] < p.slabkey)) {
-        t.init();
-        scan_range<false>(p, 0, p.M, lane, px, py, t);
-        warp_top3(t, key, idx);
-      }
-      if (lane == k) {
-        mine[0] = idx[0];
-        mine[1] = idx[1];
-        mine[2] = idx[2];
+    };
+    if (whole) {
+      collect(0, p.M);
+    } else {
+      const int lo = iy - p.K - 2, hi = iy + p.K + 1;  // rows [lo, hi) of base nodes, wrapped
+      if (lo < 0) {
+        collect(p.cell_start[lo + n], p.cell_start[n]);
+        collect(p.cell_start[0], p.cell_start[hi]);
+      } else if (hi > n) {
+        collect(p.cell_start[lo], p.cell_start[n]);
+        collect(p.cell_start[0], p.cell_start[hi - n]);
+      } else {
+        collect(p.cell_start[lo], p.cell_start[hi]);
       }
     }
-    if (mine[0] >= 0) near_tail(p, p.list[base + lane], mine);
+    flush();
+    // not within m1·h of Γ (a point outside the rows and columns collected is farther still)
+    const bool near = take && t.k0 < p.r1key;
+    for (unsigned redo = __ballot_sync(0xffffffffu, near && !whole && !(t.k2 < p.slabkey)); redo; redo &= redo - 1) {
+      const int k = __ffs(redo) - 1;
+      Top3 a;
+      a.init();
+      scan_all(p, lane, node_x(p, x0 + k), py, a);
+      unsigned long long key[3];
+      int idx[3];
+      warp_top3(a, key, idx);
+      if (lane == k) {
+        t.i0 = idx[0];
+        t.i1 = idx[1];
+        t.i2 = idx[2];
+      }
+    }
+    if (near) {
+      const int mine[3] = {t.i0, t.i1, t.i2};
+      near_tail(p, cell0 + lane, mine);
+    }
   }
 }
 
@@ -385,7 +409,7 @@ ibdl_status near_boundary_impl(Geometry* g, const double* Ub, const double* u, c
   const int k1 = (int)std::ceil(m1) + 2;
   k_mark<<<pp_blocks((int64_t)g->M * (2 * k1 + 1) * (2 * k1 + 1)), kPPThreads, 0, s>>>(n, (int)g->M, k1, g->base,
                                                                                         marks);
-  k_compact<<<pp_blocks(cells), kPPThreads, 0, s>>>(cells, marks, omega, list, count);
+  k_compact<<<pp_blocks(cells), kPPThreads, 0, s>>>(n, cells, marks, omega, list, count);
   NearParams p;
   p.n = n;
   p.M = (int)g->M;
@@ -402,18 +426,20 @@ ibdl_status near_boundary_impl(Geometry* g, const double* Ub, const double* u, c
   p.halfL = 0.5 * g->box;
   std::memcpy(&p.r1key, &r1sq, 8);
   std::memcpy(&p.slabkey, &slabsq, 8);
-  std::memcpy(&p.slabbits, &slab, 8);
   std::memcpy(&p.halfbits, &p.halfL, 8);
   p.m2h = m2 * g->h;
   p.X = g->X64;
+  p.base = g->base;
   p.perm = g->perm;
   p.cell_start = g->cell_start;
   p.Ub = Ub;
   p.u = u;
   p.out = out;
+  p.marks = marks;
+  p.omega = omega;
   p.list = list;
   p.count = count;
-  k_near<<<152 * 4, kPPThreads, 0, s>>>(p);
+  k_near<<<152 * 16, 32, 0, s>>>(p);
   g->launches += 3;
   IBDL_CUDA(cudaGetLastError());
   return IBDL_OK;
