@@ -46,6 +46,7 @@ struct Slot2<double> {
   static constexpr int pi = 0;
   static const PointTable<double>& points(const Geometry* g) { return g->t64; }
   static const void* tw(const Geometry* g) { return g->tw64; }
+  static const void* tw_few(const Geometry* g) { return g->tw64_few; }
   static const void* lap(const Geometry* g) { return g->lap64; }
   static const void* der(const Geometry* g) { return g->der64; }
 };
@@ -54,6 +55,7 @@ struct Slot2<float> {
   static constexpr int pi = 1;
   static const PointTable<float>& points(const Geometry* g) { return g->t32; }
   static const void* tw(const Geometry* g) { return g->tw32; }
+  static const void* tw_few(const Geometry*) { return nullptr; }
   static const void* lap(const Geometry* g) { return g->lap32; }
   static const void* der(const Geometry* g) { return g->der32; }
 };
@@ -62,6 +64,7 @@ struct Slot2<ff> {
   static constexpr int pi = 2;
   static const PointTable<double>& points(const Geometry* g) { return g->t64; }
   static const void* tw(const Geometry* g) { return g->twff; }
+  static const void* tw_few(const Geometry* g) { return g->twff_few; }
   static const void* lap(const Geometry* g) { return g->lapff; }
   static const void* der(const Geometry* g) { return g->derff; }
 };
@@ -143,18 +146,18 @@ static bool no_mean_2d(const Geometry* g) {
 // Launch shape of one operator at one precision: threads and shared memory of the three kernels
 // for band height R, column group C and the row kernels' least thread count `floor`, or an error
 // if they do not fit.
-static int row_threads(int nf, int R, int L, bool f32, int floor) {
-  const int ng = field_groups_2d(nf, L, f32);
-  const int need = ng * group_threads_2d(ng, (R / 2) * threads_per_seq_2d(L, f32));
+static int row_threads(int nf, int R, int L, bool f32, int floor, int E = 8) {
+  const int ng = field_groups_2d(nf, L, f32, E);
+  const int need = ng * group_threads_2d(ng, (R / 2) * threads_per_seq_2d(L, f32, E));
   return need > floor ? need : (floor < kMaxThreads2d ? floor : kMaxThreads2d);
 }
-static int col_threads(int nf, int C, int L, bool f32) {
-  const int ng = field_groups_2d(nf, L, f32);
-  return ng * group_threads_2d(ng, C * threads_per_seq_2d(L, f32));
+static int col_threads(int nf, int C, int L, bool f32, int E = 8) {
+  const int ng = field_groups_2d(nf, L, f32, E);
+  return ng * group_threads_2d(ng, C * threads_per_seq_2d(L, f32, E));
 }
 
 template <typename T, int OP>
-static ibdl_status launch_shape(const Geometry* g, int R, int C, int floor, Launch2D* lc) {
+static ibdl_status launch_shape(const Geometry* g, int R, int C, int floor, Launch2D* lc, bool single = true) {
   // one field per launch: every kernel holds one field
   const bool split = g->split[Slot2<T>::pi] != 0;
   const int NIN = split ? 1 : Traits<OP>::NIN, NOUT = split ? 1 : Traits<OP>::NOUT;
@@ -169,9 +172,15 @@ static ibdl_status launch_shape(const Geometry* g, int R, int C, int floor, Laun
   lc->smem_gather = smem_rows_2d<T>(NOUT, R, L);
   lc->smem_col = smem_cols_2d<T>(NMAX, C, L);
   constexpr bool f32 = sizeof(T) == 4;
-  lc->threads_row = row_threads(NIN, R, L, f32, floor);
-  lc->threads_gather = row_threads(NOUT, R, L, f32, floor);
-  lc->threads_col = col_threads(NMAX, C, L, f32);
+  // few elements per lane: two-row bands and single columns of a geometry that has the table, one
+  // thread group per field
+  const int few = few_elements_2d<T>(L);
+  const int E = single && few != 8 && Slot2<T>::tw_few(g) && R == 2 && C == 1 && !split &&
+                        field_groups_2d(NMAX, L, f32, few) == NMAX ? few : 8;
+  lc->elems = E;
+  lc->threads_row = row_threads(NIN, R, L, f32, floor, E);
+  lc->threads_gather = row_threads(NOUT, R, L, f32, floor, E);
+  lc->threads_col = col_threads(NMAX, C, L, f32, E);
   if (lc->smem_row > kSmemLimit2d || lc->smem_gather > kSmemLimit2d || lc->smem_col > kSmemLimit2d)
     return fail(IBDL_ERR_UNSUPPORTED, "grid too large for the shared-memory FFT at this precision");
   if (lc->threads_row > kMaxThreads2d || lc->threads_gather > kMaxThreads2d || lc->threads_col > kMaxThreads2d)
@@ -252,6 +261,7 @@ static ibdl_status run_op(Geometry* g, const double* in, double* out, cudaStream
     rp.on_out = cp.on_out = nullptr;
     lc.units_out = g->n / rp.R;
   }
+  if (lc.elems != 8) rp.tw = cp.tw = static_cast<const cplx<T>*>(Slot2<T>::tw_few(g));
   rp.late = late_rows_2d(pi, Traits<OP>::NIN, lc.units_in);
   cp.late = pi == 2 && Traits<OP>::NIN > 1;
   return launch_for_size<T, OP, kMinL2d>(log2i(g->n), g, rp, cp, lc, s);
@@ -480,7 +490,7 @@ template <typename T, int OP>
 static ibdl_status batch_shape(Batch* B, Geometry* g, int pi) {
   if (g->split[pi]) return fail(IBDL_ERR_UNSUPPORTED, "batched launches hold every field of a band at once");
   Launch2D lc;
-  IBDL_TRY((launch_shape<T, OP>(g, g->rows_per_cta[pi], g->cols_per_cta[pi], g->threads[pi], &lc)));
+  IBDL_TRY((launch_shape<T, OP>(g, g->rows_per_cta[pi], g->cols_per_cta[pi], g->threads[pi], &lc, false)));
   BatchSize& z = B->lv[pi][log2i(g->n)];
   z.smem_row = std::max(z.smem_row, lc.smem_row);
   z.smem_col = std::max(z.smem_col, lc.smem_col);

@@ -94,29 +94,50 @@ constexpr int kMinL2d = 4, kMaxL2d = 13;
 __host__ __device__ constexpr int lanes_per_thread_2d(int L, bool f32) {
   return f32 ? (L >= 13 ? 4 : (L >= 11 ? 2 : 1)) : (L >= 13 ? 2 : 1);
 }
-__host__ __device__ constexpr int threads_per_seq_2d(int L, bool f32) { return (1 << L) / 8 / lanes_per_thread_2d(L, f32); }
+__host__ __device__ constexpr int threads_per_seq_2d(int L, bool f32, int E = 8) {
+  return (1 << L) / E / (E == 8 ? lanes_per_thread_2d(L, f32) : 1);
+}
+
+// Elements per lane of a single problem's FP64 and float-float kernels with two-row bands and single
+// columns, where a grid leaves most of the GPU idle (8: the ordinary kernels only). An FP64 warp
+// instruction takes about 64 cycles whatever its active lanes, so the 312 instructions of a 64-point
+// column on eight lanes took 10 µs on one sub-partition, three of four idle. Applications back to back
+// with 8 / few elements (µs): FP64 scalar 64² 32.1 / 13.6, 256² 41.3 / 21.9, Stokes 64² 37.0 / 17.4, 256² 49.8 /
+// 37.9; float-float scalar 64² 23.4 / 11.0, 256² 30.1 / 15.9, 512² (four elements) 29.5 / 21.8, Stokes 512² 49.0 /
+// 45.1. From 512² one FP64 warp per sub-partition is there anyhow. Batches keep the ordinary kernels,
+// whose operations per element are fewer.
+template <typename T>
+constexpr int few_elements_2d(int L) {
+  return sizeof(T) == 4 ? 8 : (L <= 8 ? 2 : (!std::is_same<T, double>::value && L == 9 ? 4 : 8));
+}
 
 // Thread groups across the NF fields of a kernel: one group per field when NF·QT threads fit in a
 // CTA (each thread transforms one field), else a single group that transforms the fields one
 // after another.
-__host__ __device__ constexpr int field_groups_2d(int nf, int L, bool f32) {
-  return nf * threads_per_seq_2d(L, f32) <= kMaxThreads2d ? nf : 1;
+__host__ __device__ constexpr int field_groups_2d(int nf, int L, bool f32, int E = 8) {
+  return nf * threads_per_seq_2d(L, f32, E) <= kMaxThreads2d ? nf : 1;
 }
+
+template <typename T, int L, int E>
+struct FewTw {
+  using type = TwFew<T, L, E == 8 ? 2 : E>;
+};
 
 // Per-precision register policy: twiddles in registers when they fit the budget, else read from
 // the table at each use.
-template <typename T, int L, int NF>
+template <typename T, int L, int NF, int E = 8>
 struct Cfg2 {
   static constexpr bool F32 = sizeof(T) == 4;
-  static constexpr int V = lanes_per_thread_2d(L, F32);
-  static constexpr int QT = threads_per_seq_2d(L, F32);
-  static constexpr int NGRP = field_groups_2d(NF, L, F32);
+  static constexpr int V = E == 8 ? lanes_per_thread_2d(L, F32) : 1;
+  static constexpr int QT = threads_per_seq_2d(L, F32, E);
+  static constexpr int NGRP = field_groups_2d(NF, L, F32, E);
   static constexpr int NTW = TwLayout<T, L>::NTW;
   // register budget for twiddles: 42 FP32 registers; 56 in FP64; 28 in float-float, whose
   // arithmetic needs the most temporaries
   static constexpr bool TWR =
       F32 ? (NTW * V <= 21) : (std::is_same<T, ff>::value ? (NTW * V <= 7) : (NTW * V <= 14));
-  using TW = std::conditional_t<TWR, TwRegs<T, L>, TwTable<T, L>>;
+  using TW = typename std::conditional_t<E == 8, std::conditional<TWR, TwRegs<T, L>, TwTable<T, L>>,
+                                         FewTw<T, L, E>>::type;
 };
 
 // Column kernels (and the row kernels, with the row pairs of a band in place of the columns):
@@ -258,6 +279,19 @@ template <typename P>
 __device__ __forceinline__ unsigned rows_on(const unsigned char* on, const P& j) {
   return on ? (unsigned)on[j] : 0xffu;
 }
+// bit s: row j + s·n/E, for lanes of E elements
+template <int L, int E>
+__device__ __forceinline__ unsigned lane_rows_on(const unsigned char* on, int j) {
+  if constexpr (E == 8) return rows_on(on, j);
+  constexpr int n = 1 << L;
+  unsigned m = 0;
+#pragma unroll
+  for (int s = 0; s < E; ++s) {
+    const int row = j + s * (n / E);
+    m |= ((rows_on(on, row & (n / 8 - 1)) >> (row / (n / 8))) & 1u) << s;
+  }
+  return m;
+}
 
 // Sorted points whose base row lies in the cell rows [r0 − 3, r0 + R) (mod n): at most two
 // contiguous ranges of the cell-sorted order.
@@ -342,7 +376,7 @@ __device__ __forceinline__ SpreadItem<typename Prec2<T>::PT> spread_item(const R
 // SPLIT: one input field (p.fsel) per launch, for grids whose row bands of every field do not
 // fit shared memory together: the band holds that field only, and the first launch (field 0)
 // also writes the jump term and the completed method's rows.
-template <typename T, int OP, int L, bool PF = true, bool SPLIT = false>
+template <typename T, int OP, int L, bool PF = true, bool SPLIT = false, int E = 8>
 __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int ord, int nords,
                                                    unsigned char* smem_raw) {
   // the band (ord of nords in this launch)
@@ -350,8 +384,8 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   constexpr int NIN = Traits<OP>::NIN;
   constexpr int NB = SPLIT ? 1 : NIN;  // fields held in shared memory
   constexpr int NC = Traits<OP>::C;
-  using CF = Cfg2<T, L, NB>;
-  using F = F8<L, CF::V>;
+  using CF = Cfg2<T, L, NB, E>;
+  using F = F8<L, CF::V, E>;
   using PT = typename Prec2<T>::PT;
   constexpr int n = F::N, V = CF::V, QT = CF::QT, NGRP = CF::NGRP;
   const int R = p.R, half = R >> 1, M = p.M;
@@ -512,19 +546,19 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   for (int k = 0; k < NB / NGRP; ++k) {
     const int f = g + k * NGRP;
     cplx<T>* sb = buf + ((size_t)f * half + rp) * PN;
-    cplx<T> x[1][V][8];
+    cplx<T> x[1][V][E];
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) x[0][v][s] = Prec2<T>::acc_load(sb, ppos_strided<F::Q>(j0 + v * QT, s));
+        for (int s = 0; s < E; ++s) x[0][v][s] = Prec2<T>::acc_load(sb, ppos_strided<F::Q>(j0 + v * QT, s));
     }
-    f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, active);
+    fft_lanes<T, false, L, V, E>(x, sb, j0, tw, active);
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) sb[ppos_strided<F::Q>(j0 + v * QT, s)] = x[0][v][s];
+        for (int s = 0; s < E; ++s) sb[ppos_strided<F::Q>(j0 + v * QT, s)] = x[0][v][s];
     }
   }
   __syncthreads();
@@ -556,10 +590,10 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   }
 }
 
-template <typename T, int OP, int L>
+template <typename T, int OP, int L, int E = 8>
 __global__ void __launch_bounds__(kMaxThreads2d) k_spread_rowfft(RowParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  spread_rowfft_body<T, OP, L>(p, blockIdx.x, gridDim.x, smem_raw);
+  spread_rowfft_body<T, OP, L, true, false, E>(p, blockIdx.x, gridDim.x, smem_raw);
 }
 // one input field (p.fsel) per launch
 template <typename T, int OP, int L>
@@ -667,19 +701,19 @@ __device__ __forceinline__ int col_at(int f, int m, int k, int R) {
 }
 // row j + s·Q of a lane (j < Q = n/8): with R ≤ Q (the planner keeps it so) the rows j + s·Q
 // lie in bands s·Q/R apart at the same offset, so the element is col_at(f, j, k, R) + s·Q·n/2
-template <int L>
+template <int L, int E = 8>
 __device__ __forceinline__ int col_at_s(int f, int j, int s, int k, int R) {
-  constexpr int Q = (1 << L) / 8, nh = (1 << L) / 2;
+  constexpr int Q = (1 << L) / E, nh = (1 << L) / 2;
   return col_at<L>(f, j, k, R) + s * (Q * nh);
 }
 
-template <typename T, int OP, int L, bool PF = true>
+template <typename T, int OP, int L, bool PF = true, int E = 8>
 __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, unsigned char* smem_raw) {
   constexpr int NIN = Traits<OP>::NIN;
   constexpr int NOUT = Traits<OP>::NOUT;
   constexpr int NMAX = NIN > NOUT ? NIN : NOUT;
-  using CF = Cfg2<T, L, NMAX>;
-  using F = F8<L, CF::V>;
+  using CF = Cfg2<T, L, NMAX, E>;
+  using F = F8<L, CF::V, E>;
   constexpr int n = F::N, nh = n / 2, V = CF::V, QT = CF::QT, NGRP = CF::NGRP, Q = F::Q;
   const int C = p.C, R = p.R;
   const int k0 = unit * C;
@@ -700,7 +734,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
   constexpr bool PREF = PF && NIN == 1 && NOUT == 1;
   const bool packed = k0 == 0;  // uniform over the CTA: column 0 holds kx = 0 and kx = n/2
   T lapx = T(0), derx = T(0), lapn = T(0), dern = T(0);
-  T lapy[PREF ? V : 1][8], dery[PREF ? V : 1][8];
+  T lapy[PREF ? V : 1][E], dery[PREF ? V : 1][E];
   if (active) {
     lapx = p.lap1[kx];
     derx = p.der1[kx];
@@ -710,7 +744,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
+        for (int s = 0; s < E; ++s) {
           lapy[v][s] = p.lap1[j0 + v * QT + s * Q];
           dery[v][s] = p.der1[j0 + v * QT + s * Q];
         }
@@ -726,8 +760,8 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
   unsigned oni[V], ono[V];  // the lane's rows to read and to store
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    oni[v] = rows_on(p.on_in, j0 + v * QT);
-    ono[v] = rows_on(p.on_out, j0 + v * QT);
+    oni[v] = lane_rows_on<L, E>(p.on_in, j0 + v * QT);
+    ono[v] = lane_rows_on<L, E>(p.on_out, j0 + v * QT);
   }
   cudaGridDependencySynchronize();
   if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
@@ -735,15 +769,15 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
   if constexpr (NIN == 1 && NOUT == 1) {
     // one field in and out: the symbol is applied to the registers between the transforms
     cplx<T>* sb = buf + (size_t)c * PN;
-    cplx<T> x[1][V][8];
+    cplx<T> x[1][V][E];
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
-          x[0][v][s] = (oni[v] >> s) & 1u ? p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, R)] : mk(T(0), T(0));
+        for (int s = 0; s < E; ++s)
+          x[0][v][s] = (oni[v] >> s) & 1u ? p.spec[col_at_s<L, E>(0, j0 + v * QT, s, kx, R)] : mk(T(0), T(0));
     }
-    f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, active);
+    fft_lanes<T, false, L, V, E>(x, sb, j0, tw, active);
     if (packed) {
       // the packed column needs P(−ky): every lane stores its own positions (free of conflicts
       // with the last exchange, which read only those), then reads the partner's
@@ -751,7 +785,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
+          for (int s = 0; s < E; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
       }
       __syncthreads();
     }
@@ -759,7 +793,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
+        for (int s = 0; s < E; ++s) {
           const cplx<T> in[1] = {x[0][v][s]};
           cplx<T> out[1];
           const int ky = j0 + v * QT + s * Q;
@@ -774,14 +808,14 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
         }
     }
     // (the inverse transform's first exchange barrier orders the partner reads before its writes)
-    f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, active);
+    fft_lanes<T, true, L, V, E>(x, sb, j0, tw, active);
     if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
-          if ((ono[v] >> s) & 1u) p.spec[col_at_s<L>(0, j0 + v * QT, s, kx, R)] = x[0][v][s];
+        for (int s = 0; s < E; ++s)
+          if ((ono[v] >> s) & 1u) p.spec[col_at_s<L, E>(0, j0 + v * QT, s, kx, R)] = x[0][v][s];
     }
   } else {
     // forward transforms of the NIN input fields, results left in shared memory
@@ -790,20 +824,20 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
       const int f = g + k * NGRP;
       const bool act = active && f < NIN;
       cplx<T>* sb = buf + ((size_t)f * C + c) * PN;
-      cplx<T> x[1][V][8];
+      cplx<T> x[1][V][E];
       if (act) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s)
-            x[0][v][s] = (oni[v] >> s) & 1u ? p.spec[col_at_s<L>(f, j0 + v * QT, s, kx, R)] : mk(T(0), T(0));
+          for (int s = 0; s < E; ++s)
+            x[0][v][s] = (oni[v] >> s) & 1u ? p.spec[col_at_s<L, E>(f, j0 + v * QT, s, kx, R)] : mk(T(0), T(0));
       }
-      f8_fft<T, false, L, V, 1>(x, sb, 0, j0, tw, act);
+      fft_lanes<T, false, L, V, E>(x, sb, j0, tw, act);
       if (act) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
+          for (int s = 0; s < E; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
       }
     }
     __syncthreads();
@@ -815,7 +849,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) {
+          for (int s = 0; s < E; ++s) {
             if (s % NGRP != g) continue;
             const int ky = j0 + v * QT + s * Q;
             cplx<T> in[NIN], o[NOUT];
@@ -827,12 +861,12 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
           }
       }
     } else {
-      cplx<T> o[V][8][NOUT];
+      cplx<T> o[V][E][NOUT];
       if (active) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) {
+          for (int s = 0; s < E; ++s) {
             if (s % NGRP != g) continue;
             const int ky = j0 + v * QT + s * Q;
             cplx<T> in[NIN];
@@ -853,7 +887,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) {
+          for (int s = 0; s < E; ++s) {
             if (s % NGRP != g) continue;
 #pragma unroll
             for (int f = 0; f < NOUT; ++f) buf[((size_t)f * C + c) * PN + ppos_strided<Q>(j0 + v * QT, s)] = o[v][s][f];
@@ -867,21 +901,21 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
       const int f = g + k * NGRP;
       const bool act = active && f < NOUT;
       cplx<T>* sb = buf + ((size_t)f * C + c) * PN;
-      cplx<T> x[1][V][8];
+      cplx<T> x[1][V][E];
       if (act) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s) x[0][v][s] = sb[ppos_strided<Q>(j0 + v * QT, s)];
+          for (int s = 0; s < E; ++s) x[0][v][s] = sb[ppos_strided<Q>(j0 + v * QT, s)];
       }
-      f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, act);
+      fft_lanes<T, true, L, V, E>(x, sb, j0, tw, act);
       if (PF && p.late && k + 1 == (NOUT + NGRP - 1) / NGRP) cudaTriggerProgrammaticLaunchCompletion();
       if (act) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int s = 0; s < 8; ++s)
-            if ((ono[v] >> s) & 1u) p.spec[col_at_s<L>(f, j0 + v * QT, s, kx, R)] = x[0][v][s];
+          for (int s = 0; s < E; ++s)
+            if ((ono[v] >> s) & 1u) p.spec[col_at_s<L, E>(f, j0 + v * QT, s, kx, R)] = x[0][v][s];
       }
     }
   }
@@ -998,10 +1032,10 @@ __global__ void __launch_bounds__(kMaxThreads2d) kbp_colpass(const ColParams<T>*
   }
 }
 
-template <typename T, int OP, int L>
+template <typename T, int OP, int L, int E = 8>
 __global__ void __launch_bounds__(kMaxThreads2d) k_colpass(ColParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  colpass_body<T, OP, L>(p, blockIdx.x, smem_raw);
+  colpass_body<T, OP, L, true, E>(p, blockIdx.x, smem_raw);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1446,13 +1480,13 @@ __device__ __forceinline__ GatherItem<typename Prec2<T>::PT> gather_item(const R
 
 // SPLIT: one output field (p.fsel) per launch (see the spread kernel); its contribution to every
 // boundary component is added to Y (the operator is linear in the interpolated fields).
-template <typename T, int OP, int GMODE, int L, bool PF = true, bool SPLIT = false>
+template <typename T, int OP, int GMODE, int L, bool PF = true, bool SPLIT = false, int E = 8>
 __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int ord, unsigned char* smem_raw) {
   const int unit = p.bands_out ? p.bands_out[ord] : (ord + p.band0_out) & (p.n / p.R - 1);
   constexpr int NOUT = Traits<OP>::NOUT;
   constexpr int NB = SPLIT ? 1 : NOUT;  // fields held in shared memory
-  using CF = Cfg2<T, L, NB>;
-  using F = F8<L, CF::V>;
+  using CF = Cfg2<T, L, NB, E>;
+  using F = F8<L, CF::V, E>;
   using PT = typename Prec2<T>::PT;
   constexpr int n = F::N, V = CF::V, QT = CF::QT, NGRP = CF::NGRP, Q = F::Q;
   const int R = p.R, half = R >> 1, M = p.M;
@@ -1469,7 +1503,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   for (int v = 0; v < V; ++v) tw[v].load(p.tw, j0 + v * QT);
   // whether this lane's row pair is touched (else its spectra are not read: the transform of zeros)
   const int prow = r0 + 2 * rp;
-  const bool pair_on = active && ((rows_on(p.on_out, prow & (Q - 1)) >> (prow / Q)) & 1u);
+  const bool pair_on = active && ((rows_on(p.on_out, prow & (n / 8 - 1)) >> (prow / (n / 8))) & 1u);
   // the points whose stencil meets the band and this thread's first work item (4 per point),
   // loaded before the wait: the point tables are constant
   const PointRanges pr = band_points(p.cell_start, n, r0, R);
@@ -1492,21 +1526,21 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   for (int k = 0; k < NB / NGRP; ++k) {
     const int f = g + k * NGRP;
     cplx<T>* sb = buf + ((size_t)f * half + rp) * PN;
-    cplx<T> x[1][V][8];
+    cplx<T> x[1][V][E];
     const int fs = SPLIT ? p.fsel : f;  // the spectrum field read
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
+        for (int s = 0; s < E; ++s)
           x[0][v][s] = pair_on ? row_z<T, L>(p.spec, fs, r0, rp, R, j0 + v * QT + s * Q) : mk(T(0), T(0));
     }
-    f8_fft<T, true, L, V, 1>(x, sb, 0, j0, tw, active);
+    fft_lanes<T, true, L, V, E>(x, sb, j0, tw, active);
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
+        for (int s = 0; s < E; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
     }
   }
   __syncthreads();
@@ -1641,10 +1675,10 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   }
 }
 
-template <typename T, int OP, int GMODE, int L>
+template <typename T, int OP, int GMODE, int L, int E = 8>
 __global__ void __launch_bounds__(kMaxThreads2d) k_rowifft_gather(RowParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rowifft_gather_body<T, OP, GMODE, L>(p, blockIdx.x, smem_raw);
+  rowifft_gather_body<T, OP, GMODE, L, true, false, E>(p, blockIdx.x, smem_raw);
 }
 // one output field (p.fsel) per launch
 template <typename T, int OP, int GMODE, int L>
@@ -1717,6 +1751,7 @@ struct Launch2D {
   int units_in, units_out;  // bands the spread and the gather run
   int grid_mode;            // G_INTERP or G_GRID
   bool split;               // one field per launch (the shapes above are those of one field)
+  int elems;                // elements per lane (few_elements_2d; 8: the ordinary kernels)
 };
 
 template <typename T, int OP, int L>

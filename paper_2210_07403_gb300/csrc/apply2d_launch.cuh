@@ -257,6 +257,31 @@ ibdl_status launch_apply_2d(Geometry* g, const RowParams<T>& rp, const ColParams
     if (lc.split) return launch_apply_split_2d<T, OP, L>(g, rp, cp, lc, s);
   }
   const int st0 = pi ? IBDL_STAGE_SPREAD_ROWFFT_FP32 : IBDL_STAGE_SPREAD_ROWFFT_FP64;
+  if constexpr (few_elements_2d<T>(L) != 8) {
+    if (lc.elems != 8) {
+      // few elements per lane (at most 37 KB of shared memory: no opt-in)
+      constexpr int E = few_elements_2d<T>(L);
+      if (g->timing) timing_mark(g, s, -1);
+      IBDL_CUDA(launch_k(k_spread_rowfft<T, OP, L, E>, lc.units_in, lc.threads_row, lc.smem_row, s, lc.pdl, rp));
+      if (g->timing) timing_mark(g, s, st0);
+      IBDL_CUDA(launch_k(k_colpass<T, OP, L, E>, n / 2, lc.threads_col, lc.smem_col, s, lc.pdl, cp));
+      if (g->timing) timing_mark(g, s, st0 + 1);
+      if constexpr (std::is_same<T, double>::value) {
+        if (lc.grid_mode == G_GRID)
+          IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_GRID, L, E>, lc.units_out, lc.threads_gather, lc.smem_gather, s,
+                             lc.pdl, rp));
+      } else if (lc.grid_mode == G_GRID) {
+        return fail(IBDL_ERR_UNSUPPORTED, "float-float grid output");
+      }
+      if (lc.grid_mode != G_GRID)
+        IBDL_CUDA(launch_k(k_rowifft_gather<T, OP, G_INTERP, L, E>, lc.units_out, lc.threads_gather, lc.smem_gather, s,
+                           lc.pdl, rp));
+      if (g->timing) timing_mark(g, s, st0 + 2);
+      g->launches += 3;
+      IBDL_CUDA(cudaGetLastError());
+      return IBDL_OK;
+    }
+  }
   if (g->timing) timing_mark(g, s, -1);
   IBDL_CUDA(launch_k(k_spread_rowfft<T, OP, L>, lc.units_in, lc.threads_row, lc.smem_row, s, lc.pdl, rp));
   if (g->timing) timing_mark(g, s, st0);

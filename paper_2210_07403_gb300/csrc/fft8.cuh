@@ -48,11 +48,11 @@ __device__ __forceinline__ void static_for(F&& f) {
   }
 }
 
-template <int L, int V_>
+template <int L, int V_, int E = 8>
 struct F8 {
   static_assert(L >= 4 && L <= 13, "transform lengths 16 … 8192");
   static constexpr int N = 1 << L;
-  static constexpr int Q = N / 8;                        // lanes of a sequence
+  static constexpr int Q = N / E;                        // lanes of a sequence (E elements each)
   static constexpr int S8 = L / 3;                       // radix-8 stages
   static constexpr int LT = L % 3;                       // log2 of the tail radix (0: none)
   static constexpr int RT = 1 << LT;
@@ -371,6 +371,111 @@ __device__ __forceinline__ void f8_fft(cplx<T> (&x)[FL][V][8], cplx<T>* buf, int
       }
     }
   });
+}
+
+// ------------------------------------------------------------------------------------------
+// The same transform with E = 2 or 4 elements per lane (Q = N/E lanes): radix-E stages, and for
+// E = 4 and odd L a radix-2 tail. A lane's chain of operations is shorter (64 points: 34 FP64
+// instructions per transform with E = 2, 124 with E = 8) and a sequence spreads over more warps, at
+// the price of more exchanges and somewhat more operations in all: for single problems too small to
+// fill the GPU. 8-byte element types (FP64 and float-float) only.
+// ------------------------------------------------------------------------------------------
+__host__ __device__ constexpr int ipow(int b, int e) { return e == 0 ? 1 : b * ipow(b, e - 1); }
+
+// Twiddles: NV values per stage S ≥ 1 and k = j mod E^S (E = 2: w; E = 4: w, w², w³, or w, w² in the fused
+// form), then for the tail two per lane j (w of i = j, j + Q); 16-byte values, value c of k at
+// offset(S) + c·E^S + k.
+template <typename T, int L, int E>
+struct FewLayout {
+  static constexpr int LE = E == 2 ? 1 : 2, NS = L / LE, LT = L % LE, Q = (1 << L) / E;
+  static constexpr int NV = E == 2 ? 1 : (kFused8<T> ? 2 : 3), NT = LT ? 2 : 0;
+  __host__ __device__ static constexpr int offset(int S) { return NV * ((ipow(E, S) - E) / (E - 1)); }
+  static constexpr int NTW = NV * (NS - 1) + NT;
+};
+
+template <typename T, int L, int E>
+struct TwFew {
+  using Y = FewLayout<T, L, E>;
+  cplx<T> w[Y::NTW];
+  __device__ __forceinline__ void load(const cplx<T>* __restrict__ tab, int j) {
+    static_for<1, Y::NS>([&](auto st) {
+      constexpr int S = decltype(st)::value, p = ipow(E, S);
+#pragma unroll
+      for (int c = 0; c < Y::NV; ++c) w[(S - 1) * Y::NV + c] = tab[Y::offset(S) + c * p + (j & (p - 1))];
+    });
+#pragma unroll
+    for (int m = 0; m < Y::NT; ++m) w[(Y::NS - 1) * Y::NV + m] = tab[Y::offset(Y::NS) + m * Y::Q + j];
+  }
+};
+
+// (a, b) ← (a + w·b, a − w·b)
+template <typename T, bool INV>
+__device__ __forceinline__ void bfly(cplx<T>& a, cplx<T>& b, cplx<T> w) {
+  if constexpr (kFused8<T>) {
+    bfly_tan<T, INV, false>(a, b, w);
+  } else {
+    const cplx<T> t = cmul_tw<T, INV>(b, w);
+    b = csub(a, t);
+    a = cadd(a, t);
+  }
+}
+
+template <typename T, bool INV, int L, int E>
+__device__ __forceinline__ void few_fft(cplx<T> (&x)[E], cplx<T>* buf, int j, const TwFew<T, L, E>& tw, bool active) {
+  using Y = FewLayout<T, L, E>;
+  constexpr int NST = Y::NS + (Y::LT ? 1 : 0), Q = Y::Q;
+  static_for<0, NST>([&](auto st) {
+    constexpr int S = decltype(st)::value;
+    if (active) {
+      if constexpr (E == 2) {
+        if constexpr (S == 0)
+          dft2<T, INV>(x);
+        else
+          bfly<T, INV>(x[0], x[1], tw.w[S - 1]);
+      } else if constexpr (S == Y::NS) {  // tail: butterflies i = j, j + Q
+        bfly<T, INV>(x[0], x[2], tw.w[(S - 1) * Y::NV]);
+        bfly<T, INV>(x[1], x[3], tw.w[(S - 1) * Y::NV + 1]);
+      } else if constexpr (S == 0) {
+        dft4<T, INV>(x[0], x[1], x[2], x[3]);
+      } else if constexpr (kFused8<T>) {
+        const cplx<T> w1 = tw.w[(S - 1) * Y::NV], w2 = tw.w[(S - 1) * Y::NV + 1];
+        bfly_tan<T, INV, false>(x[0], x[2], w2);
+        bfly_tan<T, INV, false>(x[1], x[3], w2);
+        bfly_tan<T, INV, false>(x[0], x[1], w1);  // outputs 0, 2
+        bfly_tan<T, INV, true>(x[2], x[3], w1);   // outputs 1, 3
+        const cplx<T> y1 = x[2], y2 = x[1];
+        x[1] = y1;
+        x[2] = y2;
+      } else {
+#pragma unroll
+        for (int r = 1; r < 4; ++r) x[r] = cmul_tw<T, INV>(x[r], tw.w[(S - 1) * Y::NV + r - 1]);
+        dft4<T, INV>(x[0], x[1], x[2], x[3]);
+      }
+    }
+    if constexpr (S + 1 < NST) {
+      constexpr int p = ipow(E, S);
+      __syncthreads();
+      if (active) {
+        const int k = j & (p - 1), b = (j - k) * E + k;
+#pragma unroll
+        for (int t = 0; t < E; ++t) buf[ppos(b + t * p)] = x[t];
+      }
+      __syncthreads();
+      if (active) {
+#pragma unroll
+        for (int s = 0; s < E; ++s) x[s] = buf[ppos_strided<Q>(j, s)];
+      }
+    }
+  });
+}
+
+// the transform of one sequence with E elements per lane
+template <typename T, bool INV, int L, int V, int E, class TW>
+__device__ __forceinline__ void fft_lanes(cplx<T> (&x)[1][V][E], cplx<T>* buf, int j0, const TW (&tw)[V], bool active) {
+  if constexpr (E == 8)
+    f8_fft<T, INV, L, V, 1>(x, buf, 0, j0, tw, active);
+  else
+    few_fft<T, INV, L, E>(x[0][0], buf, j0, tw[0], active);
 }
 
 }  // namespace ibdl

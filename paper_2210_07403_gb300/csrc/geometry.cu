@@ -169,6 +169,44 @@ __global__ void k_twiddles(int L, int chunks, cplx<T>* tw) {
     tw_put<T>(tw + (size_t)e * per + i, co, s);
   }
 }
+// the table of few elements per lane (FewLayout): thread e writes value e
+template <typename T>
+__global__ void k_twiddles_few(int L, int E, int count, cplx<T>* tw) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= count) return;
+  const int n = 1 << L, NS = E == 2 ? L : L / 2, nv = E == 2 ? 1 : (kFused8<T> ? 2 : 3);
+  int S = 1, p = E, off = 0;
+  while (S < NS && e >= off + nv * p) {
+    off += nv * p;
+    p *= E;
+    ++S;
+  }
+  if (S == NS) p = n / E;  // the radix-2 tail of E = 4
+  const int c = (e - off) / p, k = (e - off) - c * p;
+  const int m = S < NS ? (c + 1) * k * (n / (E * p)) : k + c * p;
+  double s, co;
+  sincospi(-2.0 * (double)m / (double)n, &s, &co);
+  tw_put<T>(tw + e, co, s);
+}
+// values of that table (0: grids this large have none)
+template <typename T>
+static int few_values(int n) {
+  const int L = __builtin_ctz(n);
+  const bool is_ff = !std::is_same<T, double>::value;
+  if (L <= 8) return n - 2;                                    // E = 2: 2 + 4 + … + n/2
+  if (is_ff && L == 9) return 3 * (ipow(4, 4) - 4) / 3 + n / 2;  // E = 4: 3·(4 + 16 + 64), and the tail
+  return 0;
+}
+template <typename T>
+static ibdl_status make_few_table(int n, void** tw, cudaStream_t s) {
+  const int v = few_values<T>(n);
+  if (!v) return IBDL_OK;
+  IBDL_CUDA(cudaMalloc(tw, 16 * (size_t)v));
+  const int L = __builtin_ctz(n);
+  k_twiddles_few<T><<<(v + 127) / 128, 128, 0, s>>>(L, L <= 8 ? 2 : 4, v, static_cast<cplx<T>*>(*tw));
+  IBDL_CUDA(cudaGetLastError());
+  return IBDL_OK;
+}
 template <typename T>
 static void launch_twiddles(int n, void* tw, cudaStream_t s) {
   const int ch = tw_chunks<T>(n);
@@ -345,7 +383,7 @@ static void free_geometry(Geometry* g) {
   void* ptrs[] = {g->perm, g->base, g->cell_start, g->t64.phi, g->t64.dphi, g->t64.wscale, g->t64.nrm,
                   g->t32.phi, g->t32.dphi, g->t32.wscale, g->t32.nrm, g->spec, g->tw64, g->tw32,
                   g->lap64, g->der64, g->lap32, g->der32, g->ubuf, g->tmp_m, g->V, g->gm, g->vec,
-                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->bands};
+                  g->ddphi64, g->vjp_buf, g->X64, g->pp_buf, g->src_buf, g->twff, g->lapff, g->derff, g->bands, g->tw64_few, g->twff_few};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int i = 0; i < 4; ++i)
@@ -556,6 +594,10 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     GTRY(dalloc(&g->der32, sizeof(float) * n));
     // float-float twiddles and symbols (2-D and 3-D)
     GTRY(dalloc(&g->twff, 16 * (size_t)tw_chunks<ff>(n)));
+    if (dim == 2) {
+      GTRY(make_few_table<double>(n, &g->tw64_few, s));
+      GTRY(make_few_table<ff>(n, &g->twff_few, s));
+    }
     GTRY(dalloc(&g->lapff, sizeof(ff) * n));
     GTRY(dalloc(&g->derff, sizeof(ff) * n));
     GTRY(dalloc(&g->tmp_m, sizeof(double) * (g->ncomp * M + g->ncomp)));  // room for ū / constraint rows
