@@ -88,6 +88,11 @@ struct GlobSt3 {
   __device__ __forceinline__ void operator()(int b, C*, int m, int, C v) const { io.store(b, m, v); }
 };
 
+template <typename T, int L, int E>
+struct FewTw3 {
+  using type = TwFew<T, L, E == 8 ? 2 : E>;
+};
+
 // The register FFT (fft8.cuh) of `nseq` sequences of length 2^L, sequence b exchanging through
 // buf + b·(n + n/8): lane j of a sequence reads its elements j + s·Q through `ld` before the
 // transform and writes their transforms through `st` after it. kThreads3/QT sequences per pass;
@@ -95,23 +100,32 @@ struct GlobSt3 {
 // Register FFT configuration of the 3-D transforms (n ≤ 256: one lane per thread); twiddles in
 // registers when they fit the budget of the 2-D kernels (42 FP32, 56 FP64, 28 float-float
 // registers), else read from the table at each use.
+//
+// Elements per lane: two in FP64 and float-float where a grid leaves most sub-partitions idle
+// (fft8.cuh). Spheres, applications back to back with eight / two (µs): FP64 16³ 30.9 / 22.8, 32³ 38.9 / 31.5,
+// 64³ 79.3 / 76.9, 128³ 221 / 290; float-float 16³ 24.5 / 17.7, 32³ 30.0 / 22.4, 64³ 51.2 / 58.0.
+template <typename T>
+constexpr int few_elements_3d(int L) {
+  return sizeof(T) != 4 && L <= 5 ? 2 : 8;
+}
 template <typename T, int L>
 struct Cfg3 {
   static constexpr int V = 1;
-  static constexpr int QT = (1 << L) / 8;
+  static constexpr int E = few_elements_3d<T>(L);
+  static constexpr int QT = (1 << L) / E;
   static constexpr int NTW = TwLayout<T, L>::NTW;
   static constexpr bool TWR =
       sizeof(T) == 4 ? NTW <= 21 : (std::is_same<T, ff>::value ? NTW <= 7 : NTW <= 14);
-  using TW = std::conditional_t<TWR, TwRegs<T, L>, TwTable<T, L>>;
+  using TW = typename std::conditional_t<E == 8, std::conditional<TWR, TwRegs<T, L>, TwTable<T, L>>, FewTw3<T, L, E>>::type;
 };
 
 // Stride (elements) between the exchange buffers of sequences interleaved across threads: the
 // padded sequence rounded up to ≡ max(1, w/W) (mod w), w = 16 for 8-byte and 8 for 16-byte
 // elements, W = min(32, the sequences of a pass) interleaved in a warp: the rule of the 2-D column
 // groups, which puts the warp's sequences in different shared-memory banks.
-__host__ __device__ constexpr int seq_stride3(int L, int esize) {
+__host__ __device__ constexpr int seq_stride3(int L, int esize, int E) {
   const int pn = (1 << L) + (1 << L) / 8;
-  const int sp = kThreads3 / ((1 << L) / 8);
+  const int sp = kThreads3 / ((1 << L) / E);
   const int W = sp < 32 ? sp : 32;
   const int w = esize == 8 ? 16 : 8;
   const int t = (w / W > 1 ? w / W : 1) % w;
@@ -126,10 +140,11 @@ template <typename T, bool INV, int L, bool IL = false, class LD, class ST>
 __device__ __forceinline__ void fft3_run(cplx<T>* buf, int nseq, const cplx<T>* __restrict__ twg, const LD& ld,
                                          const ST& st) {
   using CF = Cfg3<T, L>;
-  using F = F8<L, CF::V>;
-  constexpr int V = CF::V, QT = CF::QT, Q = F::Q, SP = kThreads3 / QT;
+  constexpr int V = CF::V, E = CF::E, QT = CF::QT, SP = kThreads3 / QT;
+  using F = F8<L, V, E>;
+  constexpr int Q = F::Q;
   static_assert(kThreads3 % QT == 0, "whole sequences per pass");
-  constexpr int PS = IL ? seq_stride3(L, (int)sizeof(cplx<T>)) : F::PN;
+  constexpr int PS = IL ? seq_stride3(L, (int)sizeof(cplx<T>), E) : F::PN;
   const int sl = IL ? (int)threadIdx.x % SP : (int)threadIdx.x / QT;
   const int j0 = IL ? (int)threadIdx.x / SP : (int)threadIdx.x - sl * QT;
   typename CF::TW tw[V];
@@ -139,20 +154,20 @@ __device__ __forceinline__ void fft3_run(cplx<T>* buf, int nseq, const cplx<T>* 
     const int b = b0 + sl;
     const bool act = b < nseq;
     cplx<T>* sb = buf + (size_t)(act ? b : 0) * PS;
-    cplx<T> x[1][V][8];
+    cplx<T> x[1][V][E];
     if (act) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
+        for (int s = 0; s < E; ++s)
           x[0][v][s] = ld(b, sb, j0 + v * QT + s * Q, ppos_strided<Q>(j0 + v * QT, s));
     }
-    f8_fft<T, INV, L, V, 1>(x, sb, 0, j0, tw, act);
+    fft_lanes<T, INV, L, V, E>(x, sb, j0, tw, act);
     if (act) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < 8; ++s) st(b, sb, j0 + v * QT + s * Q, ppos_strided<Q>(j0 + v * QT, s), x[0][v][s]);
+        for (int s = 0; s < E; ++s) st(b, sb, j0 + v * QT + s * Q, ppos_strided<Q>(j0 + v * QT, s), x[0][v][s]);
     }
   }
 }
@@ -215,6 +230,19 @@ struct Col3Params {
 // which a lane of a column transform holds them; rows count in the pairs (2i, 2i + 1) of the
 // row kernels' packed transforms.
 __device__ __forceinline__ unsigned mask3(const unsigned char* m, size_t j) { return m ? (unsigned)m[j] : 0xffu; }
+// bit s: row (or plane) j + s·n/E of the mask m, for lanes of E elements
+template <int L, int E>
+__device__ __forceinline__ unsigned lane_mask3(const unsigned char* m, int j) {
+  if constexpr (E == 8) return mask3(m, j);
+  constexpr int n = 1 << L;
+  unsigned r = 0;
+#pragma unroll
+  for (int s = 0; s < E; ++s) {
+    const int row = j + s * (n / E);
+    r |= ((mask3(m, row & (n / 8 - 1)) >> (row / (n / 8))) & 1u) << s;
+  }
+  return r;
+}
 
 __device__ __forceinline__ void resolve_io3(const Row3Params& p, const double*& in, double*& out) {
   in = p.in;
@@ -411,7 +439,7 @@ template <typename T>
 struct YColumnIO {
   cplx<T>* spec;
   int n, nh, z, k0, lc, C;
-  int lq;             // log2(n/8): row m is bit m >> lq of the lane's masks
+  int lq;             // log2(n/E): row m is bit m >> lq of the lane's masks (E elements per lane)
   unsigned in, out;   // the lane's rows to read and to store
   __device__ __forceinline__ size_t at(int bi, int m) const {
     return (((size_t)(bi >> lc) * n + z) * n + m) * nh + k0 + (bi & (C - 1));
@@ -441,10 +469,11 @@ __global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
   const int z = p.planes ? p.planes[zi] : zi;
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
   // the forward pass reads the touched rows of its plane and writes every ky; the inverse the reverse
-  constexpr int Q = n / 8;
+  constexpr int E = Cfg3<T, L>::E, lq = L - (E == 8 ? 3 : 1);
   const int j0 = lane3<T, L>();
-  const unsigned in = INV ? 0xffu : mask3(p.rows_in, z * Q + j0), out = INV ? mask3(p.rows_out, z * Q + j0) : 0xffu;
-  const YColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, z, k0, p.lc, C, L - 3, in, out};
+  const unsigned char* rows = INV ? p.rows_out : p.rows_in;
+  const unsigned on = lane_mask3<L, E>(rows ? rows + (size_t)z * (n / 8) : nullptr, j0);
+  const YColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, z, k0, p.lc, C, lq, INV ? 0xffu : on, INV ? on : 0xffu};
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
   fft3_run<T, INV, L, true>(bufA, p.nf * C, static_cast<const cplx<T>*>(p.tw), GlobLd3<YColumnIO<T>>{io},
@@ -459,7 +488,7 @@ template <typename T>
 struct ZColumnIO {
   cplx<T>* spec;
   int n, nh, ky1, ky2, k0, lc, C;
-  int lq;             // log2(n/8)
+  int lq;             // log2(n/E)
   unsigned in, out;   // the lane's planes to read and to store
   __device__ __forceinline__ size_t at(int bi, int m) const {
     const int c = bi & (C - 1), fq = bi >> lc;
@@ -509,7 +538,8 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
   const int ky1 = pair, ky2 = (n - pair) & (n - 1);
   const int nq = ky1 == ky2 ? 1 : 2;  // y-frequency columns in this CTA
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
-  constexpr int PS = seq_stride3(L, (int)sizeof(cplx<T>));  // sequences interleaved (fft3_run)
+  constexpr int E = Cfg3<T, L>::E, lq = L - (E == 8 ? 3 : 1);
+  constexpr int PS = seq_stride3(L, (int)sizeof(cplx<T>), E);  // sequences interleaved (fft3_run)
   T* lap1 = reinterpret_cast<T*>(bufA + (size_t)NMAX * 2 * C * PS);
   T* der1 = lap1 + n;
   const cplx<T>* twg = static_cast<const cplx<T>*>(p.tw);
@@ -518,8 +548,8 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
     der1[i] = static_cast<const T*>(p.der1)[i];
   }
   const int j0 = lane3<T, L>();
-  const ZColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, ky1, ky2, k0, lc, C, L - 3,
-                        mask3(p.planes_in, j0), mask3(p.planes_out, j0)};
+  const ZColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, ky1, ky2, k0, lc, C, lq,
+                        lane_mask3<L, E>(p.planes_in, j0), lane_mask3<L, E>(p.planes_out, j0)};
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
   __syncthreads();
@@ -700,11 +730,13 @@ __host__ __device__ constexpr size_t smem_rows3(int n, int nf, int R) {
 }
 template <typename T>
 constexpr size_t smem_y3(int n, int nf, int C) {  // host side (launch shapes)
-  return (size_t)nf * C * seq_stride3(__builtin_ctz(n), (int)sizeof(cplx<T>)) * sizeof(cplx<T>);
+  const int L = __builtin_ctz(n);
+  return (size_t)nf * C * seq_stride3(L, (int)sizeof(cplx<T>), few_elements_3d<T>(L)) * sizeof(cplx<T>);
 }
 template <typename T>
 constexpr size_t smem_z3(int n, int nf, int C) {  // host side (launch shapes)
-  return (size_t)nf * 2 * C * seq_stride3(__builtin_ctz(n), (int)sizeof(cplx<T>)) * sizeof(cplx<T>) +
+  const int L = __builtin_ctz(n);
+  return (size_t)nf * 2 * C * seq_stride3(L, (int)sizeof(cplx<T>), few_elements_3d<T>(L)) * sizeof(cplx<T>) +
          2 * n * sizeof(T);
 }
 
@@ -758,8 +790,11 @@ inline cudaError_t launch3(void (*kernel)(KArgs...), int grid, size_t smem, cuda
 }
 
 template <typename T, int OP, int L>
-ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp, const Col3Params& cp, const Launch3D& lc,
+ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp0, const Col3Params& cp0, const Launch3D& lc,
                             cudaStream_t s) {
+  Row3Params rp = rp0;
+  Col3Params cp = cp0;
+  if constexpr (few_elements_3d<T>(L) != 8) rp.tw = cp.tw = std::is_same<T, double>::value ? g->tw64_few : g->twff_few;
   const int R = lc.R, C = lc.C, Cz = lc.Cz;
   constexpr int NIN = Traits3<OP>::NIN, NOUT = Traits3<OP>::NOUT, NMAX = NIN > NOUT ? NIN : NOUT;
   constexpr int n = 1 << L;

@@ -594,10 +594,8 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     GTRY(dalloc(&g->der32, sizeof(float) * n));
     // float-float twiddles and symbols (2-D and 3-D)
     GTRY(dalloc(&g->twff, 16 * (size_t)tw_chunks<ff>(n)));
-    if (dim == 2) {
-      GTRY(make_few_table<double>(n, &g->tw64_few, s));
-      GTRY(make_few_table<ff>(n, &g->twff_few, s));
-    }
+    GTRY(make_few_table<double>(n, &g->tw64_few, s));
+    GTRY(make_few_table<ff>(n, &g->twff_few, s));
     GTRY(dalloc(&g->lapff, sizeof(ff) * n));
     GTRY(dalloc(&g->derff, sizeof(ff) * n));
     GTRY(dalloc(&g->tmp_m, sizeof(double) * (g->ncomp * M + g->ncomp)));  // room for ū / constraint rows

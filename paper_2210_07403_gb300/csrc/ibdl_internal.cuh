@@ -120,7 +120,7 @@ struct Geometry {
   size_t spec_bytes;
   void* tw64;      // twiddle tables of the transforms (TwLayout in fft8.cuh)
   void* tw32;
-  void* tw64_few;  // and of few elements per lane (FewLayout; 2-D, small grids, else NULL)
+  void* tw64_few;  // and of few elements per lane (FewLayout; small grids, else NULL)
   void* twff_few;
   // per-axis Fourier symbols indexed by FFT index j (wavenumber 2π m/box, m = j or j − n):
   // lap = symbol of −∂² along one axis, der = k̃ with ∂ ↦ i k̃ (0 at Nyquist)
