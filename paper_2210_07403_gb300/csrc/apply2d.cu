@@ -571,15 +571,25 @@ static ibdl_status batch_prepare_t(Batch* B, const int* kptr /* device &st[b].k,
     B->nrow_units[pi] = B->ncol_units[pi] = 0;
     return IBDL_OK;
   }
+  // float-float batches with up to ten CTAs of a size per SM trigger late as well (late_rows_2d): 16
+  // ellipses to 512² 137 / 119 µs, 64 of them 234 / 230, 64 to 256² 130 / 124; 256 to 512² 764 / 772
+  int bands[14] = {};
+  for (int b = 0; b < B->count; ++b) {
+    int cnt = 0, first;
+    touched_bands(B->geoms[b], B->geoms[b]->rows_per_cta[pi], &cnt, &first);
+    bands[log2i(B->geoms[b]->n)] += cnt;
+  }
   for (int b = 0; b < B->count; ++b) {
     Geometry* g = B->geoms[b];
     if (batch_shape_any<T>(B, g, pi) != IBDL_OK)
       return fail(IBDL_ERR_UNSUPPORTED, "problem " + std::to_string(b) + ": its grid is too large for a batched launch");
     user[b] = row_params<T>(g, nullptr, nullptr, nullptr, nullptr);
+    user[b].late = std::is_same<T, ff>::value && bands[log2i(g->n)] <= 10 * 152;
     user[b].io_off = B->off[b];
     kry[b] = user[b];
     col[b] = col_params<T>(g, nullptr);
     if (no_mean_2d(g)) col[b].drop0 = 1;
+    col[b].late = user[b].late;
     if (kptr) {
       const int* kb = reinterpret_cast<const int*>(reinterpret_cast<const char*>(kptr) + kstride * b);
       kry[b].idx = kb;                               // &st[b].k

@@ -225,7 +225,7 @@ struct RowParams {
   double eta;             // η
   double hd;              // h^d
   PT eta_src;             // weight of the ηSQ source: η (scalar) or η/μ (Stokes, projected part)
-  int late;               // single problems: let the next kernel launch after the transforms, not before
+  int late;               // let the next kernel launch after the transforms, not before (late_rows_2d)
   int fsel;               // one-field launches: the field this launch spreads or interpolates
   // the bands some stencil meets (NULL: every band), for the spread and for the gather, and the
   // rows whose spectra the gather needs (see touched rows below; NULL: every row)
@@ -292,6 +292,10 @@ __device__ __forceinline__ unsigned lane_rows_on(const unsigned char* on, int j)
   }
   return m;
 }
+
+// kernels that may trigger late: single problems, and float-float batches
+template <typename T, bool PF>
+constexpr bool kLate2d = PF || std::is_same<T, ff>::value;
 
 // Sorted points whose base row lies in the cell rows [r0 − 3, r0 + R) (mod n): at most two
 // contiguous ranges of the cell-sorted order.
@@ -426,7 +430,7 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // Let the next kernel launch and run its prologue. Triggered only after this kernel's own
   // wait, so every kernel before the previous one has completed by then: a prologue overlaps
   // its direct predecessor only (its wait still covers this grid's completion and writes).
-  if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();
+  if (!kLate2d<T, PF> || !p.late) cudaTriggerProgrammaticLaunchCompletion();
   // In a GMRES cycle the step just before this kernel writes the stop flag and the Krylov index:
   // both loads go out together, then the branch
   const int stopped = p.stop ? *p.stop : 0;
@@ -568,7 +572,7 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // one (field, row pair), reads Z_k and Z_{n−k} once and writes A_k and B_k, adjacent in the
   // band-major block (offset k·R + 2j), with one store. Both are left doubled (the ½ is in the
   // symbol's scale: half the arithmetic of this step)
-  if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
+  if (kLate2d<T, PF> && p.late) cudaTriggerProgrammaticLaunchCompletion();
   const cplx<T>* res = buf;
   constexpr int nh = n >> 1, lnh = L - 1;
   for (int t = threadIdx.x; t < NB * half * nh; t += blockDim.x) {
@@ -764,7 +768,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
     ono[v] = lane_rows_on<L, E>(p.on_out, j0 + v * QT);
   }
   cudaGridDependencySynchronize();
-  if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
+  if (!kLate2d<T, PF> || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
 
   if constexpr (NIN == 1 && NOUT == 1) {
     // one field in and out: the symbol is applied to the registers between the transforms
@@ -809,7 +813,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
     }
     // (the inverse transform's first exchange barrier orders the partner reads before its writes)
     fft_lanes<T, true, L, V, E>(x, sb, j0, tw, active);
-    if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
+    if (kLate2d<T, PF> && p.late) cudaTriggerProgrammaticLaunchCompletion();
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
@@ -909,7 +913,7 @@ __device__ __forceinline__ void colpass_body(const ColParams<T>& p, int unit, un
           for (int s = 0; s < E; ++s) x[0][v][s] = sb[ppos_strided<Q>(j0 + v * QT, s)];
       }
       fft_lanes<T, true, L, V, E>(x, sb, j0, tw, act);
-      if (PF && p.late && k + 1 == (NOUT + NGRP - 1) / NGRP) cudaTriggerProgrammaticLaunchCompletion();
+      if (kLate2d<T, PF> && p.late && k + 1 == (NOUT + NGRP - 1) / NGRP) cudaTriggerProgrammaticLaunchCompletion();
       if (act) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
@@ -1519,7 +1523,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   double* pout;
   resolve_io(p, pin, pout);
   cudaGridDependencySynchronize();
-  if (!PF || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
+  if (!kLate2d<T, PF> || !p.late) cudaTriggerProgrammaticLaunchCompletion();  // after the wait (see the spread kernel)
 
   // inverse FFT of every (field, row pair) sequence, its first stage fed from the half spectra
 #pragma unroll
@@ -1544,7 +1548,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
     }
   }
   __syncthreads();
-  if (PF && p.late) cudaTriggerProgrammaticLaunchCompletion();
+  if (kLate2d<T, PF> && p.late) cudaTriggerProgrammaticLaunchCompletion();
   // real values: field f, local row lr, column x at element e = (f·half + lr/2)·n + x, part lr & 1
   const T* u = reinterpret_cast<const T*>(buf);
 
