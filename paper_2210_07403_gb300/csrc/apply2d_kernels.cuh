@@ -178,8 +178,10 @@ __device__ __forceinline__ void col_lane_2d(int C, int& g, int& c, int& j0, bool
 // row pair per run of consecutive threads and the plain padded stride.
 __host__ __device__ constexpr bool row_interleave_2d(int L, bool f32) { return lanes_per_thread_2d(L, f32) < 4; }
 __host__ __device__ constexpr int row_stride_2d(int L, int half, int esize) {
-  return row_interleave_2d(L, esize == 8) ? col_stride_2d(L, half, esize) : (1 << L) + (1 << L) / 8;
+  return row_interleave_2d(L, esize == 8) ? col_stride_2d(L, half, esize) : (1 << L) + (1 << L) / 16;
 }
+// pads of a row sequence (ppos): those of 8-byte elements with one sequence per warp where not interleaved
+__host__ __device__ constexpr int row_pad_2d(int L, bool f32) { return row_interleave_2d(L, f32) ? 3 : 4; }
 template <int QT, int NGRP, bool IL>
 __device__ __forceinline__ void row_lane_2d(int half, int& g, int& rp, int& j0, bool& active) {
   if constexpr (IL) {
@@ -399,9 +401,10 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
   // lr, column x → real part (even lr) or imaginary part (odd lr) of element ppos(x) of sequence
   // f·half + lr/2
   const int PN = row_stride_2d(L, half, (int)sizeof(cplx<T>));
+  constexpr int PS = row_pad_2d(L, sizeof(T) == 4);
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
   PT* acc = reinterpret_cast<PT*>(buf);
-  auto aidx = [&](int seq, int x) { return 2 * (seq * PN + ppos(x)); };
+  auto aidx = [&](int seq, int x) { return 2 * (seq * PN + ppos<PS>(x)); };
   const int r0 = unit * R;
   // FFT lanes: thread (group g, row pair rp, lane j0); threads past NGRP·half·QT only help with
   // the loops (clearing, spreading, unpacking)
@@ -555,14 +558,14 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < E; ++s) x[0][v][s] = Prec2<T>::acc_load(sb, ppos_strided<F::Q>(j0 + v * QT, s));
+        for (int s = 0; s < E; ++s) x[0][v][s] = Prec2<T>::acc_load(sb, ppos_strided<F::Q, PS>(j0 + v * QT, s));
     }
-    fft_lanes<T, false, L, V, E>(x, sb, j0, tw, active);
+    fft_lanes<T, false, L, V, E, PS>(x, sb, j0, tw, active);
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < E; ++s) sb[ppos_strided<F::Q>(j0 + v * QT, s)] = x[0][v][s];
+        for (int s = 0; s < E; ++s) sb[ppos_strided<F::Q, PS>(j0 + v * QT, s)] = x[0][v][s];
     }
   }
   __syncthreads();
@@ -582,11 +585,11 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
     const int fo = SPLIT ? p.fsel : f;  // the spectrum field written
     cplx<T> a, b;
     if (k == 0) {
-      const cplx<T> z0 = res[zb], zh = res[zb + ppos(nh)];
+      const cplx<T> z0 = res[zb], zh = res[zb + ppos<PS>(nh)];
       a = mk(z0.x + z0.x, zh.x + zh.x);
       b = mk(z0.y + z0.y, zh.y + zh.y);
     } else {
-      const cplx<T> zk = res[zb + ppos(k)], zc = res[zb + ppos(n - k)];
+      const cplx<T> zk = res[zb + ppos<PS>(k)], zc = res[zb + ppos<PS>(n - k)];
       a = mk(zk.x + zc.x, zk.y - zc.y);
       b = mk(zk.y + zc.y, zc.x - zk.x);
     }
@@ -1496,6 +1499,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
   const int R = p.R, half = R >> 1, M = p.M;
   // sequences and lanes as in the spread kernel (row pairs interleaved across threads)
   const int PN = row_stride_2d(L, half, (int)sizeof(cplx<T>));
+  constexpr int PS = row_pad_2d(L, sizeof(T) == 4);
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
   const int r0 = unit * R;
   // FFT lanes: thread (group g, row pair rp, lane j0); threads past NGRP·half·QT only gather
@@ -1539,12 +1543,12 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
         for (int s = 0; s < E; ++s)
           x[0][v][s] = pair_on ? row_z<T, L>(p.spec, fs, r0, rp, R, j0 + v * QT + s * Q) : mk(T(0), T(0));
     }
-    fft_lanes<T, true, L, V, E>(x, sb, j0, tw, active);
+    fft_lanes<T, true, L, V, E, PS>(x, sb, j0, tw, active);
     if (active) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int s = 0; s < E; ++s) sb[ppos_strided<Q>(j0 + v * QT, s)] = x[0][v][s];
+        for (int s = 0; s < E; ++s) sb[ppos_strided<Q, PS>(j0 + v * QT, s)] = x[0][v][s];
     }
   }
   __syncthreads();
@@ -1561,7 +1565,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
       // the completed method's field is u₀ + ū (ū after the density in the input vector)
       const double ub = p.aug ? p.in[(size_t)Traits<OP>::C * M + fo] : 0.0;
       p.grid[((size_t)fo * n + r0 + lr) * n + x] =
-          double(Prec2<T>::to_pt(u[2 * ((f * half + (lr >> 1)) * PN + ppos(x)) + (lr & 1)])) + ub;
+          double(Prec2<T>::to_pt(u[2 * ((f * half + (lr >> 1)) * PN + ppos<PS>(x)) + (lr & 1)])) + ub;
     }
     return;
   }
@@ -1583,7 +1587,7 @@ __device__ __forceinline__ void rowifft_gather_body(const RowParams<T>& p, int o
     const PT dy = (OP == OP_ADJ_AN || OP == OP_STOKES_T) ? it.dy : PT(0);
     // value of sequence lr/2 + field·half at column x (part lr & 1)
     const int eb = 2 * (lr >> 1) * PN + (lr & 1), fs2 = 2 * half * PN;
-    auto uval = [&](int f, int x) { return Prec2<T>::to_pt(u[eb + f * fs2 + 2 * ppos(x)]); };
+    auto uval = [&](int f, int x) { return Prec2<T>::to_pt(u[eb + f * fs2 + 2 * ppos<PS>(x)]); };
     if constexpr (SPLIT) {
       // the value, x-gradient and y-gradient gathers of field p.fsel (first slot)
       PT a = 0, gx = 0, gy = 0;

@@ -250,15 +250,22 @@ __device__ __forceinline__ void f8_stage(cplx<T> (&x)[8], const TW& tw) {
   }
 }
 
-// padded position of element e of a sequence (see pidx); e < N
-__device__ __forceinline__ int ppos(int e) { return e + (e >> 3); }
-// padded position of j + s·Q: ppos(j) + s·(Q + Q/8) when Q is a multiple of 8 (n ≥ 64)
-template <int Q>
+// padded position of element e < N of a sequence: one pad after every 2^PS elements. A warp's access takes
+// groups of 16 lanes of 8-byte elements or 8 of 16-byte ones, and the least wavefronts when a group's
+// positions differ mod its size. PS = 3 gives that for 16-byte elements, and for 8-byte ones where the
+// lanes of several sequences alternate in a warp; PS = 4 for 8-byte elements with one sequence per warp
+// (there, 16 adjacent elements at PS = 3 meet one bank twice, half of the shared-memory wavefronts of
+// the 8192² FP32 row kernels; at PS = 4 only the second stage's writes do: spread 111 / 93 µs,
+// gather 98 / 84, the application 499 / 469).
+template <int PS = 3>
+__device__ __forceinline__ int ppos(int e) { return e + (e >> PS); }
+// padded position of j + s·Q: ppos(j) + s·ppos(Q) when Q is a multiple of 2^PS (PS = 3: n ≥ 64)
+template <int Q, int PS = 3>
 __device__ __forceinline__ int ppos_strided(int j, int s) {
-  if constexpr (Q % 8 == 0)
-    return ppos(j) + s * (Q + Q / 8);
+  if constexpr (Q % (1 << PS) == 0)
+    return ppos<PS>(j) + s * (Q + (Q >> PS));
   else
-    return ppos(j + s * Q);
+    return ppos<PS>(j + s * Q);
 }
 
 // The same transform for one sequence with the radix-8 stages as a loop over a runtime
@@ -324,7 +331,7 @@ __device__ __forceinline__ void f8_fft_rolled(cplx<T> (&x)[1][V][8], cplx<T>* bu
 // false for threads that hold no sequence. Each lane reads its inputs before the call and writes
 // its results after it only at its own positions j + s·Q, so neither needs a barrier against the
 // exchanges inside.
-template <typename T, bool INV, int L, int V, int FL, class TW>
+template <typename T, bool INV, int L, int V, int FL, int PS = 3, class TW>
 __device__ __forceinline__ void f8_fft(cplx<T> (&x)[FL][V][8], cplx<T>* buf, int fstride, int j0,
                                        const TW (&tw)[V], bool active) {
   using F = F8<L, V>;
@@ -348,14 +355,13 @@ __device__ __forceinline__ void f8_fft(cplx<T> (&x)[FL][V][8], cplx<T>* buf, int
 #pragma unroll
         for (int v = 0; v < V; ++v) {
           const int j = j0 + v * F::QT, k = j & (p - 1);
-          // base + t·p (t < 8) keeps base's low three bits when p ≥ 8 (and is 8j + t when
-          // p = 1), so its padded position is ppos(base) plus a constant per t
-          const int pb = ppos((j - k) * 8 + k);
-          constexpr int dt = p == 1 ? 1 : p + p / 8;
+          // adding t·p (t < 8) to base carries nothing out of its low PS bits, so the padded position is
+          // ppos(base) plus a constant per t
+          const int pb = ppos<PS>((j - k) * 8 + k);
 #pragma unroll
           for (int f = 0; f < FL; ++f)
 #pragma unroll
-            for (int t = 0; t < 8; ++t) buf[f * fstride + pb + t * dt] = x[f][v][t];
+            for (int t = 0; t < 8; ++t) buf[f * fstride + pb + t * p + ((t * p) >> PS)] = x[f][v][t];
         }
       }
       __syncthreads();
@@ -366,7 +372,7 @@ __device__ __forceinline__ void f8_fft(cplx<T> (&x)[FL][V][8], cplx<T>* buf, int
 #pragma unroll
           for (int f = 0; f < FL; ++f)
 #pragma unroll
-            for (int s = 0; s < 8; ++s) x[f][v][s] = buf[f * fstride + ppos_strided<F::Q>(j, s)];
+            for (int s = 0; s < 8; ++s) x[f][v][s] = buf[f * fstride + ppos_strided<F::Q, PS>(j, s)];
         }
       }
     }
@@ -470,10 +476,10 @@ __device__ __forceinline__ void few_fft(cplx<T> (&x)[E], cplx<T>* buf, int j, co
 }
 
 // the transform of one sequence with E elements per lane
-template <typename T, bool INV, int L, int V, int E, class TW>
+template <typename T, bool INV, int L, int V, int E, int PS = 3, class TW>
 __device__ __forceinline__ void fft_lanes(cplx<T> (&x)[1][V][E], cplx<T>* buf, int j0, const TW (&tw)[V], bool active) {
   if constexpr (E == 8)
-    f8_fft<T, INV, L, V, 1>(x, buf, 0, j0, tw, active);
+    f8_fft<T, INV, L, V, 1, PS>(x, buf, 0, j0, tw, active);
   else
     few_fft<T, INV, L, E>(x[0][0], buf, j0, tw[0], active);
 }
