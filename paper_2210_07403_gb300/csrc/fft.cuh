@@ -1,26 +1,10 @@
-// Shared-memory Stockham FFT and the regularised-delta kernels used by the IBDL kernels.
+// Butterflies, Fourier-symbol quotients and the regularised-delta kernels used by the IBDL kernels.
 #pragma once
-
-#include <type_traits>
 
 #include "ibdl_internal.cuh"
 
 namespace ibdl {
 
-// ------------------------------------------------------------------------------------------
-// Batched complex FFT of power-of-two length n in shared memory (Stockham autosort: every
-// stage reads one buffer and writes the other, so no bit reversal is needed).
-//
-// Stage with current sub-transform length p and radix R: butterfly i ∈ [0, n/R) of every
-// sequence reads x[i + r·n/R] (r < R), multiplies input r by ω^{r·k} with k = i mod p and
-// ω = e^{∓2πi/(pR)}, takes the R-point DFT, and writes output t to y[(i − k)·R + k + t·p].
-// Radix-8 stages run while at least three factors of two remain, then one radix-4 or radix-2.
-//
-// tw[j] = e^{−2πi j/n} (the kernels stage it in shared memory); the inverse transform (INV)
-// uses conjugates and is unnormalised. Sequences are `nb` runs of n contiguous elements,
-// sequence b starting at b·bstride. Returns the buffer that holds the result (a or b). All
-// threads of the block must call it.
-// ------------------------------------------------------------------------------------------
 template <typename T, bool INV>
 __device__ __forceinline__ void dft2(cplx<T>* u) {
   const cplx<T> t = u[0];
@@ -85,121 +69,10 @@ __device__ __forceinline__ double sym_div(double a, double b) {
   return a * fma(r, fma(e, e, e), r);
 }
 
-// Shared-memory FFT buffers are padded with one element after every eight, which keeps the
+// The 3-D row kernels' buffers are padded with one element after every eight, which keeps the
 // radix-8 stride-8 writes of the first stages free of bank conflicts for 8- and 16-byte elements.
 __device__ __forceinline__ int pidx(int x) { return x + (x >> 3); }
 __host__ __device__ constexpr size_t padded(size_t x) { return x + (x >> 3); }
-
-// element m of sequence bi in a padded shared-memory buffer of sequences of length 2^log2n
-template <typename T>
-struct SmemIO {
-  cplx<T>* buf;
-  int log2n;
-  __device__ __forceinline__ cplx<T> load(int bi, int m) const { return buf[pidx((bi << log2n) + m)]; }
-  __device__ __forceinline__ void store(int bi, int m, cplx<T> v) const { buf[pidx((bi << log2n) + m)] = v; }
-};
-
-struct NoIO {};
-
-// One Stockham stage reading through `ld` and writing through `st`.
-template <typename T, bool INV, int LR, class LD, class ST>
-__device__ __forceinline__ void fft_stage(const LD& ld, const ST& st, int log2n, int lp, int nb,
-                                          const cplx<T>* __restrict__ tw) {
-  constexpr int R = 1 << LR;
-  const int lq = log2n - LR;
-  const int q = 1 << lq;
-  const int p = 1 << lp;
-  const int total = nb << lq;
-  const int tws = 1 << (log2n - lp - LR);  // n / (pR)
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    const int bi = t >> lq, i = t & (q - 1), k = i & (p - 1);
-    cplx<T> u[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) u[r] = ld.load(bi, i + r * q);
-    if (k) {
-#pragma unroll
-      for (int r = 1; r < R; ++r) {
-        cplx<T> w = tw[r * k * tws];
-        if (INV) w.y = -w.y;
-        u[r] = cmul(u[r], w);
-      }
-    }
-    if (LR == 3)
-      dft8<T, INV>(u);
-    else if (LR == 2)
-      dft4<T, INV>(u[0], u[1], u[2], u[3]);
-    else
-      dft2<T, INV>(u);
-    const int j = ((i - k) << LR) + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) st.store(bi, j + r * p, u[r]);
-  }
-}
-
-template <typename T, bool INV, int LR, class FL, class LS>
-__device__ __forceinline__ void fft_stage_dispatch(bool first, bool last, const SmemIO<T>& in, const SmemIO<T>& out,
-                                                   const FL& fl, const LS& ls, int log2n, int lp, int nb,
-                                                   const cplx<T>* tw) {
-  constexpr bool HF = !std::is_same<FL, NoIO>::value, HL = !std::is_same<LS, NoIO>::value;
-  if constexpr (HF && HL) {
-    if (first && last) {
-      fft_stage<T, INV, LR>(fl, ls, log2n, lp, nb, tw);
-      return;
-    }
-  }
-  if constexpr (HF) {
-    if (first) {
-      fft_stage<T, INV, LR>(fl, out, log2n, lp, nb, tw);
-      return;
-    }
-  }
-  if constexpr (HL) {
-    if (last) {
-      fft_stage<T, INV, LR>(in, ls, log2n, lp, nb, tw);
-      return;
-    }
-  }
-  fft_stage<T, INV, LR>(in, out, log2n, lp, nb, tw);
-}
-
-// All stages of `nb` transforms of length 2^log2n. Stage 0 reads through `fl` (or from the padded
-// buffer a), the last stage writes through `ls` (or to its padded target buffer); in between the
-// stages ping-pong between a and b. Returns the padded buffer the last stage wrote (meaningful
-// when `ls` is NoIO). All threads of the block must call it.
-template <typename T, bool INV, class FL = NoIO, class LS = NoIO>
-__device__ cplx<T>* fft_run(cplx<T>* a, cplx<T>* b, int log2n, int nb, const cplx<T>* __restrict__ tw,
-                            const FL& fl = FL(), const LS& ls = LS()) {
-  int lp = 0;
-  int s = log2n;
-  cplx<T>* src = a;
-  cplx<T>* dst = b;
-  bool first = true;
-  while (s > 0) {
-    const int lr = s >= 3 ? 3 : s;
-    const bool last = s == lr;
-    const SmemIO<T> in{src, log2n}, out{dst, log2n};
-    if (lr == 3)
-      fft_stage_dispatch<T, INV, 3>(first, last, in, out, fl, ls, log2n, lp, nb, tw);
-    else if (lr == 2)
-      fft_stage_dispatch<T, INV, 2>(first, last, in, out, fl, ls, log2n, lp, nb, tw);
-    else
-      fft_stage_dispatch<T, INV, 1>(first, last, in, out, fl, ls, log2n, lp, nb, tw);
-    __syncthreads();
-    cplx<T>* tmp = src;
-    src = dst;
-    dst = tmp;
-    lp += lr;
-    s -= lr;
-    first = false;
-  }
-  return src;
-}
-
-// copy the n-entry twiddle table into shared memory (caller synchronises before use)
-template <typename T>
-__device__ __forceinline__ void load_twiddles(cplx<T>* dst, const cplx<T>* __restrict__ src, int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
-}
 
 // ------------------------------------------------------------------------------------------
 // One-dimensional 4-point kernels φ of δ_h (Sec. 2.2.2) and their derivatives, FP64.
