@@ -36,7 +36,7 @@
  *
  * Environment (read once per process; for experiments, none is needed for correct results):
  *   IBDL_NO_PDL=1            launch kernels without programmatic dependent launch;
- *   IBDL_UNROLL=u (1..16)    GMRES iterations per body of a cycle's captured while loop (8);
+ *   IBDL_UNROLL=u (1..16)    GMRES iterations per body of a cycle's captured while loop (4);
  *   IBDL_ARNOLDI_CLUSTER=8   run the Arnoldi step on 8-CTA clusters even where 16 fit;
  *   IBDL_PLAN_R, IBDL_PLAN_C, IBDL_THREADS   2-D launch shape before autotuning (rows per CTA of
  *                            the row kernels, columns per CTA of the column pass, least threads

@@ -12,10 +12,14 @@
 //   k_rowifft_gather  band of R rows: inverse FFT along x, then interpolate (S*) the band's part
 //                     of every point's stencil and add it to Y (which the first kernel set to ½Q).
 //
+// The row kernels run only the bands that some stencil meets and transform only the rows that some
+// stencil meets (the others are zero on the way in and unread on the way out; see touched rows below).
+//
 // The transforms are the register FFT of fft8.cuh: a thread holds eight elements (per lane) of
-// a sequence; a CTA has (R/2)·QT threads in the row kernels and C·QT in the column pass (QT
-// threads per sequence), and one padded shared-memory buffer per sequence, used for the spread's
-// accumulation, the exchanges between FFT stages and the final layout.
+// a sequence (two or four on small grids, few_elements_2d); a CTA has (R/2)·QT threads in the row
+// kernels and C·QT in the column pass (QT threads per sequence), and one padded shared-memory buffer
+// per sequence, used for the spread's accumulation, the exchanges between FFT stages and the final
+// layout.
 //
 // Packed half spectrum: for a real row a, A_k (k = 0..n/2) is stored in n/2 slots with slot 0
 // holding (A_0, A_{n/2}), both real. Along y, the kx = 0 and kx = n/2 columns are therefore one

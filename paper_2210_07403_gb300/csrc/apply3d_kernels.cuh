@@ -16,7 +16,8 @@
 //   k3_rowifft_gather  band of R y-rows: inverse FFT along x, interpolation into Y (set to ½Q by
 //                      the first kernel), or the grid itself.
 // Layout: spec[f][z][y][kx], kx ∈ [0, n/2), rows z·n + y. The transforms are the register FFT of
-// fft8.cuh (the 2-D kernels' transform): a thread holds eight elements of one lane of a sequence,
+// fft8.cuh (the 2-D kernels' transform): a thread holds eight elements (two on small grids,
+// few_elements_3d) of one lane of a sequence; rows and planes that no stencil meets are not transformed,
 // kThreads3/QT sequences per pass, each sequence in its padded shared-memory buffer (sequence b at
 // b·(n + n/8), the layout the spread's accumulation and the gather's sums index with pidx).
 #pragma once

@@ -1,6 +1,7 @@
 // GMRES for A Q = U_b (Sec. 5.3.2: the Schur operator is not symmetric) on the device.
 //
-// Arnoldi runs on one 16-CTA cluster per iteration (8 where 16 is unavailable; arnoldi.cuh):
+// Arnoldi runs on one 16-CTA cluster per iteration (8 where 16 is unavailable; in batches one of two or
+// four CTAs per problem; arnoldi.cuh):
 // classical Gram–Schmidt against the basis in FP64 with one cluster reduction per step (the
 // second projection of CGS2 is taken from the basis' Gram matrix, h = (2I − G)t), the new
 // Hessenberg column is reduced by the stored Givens rotations, and the residual estimate |g_{k}|
