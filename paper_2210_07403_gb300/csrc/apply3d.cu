@@ -40,9 +40,12 @@ ibdl_status plan_3d(Geometry* g) {
   auto clampp2 = [](int v, int lo, int hi) { v = v < lo ? lo : (v > hi ? hi : v); int r = 1; while (r * 2 <= v) r *= 2; return r; };
   for (int pi = 0; pi < 3; ++pi) {
     const bool f32 = pi == 1;
+    const int lg = __builtin_ctz(n);
+    const int ny = f32 ? y_threads3<float>(lg) : (pi == 0 ? y_threads3<double>(lg) : y_threads3<ff>(lg));
+    const int nz = f32 ? z_threads3<float>(lg) : (pi == 0 ? z_threads3<double>(lg) : z_threads3<ff>(lg));
     // FP32 column CTAs take about 2048 complex elements, FP64 (and float-float, the same element
-    // size) about 1024 (measured on the 128³ sphere).
-    const int target = f32 ? 2048 : 1024;
+    // size) four per thread (measured on the 128³ sphere).
+    const int ytarget = f32 ? 2048 : 4 * ny, ztarget = f32 ? 2048 : 4 * nz;
     // Row bands: tall ones transform untouched rows along with the touched ones and make the
     // fullest band (a pole of the sphere) the kernel's tail, short ones spread a point in more
     // bands and leave threads idle. Applications of the scalar operator on spheres at R = 8 / 16 / 32
@@ -51,21 +54,21 @@ ibdl_status plan_3d(Geometry* g) {
     // / 146, FP64 1740 / 1712 / 1742, float-float 497 / 474 / 501. R ≤ n/2 keeps the wrapped band
     // rows [y0 − 3, y0 + R) distinct (no point counted twice).
     int R = clampp2((pi == 0 || n > 128 ? 16 : 8) / nf, 2, n / 2);
-    int C = clampp2(target / (n * nf), 1, n / 2);
-    int Cz = clampp2(target / 2 / (n * nf), 1, n / 2);
-    // the column passes interleave a pass's kThreads3/(n/8) sequences across the threads of each
-    // warp: fewer sequences than that leave every warp partly idle, and an FP64 warp instruction
-    // costs its issue slot whatever the number of active lanes, so a y pass holds at least
+    int C = clampp2(ytarget / (n * nf), 1, n / 2);
+    int Cz = clampp2(ztarget / 2 / (n * nf), 1, n / 2);
+    // the column passes interleave the sequences of a pass (threads over lanes per sequence) across the
+    // threads of each warp: fewer sequences than that leave every warp partly idle, and an FP64 warp
+    // instruction costs its issue slot whatever the number of active lanes, so a y pass holds at least
     // that many columns (fields × C) and a z pass that many (fields × 2 × Cz)
-    const int sp = kThreads3 / (n / 8);
-    C = std::max(C, clampp2(sp / nf, 1, n / 2));
-    Cz = std::max(Cz, clampp2(sp / (2 * nf), 1, n / 2));
+    const int lanes = n / (f32 ? few_elements_3d<float>(lg) : few_elements_3d<double>(lg));
+    C = std::max(C, clampp2(ny / lanes / nf, 1, n / 2));
+    Cz = std::max(Cz, clampp2(nz / lanes / (2 * nf), 1, n / 2));
     if (const char* e = getenv("IBDL_PLAN3_R")) R = clampp2(atoi(e), 2, n / 2);
     if (const char* e = getenv("IBDL_PLAN3_C")) C = clampp2(atoi(e), 1, n / 2);
     if (const char* e = getenv("IBDL_PLAN3_CZ")) Cz = clampp2(atoi(e), 1, n / 2);
     auto rb = [&](int r) { return f32 ? smem_rows3<float>(n, nf, r) : smem_rows3<double>(n, nf, r); };
-    auto yb = [&](int c) { return f32 ? smem_y3<float>(n, nf, c) : smem_y3<double>(n, nf, c); };
-    auto zb = [&](int c) { return f32 ? smem_z3<float>(n, nf, c) : smem_z3<double>(n, nf, c); };
+    auto yb = [&](int c) { return f32 ? smem_y3<float>(n, nf, c) : (pi == 0 ? smem_y3<double>(n, nf, c) : smem_y3<ff>(n, nf, c)); };
+    auto zb = [&](int c) { return f32 ? smem_z3<float>(n, nf, c) : (pi == 0 ? smem_z3<double>(n, nf, c) : smem_z3<ff>(n, nf, c)); };
     while (R > 2 && rb(R) > kSmemLimit3) R /= 2;
     while (C > 1 && yb(C) > kSmemLimit3) C /= 2;
     while (Cz > 1 && zb(Cz) > kSmemLimit3) Cz /= 2;

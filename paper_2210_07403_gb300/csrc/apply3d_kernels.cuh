@@ -103,11 +103,26 @@ struct FewTw3 {
 // registers), else read from the table at each use.
 //
 // Elements per lane: two in FP64 and float-float where a grid leaves most sub-partitions idle
-// (fft8.cuh). Spheres, applications back to back with eight / two (µs): FP64 16³ 30.9 / 22.8, 32³ 38.9 / 31.5,
-// 64³ 79.3 / 76.9, 128³ 221 / 290; float-float 16³ 24.5 / 17.7, 32³ 30.0 / 22.4, 64³ 51.2 / 58.0.
+// (fft8.cuh). Spheres, applications back to back with eight / two (µs, column passes of 256 threads): FP64
+// 16³ 30.9 / 22.8, 32³ 38.9 / 31.5, 64³ 79.3 / 76.9, 128³ 221 / 290; float-float 16³ 24.5 / 17.7, 32³ 30.0 / 22.4, 64³ 51.2 / 58.0.
 template <typename T>
 constexpr int few_elements_3d(int L) {
   return sizeof(T) != 4 && L <= 5 ? 2 : 8;
+}
+// Threads of the y and z passes on a grid of 2^L. The FP64 passes are bound by the FP64 pipe, so the SM
+// with the most CTAs sets their time: at 128³ the z pass has 520 CTAs of 256 threads, four on some of 152
+// SMs where the mean is 3.4, and 1040 of 128 threads, seven where it is 6.8. On 32³ and 64³ CTAs of 256
+// threads left SMs without any. The y pass of 128³ divides no better in smaller CTAs and loses
+// coalescing, FP32 kernels wait on latency, and 16³ pays for the narrower accesses. Spheres, back to
+// back, 256 / these threads (µs): FP64 32³ 31.5 / 28.2, 64³ 79.2 / 68.2, 128³ 220.8 / 207.6 (the y pass in 128
+// threads too 231), float-float 128³ 109.3 / 107.5; with 64 threads float-float 16³ 17.7 / 18.7, 64³ 50.7 / 51.3.
+template <typename T>
+__host__ __device__ constexpr int y_threads3(int L) {
+  return std::is_same<T, double>::value && (L == 5 || L == 6) ? 64 : kThreads3;
+}
+template <typename T>
+__host__ __device__ constexpr int z_threads3(int L) {
+  return sizeof(T) != 4 && L == 7 ? 128 : y_threads3<T>(L);
 }
 template <typename T, int L>
 struct Cfg3 {
@@ -124,9 +139,9 @@ struct Cfg3 {
 // padded sequence rounded up to ≡ max(1, w/W) (mod w), w = 16 for 8-byte and 8 for 16-byte
 // elements, W = min(32, the sequences of a pass) interleaved in a warp: the rule of the 2-D column
 // groups, which puts the warp's sequences in different shared-memory banks.
-__host__ __device__ constexpr int seq_stride3(int L, int esize, int E) {
+__host__ __device__ constexpr int seq_stride3(int L, int esize, int E, int threads) {
   const int pn = (1 << L) + (1 << L) / 8;
-  const int sp = kThreads3 / ((1 << L) / E);
+  const int sp = threads / ((1 << L) / E);
   const int W = sp < 32 ? sp : 32;
   const int w = esize == 8 ? 16 : 8;
   const int t = (w / W > 1 ? w / W : 1) % w;
@@ -137,15 +152,15 @@ __host__ __device__ constexpr int seq_stride3(int L, int esize, int E) {
 // SP), each exchanging through buf + b·seq_stride3: consecutive threads then touch the same
 // element of consecutive sequences, which the column passes' global accesses want (adjacent kx
 // columns are adjacent in memory). Otherwise sequence b is thread / QT, at buf + b·(n + n/8).
-template <typename T, bool INV, int L, bool IL = false, class LD, class ST>
+template <typename T, bool INV, int L, bool IL = false, int NT = kThreads3, class LD, class ST>
 __device__ __forceinline__ void fft3_run(cplx<T>* buf, int nseq, const cplx<T>* __restrict__ twg, const LD& ld,
                                          const ST& st) {
   using CF = Cfg3<T, L>;
-  constexpr int V = CF::V, E = CF::E, QT = CF::QT, SP = kThreads3 / QT;
+  constexpr int V = CF::V, E = CF::E, QT = CF::QT, SP = NT / QT;
   using F = F8<L, V, E>;
   constexpr int Q = F::Q;
-  static_assert(kThreads3 % QT == 0, "whole sequences per pass");
-  constexpr int PS = IL ? seq_stride3(L, (int)sizeof(cplx<T>), E) : F::PN;
+  static_assert(NT % QT == 0, "whole sequences per pass");
+  constexpr int PS = IL ? seq_stride3(L, (int)sizeof(cplx<T>), E, NT) : F::PN;
   const int sl = IL ? (int)threadIdx.x % SP : (int)threadIdx.x / QT;
   const int j0 = IL ? (int)threadIdx.x / SP : (int)threadIdx.x - sl * QT;
   typename CF::TW tw[V];
@@ -454,13 +469,13 @@ struct YColumnIO {
 };
 
 // the lane of an interleaved column transform that this thread runs (fft3_run with IL)
-template <typename T, int L>
+template <typename T, int L, int NT>
 __device__ __forceinline__ int lane3() {
-  return (int)threadIdx.x / (kThreads3 / Cfg3<T, L>::QT);
+  return (int)threadIdx.x / (NT / Cfg3<T, L>::QT);
 }
 
 template <typename T, bool INV, int L>
-__global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
+__global__ void __launch_bounds__(y_threads3<T>(L)) k3_ypass(Col3Params p) {
   if (p.stop && *p.stop) return;  // final before the wait (see the spread kernel)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int n = 1 << L, nh = n >> 1;
@@ -471,13 +486,13 @@ __global__ void __launch_bounds__(kThreads3) k3_ypass(Col3Params p) {
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
   // the forward pass reads the touched rows of its plane and writes every ky; the inverse the reverse
   constexpr int E = Cfg3<T, L>::E, lq = L - (E == 8 ? 3 : 1);
-  const int j0 = lane3<T, L>();
+  const int j0 = lane3<T, L, y_threads3<T>(L)>();
   const unsigned char* rows = INV ? p.rows_out : p.rows_in;
   const unsigned on = lane_mask3<L, E>(rows ? rows + (size_t)z * (n / 8) : nullptr, j0);
   const YColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, z, k0, p.lc, C, lq, INV ? 0xffu : on, INV ? on : 0xffu};
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
-  fft3_run<T, INV, L, true>(bufA, p.nf * C, static_cast<const cplx<T>*>(p.tw), GlobLd3<YColumnIO<T>>{io},
+  fft3_run<T, INV, L, true, y_threads3<T>(L)>(bufA, p.nf * C, static_cast<const cplx<T>*>(p.tw), GlobLd3<YColumnIO<T>>{io},
                             GlobSt3<YColumnIO<T>>{io});
 }
 
@@ -526,7 +541,7 @@ __device__ __forceinline__ void symbol3(const T* lap1, const T* der1, T lam, T s
 }
 
 template <typename T, int OP, int L>
-__global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
+__global__ void __launch_bounds__(z_threads3<T>(L)) k3_zpass(Col3Params p) {
   if (p.stop && *p.stop) return;  // final before the wait (see the spread kernel)
   constexpr int NIN = Traits3<OP>::NIN;
   constexpr int NOUT = Traits3<OP>::NOUT;
@@ -540,7 +555,8 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
   const int nq = ky1 == ky2 ? 1 : 2;  // y-frequency columns in this CTA
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
   constexpr int E = Cfg3<T, L>::E, lq = L - (E == 8 ? 3 : 1);
-  constexpr int PS = seq_stride3(L, (int)sizeof(cplx<T>), E);  // sequences interleaved (fft3_run)
+  constexpr int NT = z_threads3<T>(L);
+  constexpr int PS = seq_stride3(L, (int)sizeof(cplx<T>), E, NT);  // sequences interleaved (fft3_run)
   T* lap1 = reinterpret_cast<T*>(bufA + (size_t)NMAX * 2 * C * PS);
   T* der1 = lap1 + n;
   const cplx<T>* twg = static_cast<const cplx<T>*>(p.tw);
@@ -548,7 +564,7 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
     lap1[i] = static_cast<const T*>(p.lap1)[i];
     der1[i] = static_cast<const T*>(p.der1)[i];
   }
-  const int j0 = lane3<T, L>();
+  const int j0 = lane3<T, L, NT>();
   const ZColumnIO<T> io{static_cast<cplx<T>*>(p.spec), n, nh, ky1, ky2, k0, lc, C, lq,
                         lane_mask3<L, E>(p.planes_in, j0), lane_mask3<L, E>(p.planes_out, j0)};
   cudaGridDependencySynchronize();
@@ -556,7 +572,7 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
   __syncthreads();
   // with one column (ky = −ky) only the q = 0 sequences exist: sequence index bi maps to
   // (f·2 + 0)·C + c, so transform all 2·C slots per field and ignore q = 1 (it aliases q = 0)
-  fft3_run<T, false, L, true>(bufA, NIN * 2 * C, twg, GlobLd3<ZColumnIO<T>>{io}, SmemSt3<T>());
+  fft3_run<T, false, L, true, NT>(bufA, NIN * 2 * C, twg, GlobLd3<ZColumnIO<T>>{io}, SmemSt3<T>());
   __syncthreads();
   cplx<T>* res = bufA;
   const T lam = T(p.lam), scale = T(p.scale);
@@ -610,7 +626,7 @@ __global__ void __launch_bounds__(kThreads3) k3_zpass(Col3Params p) {
     }
   }
   __syncthreads();
-  fft3_run<T, true, L, true>(bufA, NOUT * 2 * C, twg, SmemLd3<T>(), GlobSt3<ZColumnIO<T>>{io});
+  fft3_run<T, true, L, true, NT>(bufA, NOUT * 2 * C, twg, SmemLd3<T>(), GlobSt3<ZColumnIO<T>>{io});
 }
 
 // ------------------------------------------------------------------------------------------
@@ -732,12 +748,12 @@ __host__ __device__ constexpr size_t smem_rows3(int n, int nf, int R) {
 template <typename T>
 constexpr size_t smem_y3(int n, int nf, int C) {  // host side (launch shapes)
   const int L = __builtin_ctz(n);
-  return (size_t)nf * C * seq_stride3(L, (int)sizeof(cplx<T>), few_elements_3d<T>(L)) * sizeof(cplx<T>);
+  return (size_t)nf * C * seq_stride3(L, (int)sizeof(cplx<T>), few_elements_3d<T>(L), y_threads3<T>(L)) * sizeof(cplx<T>);
 }
 template <typename T>
 constexpr size_t smem_z3(int n, int nf, int C) {  // host side (launch shapes)
   const int L = __builtin_ctz(n);
-  return (size_t)nf * 2 * C * seq_stride3(L, (int)sizeof(cplx<T>), few_elements_3d<T>(L)) * sizeof(cplx<T>) +
+  return (size_t)nf * 2 * C * seq_stride3(L, (int)sizeof(cplx<T>), few_elements_3d<T>(L), z_threads3<T>(L)) * sizeof(cplx<T>) +
          2 * n * sizeof(T);
 }
 
@@ -776,10 +792,10 @@ inline bool use_pdl3() {
 }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch3(void (*kernel)(KArgs...), int grid, size_t smem, cudaStream_t s, Args&&... args) {
+inline cudaError_t launch3(void (*kernel)(KArgs...), int grid, int threads, size_t smem, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads3);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at;
@@ -800,6 +816,7 @@ ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp0, const Col3Params
   constexpr int NIN = Traits3<OP>::NIN, NOUT = Traits3<OP>::NOUT, NMAX = NIN > NOUT ? NIN : NOUT;
   constexpr int n = 1 << L;
   constexpr bool f32 = std::is_same<T, float>::value;
+  constexpr int ny = y_threads3<T>(L), nz = z_threads3<T>(L);
   static std::atomic<unsigned long long> d[6];
   IBDL_CUDA(opt_in_smem3(k3_spread_rowfft<T, OP, L>, d[0]));
   IBDL_CUDA(opt_in_smem3(k3_ypass<T, false, L>, d[1]));
@@ -810,24 +827,24 @@ ibdl_status launch_apply_3d(Geometry* g, const Row3Params& rp0, const Col3Params
   const int groups = (n / 2) / C, z_grid = (n / 2 + 1) * ((n / 2) / Cz);
   const int st0 = f32 ? IBDL_STAGE_SPREAD_ROWFFT_FP32 : IBDL_STAGE_SPREAD_ROWFFT_FP64;
   if (g->timing) timing_mark(g, s, -1);
-  IBDL_CUDA(launch3(k3_spread_rowfft<T, OP, L>, lc.bands_in, smem_rows3<T>(n, NIN, R), s, rp));
+  IBDL_CUDA(launch3(k3_spread_rowfft<T, OP, L>, lc.bands_in, kThreads3, smem_rows3<T>(n, NIN, R), s, rp));
   if (g->timing) timing_mark(g, s, st0);
   Col3Params yp = cp;
   yp.nf = NIN;
   yp.planes = cp.planes_in ? cp.planes : nullptr;
-  IBDL_CUDA(launch3(k3_ypass<T, false, L>, lc.planes_in * groups, smem_y3<T>(n, NIN, C), s, yp));
+  IBDL_CUDA(launch3(k3_ypass<T, false, L>, lc.planes_in * groups, ny, smem_y3<T>(n, NIN, C), s, yp));
   Col3Params zp = cp;
   zp.C = Cz;
   zp.lc = __builtin_ctz(Cz);
-  IBDL_CUDA(launch3(k3_zpass<T, OP, L>, z_grid, smem_z3<T>(n, NMAX, Cz), s, zp));
+  IBDL_CUDA(launch3(k3_zpass<T, OP, L>, z_grid, nz, smem_z3<T>(n, NMAX, Cz), s, zp));
   yp.nf = NOUT;
   yp.planes = cp.planes_out ? cp.planes : nullptr;
-  IBDL_CUDA(launch3(k3_ypass<T, true, L>, lc.planes_out * groups, smem_y3<T>(n, NOUT, C), s, yp));
+  IBDL_CUDA(launch3(k3_ypass<T, true, L>, lc.planes_out * groups, ny, smem_y3<T>(n, NOUT, C), s, yp));
   if (g->timing) timing_mark(g, s, st0 + 1);
   if (lc.grid)
-    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_GRID, L>, lc.bands_out, smem_rows3<T>(n, NOUT, R), s, rp));
+    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_GRID, L>, lc.bands_out, kThreads3, smem_rows3<T>(n, NOUT, R), s, rp));
   else
-    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_INTERP, L>, lc.bands_out, smem_rows3<T>(n, NOUT, R), s, rp));
+    IBDL_CUDA(launch3(k3_rowifft_gather<T, OP, G3_INTERP, L>, lc.bands_out, kThreads3, smem_rows3<T>(n, NOUT, R), s, rp));
   if (g->timing) timing_mark(g, s, st0 + 2);
   g->launches += 5;
   IBDL_CUDA(cudaGetLastError());
