@@ -131,7 +131,7 @@ static ColParams<T> col_params(Geometry* g, const int* stop) {
   cp.tw = static_cast<const cplx<T>*>(Slot2<T>::tw(g));
   cp.stop = stop;
   cp.late = 0;
-  cp.drop0 = g->lambda == 0.0;
+  cp.drop0 = double(cp.lam) == 0.0;  // the λ that the kernel adds: a tiny one rounds to zero in FP32
   cp.err = g->err_dev;
   cp.on_in = cp.on_out = g->row_on;
   return cp;

@@ -266,7 +266,7 @@ struct ColParams {
   const int* stop;
   int* err;  // the staged column pass sets it to 1 when a bounded wait runs out
   int late;  // as in RowParams
-  int drop0;  // the k = 0 mode is dropped: λ = 0, or a spread whose field has no mean (apply_symbol)
+  int drop0;  // the k = 0 mode is dropped: lam = 0, or a spread whose field has no mean (apply_symbol)
   const unsigned char* on_in;   // rows the spread wrote (NULL: every row; the others are zero)
   const unsigned char* on_out;  // rows the last kernel reads (NULL: every row)
 };

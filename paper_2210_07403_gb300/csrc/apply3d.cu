@@ -141,8 +141,9 @@ static ibdl_status run_op3(Geometry* g, const double* in, double* out, cudaStrea
   rp.bands_in = rp.bands_out = nullptr;
   rp.rows_out = cp.rows_in = cp.rows_out = cp.planes_in = cp.planes_out = nullptr;
   cp.planes = g->planes;
-  // (in huge boxes other FP32 wavenumbers underflow too: not told from k = 0)
-  cp.drop0 = cp.lam == 0.0 || (OP == OP3_SCALAR_AN && !grid_in && g->box < 1e12);
+  // (of the λ that the kernel adds: a tiny one rounds to zero in FP32; in huge boxes other FP32 wavenumbers
+  // underflow too: not told from k = 0)
+  cp.drop0 = double(T(cp.lam)) == 0.0 || (OP == OP3_SCALAR_AN && !grid_in && g->box < 1e12);
   if (!grid_in) {
     rp.bands_in = bands;
     cp.rows_in = g->row_on;

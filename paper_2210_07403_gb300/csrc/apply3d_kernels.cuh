@@ -222,7 +222,7 @@ struct Col3Params {
   int n, log2n, C, lc;
   int nf;        // fields transformed (y passes)
   double lam, scale;
-  int drop0;     // the zero mode is dropped: λ = 0, or the spread field has no mean (symbol3)
+  int drop0;     // the zero mode is dropped: T(lam) = 0, or the spread field has no mean (symbol3)
   const void* lap1;
   const void* der1;
   void* spec;
