@@ -526,12 +526,8 @@ __device__ __forceinline__ void symbol3(const T* lap1, const T* der1, T lam, T s
                                         const cplx<T>* in, cplx<T>* out) {
   const T lap = lap1[kx] + lap1[ky] + lap1[kz];
   // (the analytic dipole spread sums to zero: a small λ > 0 would amplify its zero mode's rounding)
-  const bool none = drop0 && sym_zero(lap);
-  T sig;
-  if constexpr (std::is_same<T, float>::value)
-    sig = none ? T(0) : scale / (lap + lam);  // IEEE division: it does not bound these kernels
-  else
-    sig = none ? T(0) : sym_div(scale, lap + lam);
+  // IEEE division in FP32 and FP64
+  const T sig = drop0 && sym_zero(lap) ? T(0) : scale / (lap + lam);
   if (OP == OP3_SCALAR_AN || OP == OP3_ADJ_AN) {
     out[0] = cscale(in[0], sig);
   } else if (OP == OP3_SCALAR_SD) {

@@ -53,21 +53,10 @@ __device__ __forceinline__ void dft8(cplx<T>* u) {
 __device__ __forceinline__ bool sym_zero(float a) { return a == 0.0f; }
 __device__ __forceinline__ bool sym_zero(double a) { return __double_as_longlong(a) == 0; }
 
-// a/b of a Fourier symbol: the hardware reciprocal estimate in FP32 (within 2 ulp, well inside the
-// FP32 application's rounding), a corrected quotient in float-float. In FP64 the hardware estimate r
-// (about 20 bits; no FP64-pipe instruction) with one third-order step for the reciprocal,
-// r(1 + e + e²), e = 1 − b·r, whose error e³ lies below FP64 rounding: four FP64 instructions instead
-// of the division's ten or so, on the pipe that bounds FP64 applications. Where b or its reciprocal
-// is not a normal number in a comfortable range, IEEE division.
+// a/b of a Fourier symbol: the hardware reciprocal estimate in 2-D FP32 (within 2 ulp, well inside the
+// FP32 application's rounding), a corrected quotient in float-float, IEEE division in FP64
 __device__ __forceinline__ float sym_div(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double sym_div(double a, double b) {
-  const int ex = (__double2hiint(b) >> 20) & 0x7ff;
-  if (ex < 64 || ex > 1983) return a / b;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
-  const double e = fma(-b, r, 1.0);
-  return a * fma(r, fma(e, e, e), r);
-}
+__device__ __forceinline__ double sym_div(double a, double b) { return a / b; }
 
 // The 3-D row kernels' buffers are padded with one element after every eight, which keeps the
 // radix-8 stride-8 writes of the first stages free of bank conflicts for 8- and 16-byte elements.
