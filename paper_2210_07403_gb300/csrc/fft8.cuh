@@ -26,8 +26,9 @@
 // Process. 41 (1993) 93–107, and Goedecker, SIAM J. Sci. Comput. 18 (1997) 1605–1611, describe such
 // forms): 72 instructions instead of 84 for seven complex products and the 8-point DFT; the first
 // stage's √½ factors go into its last additions (52 instead of 56). The error of c·(b_x − t·b_y)
-// is that of c·b_x − s·b_y, however large t is. The table then holds (c, t), and a
-// lane needs four entries per radix-8 stage instead of seven. FP64 applications before / after: 512²
+// is that of c·b_x − s·b_y, however large t is; b·(1 + i·t) exceeds w·b by at most 1/c < n/6 (quarter
+// turns, c = 0, are treated apart), which is the headroom the form takes off the FP64 range. The table then
+// holds (c, t), and a lane needs four entries per radix-8 stage instead of seven. FP64 applications before / after: 512²
 // Stokes star 131 / 118 µs, 2048² (finite differences, divergence dipole) 791 / 671 µs, 128³ sphere 261 /
 // 249 µs; the error against an 80-bit reference is unchanged (64² circle 4.2e−15 of S*u, 1024² 3.7e−14 /
 // 3.6e−14, 128³ 2.4e−15), which the kernel tables' rounding sets.
@@ -146,11 +147,20 @@ __device__ __forceinline__ cplx<T> cmul_tw(cplx<T> a, cplx<T> w) {
   return INV ? mk(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y) : mk(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
 }
 
-// (a, b) ← (a + w·b, a − w·b) with w = c(1 + i·t) given as (c, t) (INV: conj w; ROT: times −i, INV i)
-template <typename T, bool INV, bool ROT>
+// whether a table entry stands for −i, by its high words (off the FP64 pipe)
+__device__ __forceinline__ bool quarter_turn(cplx<double> w) {
+  return __double2hiint(w.x) == 0x3ff00000 && __double2hiint(w.y) == (int)0xbff00000;  // 1, −1
+}
+
+// (a, b) ← (a + w·b, a − w·b) with w = c(1 + i·t) given as (c, t) (INV: conj w; ROT: times −i, INV i).
+// A quarter turn has no tangent: the table holds (1, −1) for it, which is no angle's pair, and with QTR
+// (the butterflies whose twiddle can be one) p = ∓i·b then leaves the other part out. (A huge tangent
+// in its place would overflow on data far below the top of the FP64 range.)
+template <typename T, bool INV, bool ROT, bool QTR = false>
 __device__ __forceinline__ void bfly_tan(cplx<T>& a, cplx<T>& b, cplx<T> w) {
   const T t = INV ? -w.y : w.y;
-  cplx<T> p = mk(fma(-t, b.y, b.x), fma(t, b.x, b.y));
+  const bool q = QTR && quarter_turn(w);
+  cplx<T> p = mk(fma(-t, b.y, q ? T(0) : b.x), fma(t, b.x, q ? T(0) : b.y));
   if (ROT) p = rot90<T, INV>(p);
   b = mk(fma(-w.x, p.x, a.x), fma(-w.x, p.y, a.y));
   a = mk(fma(w.x, p.x, a.x), fma(w.x, p.y, a.y));
@@ -161,7 +171,7 @@ template <typename T, bool INV>
 __device__ __forceinline__ void dft8_tan(cplx<T> (&x)[8], cplx<T> w1, cplx<T> w2, cplx<T> w4, cplx<T> w1e) {
   // t mod 2 from the pairs (r, r + 4): x[r], x[r + 4]
 #pragma unroll
-  for (int r = 0; r < 4; ++r) bfly_tan<T, INV, false>(x[r], x[r + 4], w4);
+  for (int r = 0; r < 4; ++r) bfly_tan<T, INV, false, true>(x[r], x[r + 4], w4);
   // t mod 4 from the pairs (r, r + 2): t = 0, 2 in (x0, x2), (x1, x3); 1, 3 in (x4, x6), (x5, x7)
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -211,13 +221,13 @@ __device__ __forceinline__ void f8_stage(cplx<T> (&x)[8], const TW& tw) {
       dft8_tan<T, INV>(x, w[0], w[1], w[2], w[3]);
     } else if constexpr (LT == 1) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) bfly_tan<T, INV, false>(x[m], x[m + 4], w[m]);
+      for (int m = 0; m < 4; ++m) bfly_tan<T, INV, false, true>(x[m], x[m + 4], w[m]);
     } else {
       // radix 4: inputs and outputs of butterfly m at x[m + 2r], r = 0 … 3
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        bfly_tan<T, INV, false>(x[m], x[m + 4], w[2 * m + 1]);
-        bfly_tan<T, INV, false>(x[m + 2], x[m + 6], w[2 * m + 1]);
+        bfly_tan<T, INV, false, true>(x[m], x[m + 4], w[2 * m + 1]);
+        bfly_tan<T, INV, false, true>(x[m + 2], x[m + 6], w[2 * m + 1]);
         bfly_tan<T, INV, false>(x[m], x[m + 2], w[2 * m]);     // outputs 0, 2
         bfly_tan<T, INV, true>(x[m + 4], x[m + 6], w[2 * m]);  // outputs 1, 3
         const cplx<T> y1 = x[m + 4], y2 = x[m + 2];
@@ -418,7 +428,7 @@ struct TwFew {
 template <typename T, bool INV>
 __device__ __forceinline__ void bfly(cplx<T>& a, cplx<T>& b, cplx<T> w) {
   if constexpr (kFused8<T>) {
-    bfly_tan<T, INV, false>(a, b, w);
+    bfly_tan<T, INV, false, true>(a, b, w);
   } else {
     const cplx<T> t = cmul_tw<T, INV>(b, w);
     b = csub(a, t);
@@ -445,8 +455,8 @@ __device__ __forceinline__ void few_fft(cplx<T> (&x)[E], cplx<T>* buf, int j, co
         dft4<T, INV>(x[0], x[1], x[2], x[3]);
       } else if constexpr (kFused8<T>) {
         const cplx<T> w1 = tw.w[(S - 1) * Y::NV], w2 = tw.w[(S - 1) * Y::NV + 1];
-        bfly_tan<T, INV, false>(x[0], x[2], w2);
-        bfly_tan<T, INV, false>(x[1], x[3], w2);
+        bfly_tan<T, INV, false, true>(x[0], x[2], w2);
+        bfly_tan<T, INV, false, true>(x[1], x[3], w2);
         bfly_tan<T, INV, false>(x[0], x[1], w1);  // outputs 0, 2
         bfly_tan<T, INV, true>(x[2], x[3], w1);   // outputs 1, 3
         const cplx<T> y1 = x[2], y2 = x[1];

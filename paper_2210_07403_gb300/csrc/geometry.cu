@@ -115,8 +115,8 @@ __global__ void k_tables(int dim, int n, int M, int delta, const double* __restr
 
 // The twiddle table of n-point transforms (TwLayout in fft8.cuh, here for a runtime n): thread e
 // writes the values of chunk e. A value is e^{−2πi m/n} = (c, s), or (c, t) with t = s/c for the FP64
-// transforms' fused form. There, at a quarter turn, where c = 0, c = 2^−60 stands for it:
-// c·(b_x − t·b_y) with t = −2^60 is then −s·b_y to rounding (the term 2^−60·b_x lies below it).
+// transforms' fused form. A quarter turn, where c = 0, is marked by (1, s) (bfly_tan); the angles of the
+// tables stay below half a turn, so s = −1.
 static __host__ __device__ int tw_chunks8(bool fused, int per) { return ((fused ? 4 : 7) + per - 1) / per; }
 static __host__ __device__ int tw_values_tail(int lt, bool fused) {
   return lt == 0 ? 0 : (fused ? lt : (1 << lt) - 1) * (8 >> lt);
@@ -132,8 +132,7 @@ template <typename T>
 __device__ void tw_put(cplx<T>* p, double c, double s) { *p = mk(T(c), T(s)); }
 template <>
 __device__ void tw_put<double>(cplx<double>* p, double c, double s) {
-  const double cc = c == 0.0 ? 0x1p-60 : c;
-  *p = mk(cc, s / cc);
+  *p = c == 0.0 ? mk(1.0, s) : mk(c, s / c);
 }
 template <typename T>
 __global__ void k_twiddles(int L, int chunks, cplx<T>* tw) {
