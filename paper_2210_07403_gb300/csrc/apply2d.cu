@@ -825,7 +825,8 @@ void shape_for_target_2d(Geometry* g, int pi, int row_target, int col_target, in
 // and 512; never smaller than the geometry's own), 256 threads in the row kernels. Scalar ellipses,
 // a third each of n, n/2 and n/4, geometry's own / these / autotuned shapes (µs): 256 to 512² FP32
 // 353 / 176 / 174, FP64 3177 / 2670 / 2650, float-float 1235 / 749 / 714; 64 to 512² FP32 109 / 69 / 69;
-// 64 to 256² FP32 59 / 46 / 43; 4 to 512² (the geometry's own are kept) FP32 36 / 41 / 37.
+// 64 to 256² FP32 59 / 46 / 43; 4 to 512² (the geometry's own are kept) FP32 36 / 41 / 37. What the
+// environment or single-problem tuning has set (shape_set) stays as it is.
 void batch_shapes_2d(Batch* B) {
   for (int pi = 0; pi < 3; ++pi) {
     const int row_target = pi == 0 ? 1024 : 2048, col_target = pi == 0 ? 512 : 1024;
@@ -837,14 +838,15 @@ void batch_shapes_2d(Batch* B) {
     }
     for (int b = 0; b < B->count; ++b) {
       Geometry* g = B->geoms[b];
-      g->threads[pi] = 256;
+      const int set = g->shape_set[pi];
+      if (!(set & SHAPE_THREADS)) g->threads[pi] = 256;
       if (units[log2i(g->n)] <= 2 * 152 || g->split[pi]) continue;
       int R = std::max(g->rows_per_cta[pi], 2 * pow2_in(row_target / g->n, 1, g->n / 4));
       while (R > g->rows_per_cta[pi] && !row_fits(g, pi, R)) R /= 2;
       int C = std::max(g->cols_per_cta[pi], pow2_in(col_target / (g->n * nf_row_max(g)), 1, g->n / 2));
       while (C > g->cols_per_cta[pi] && !col_fits(g, pi, C)) C /= 2;
-      g->rows_per_cta[pi] = R;
-      g->cols_per_cta[pi] = C;
+      if (!(set & SHAPE_ROWS)) g->rows_per_cta[pi] = R;
+      if (!(set & SHAPE_COLS)) g->cols_per_cta[pi] = C;
     }
   }
 }
@@ -882,11 +884,11 @@ ibdl_status plan_2d(Geometry* g) {
     }
     if (const char* e = getenv("IBDL_PLAN_R")) {
       const int v = atoi(e);
-      if ((v & (v - 1)) == 0 && row_fits(g, pi, v)) R = v;
+      if ((v & (v - 1)) == 0 && row_fits(g, pi, v)) R = v, g->shape_set[pi] |= SHAPE_ROWS;
     }
     if (const char* e = getenv("IBDL_PLAN_C")) {
       const int v = atoi(e);
-      if (v >= 1 && (v & (v - 1)) == 0 && col_fits(g, pi, v)) C = v;
+      if (v >= 1 && (v & (v - 1)) == 0 && col_fits(g, pi, v)) C = v, g->shape_set[pi] |= SHAPE_COLS;
     }
     if (R == 0 || C == 0) R = C = 0;
     g->rows_per_cta[pi] = R;
@@ -902,12 +904,14 @@ ibdl_status plan_2d(Geometry* g) {
       g->rows_per_cta[pi] = tv.R;
       g->cols_per_cta[pi] = tv.C;
       g->threads[pi] = tv.floor;
+      g->shape_set[pi] = SHAPE_ROWS | SHAPE_COLS | SHAPE_THREADS;
       if (pi == 1) tuned_stage = tv.staged;
     }
   }
   if (const char* e = getenv("IBDL_THREADS")) {
     const int v = atoi(e);
-    if (v >= 0 && v <= kMaxThreads2d && v % 32 == 0) g->threads[0] = g->threads[1] = g->threads[2] = v;
+    if (v >= 0 && v <= kMaxThreads2d && v % 32 == 0)
+      for (int pi = 0; pi < 3; ++pi) g->threads[pi] = v, g->shape_set[pi] |= SHAPE_THREADS;
   }
   if (g->rows_per_cta[0] == 0 && g->rows_per_cta[1] == 0)
     return fail(IBDL_ERR_UNSUPPORTED, "grid too large for the shared-memory FFT");

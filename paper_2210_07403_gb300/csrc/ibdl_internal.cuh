@@ -80,6 +80,7 @@ struct PointTable {
   T* nrm;      // [dim][M] unit normals
 };
 
+enum { SHAPE_ROWS = 1, SHAPE_COLS = 2, SHAPE_THREADS = 4 };
 struct Geometry {
   // description
   int dim, n, pde, delta, dipole, symbol;
@@ -142,6 +143,7 @@ struct Geometry {
   int zcols_per_cta[3];  // 3-D: kx columns per CTA in the z pass
   size_t smem_row[2], smem_col[2], smem_row_inv[2];
   int threads[3];        // 2-D: least threads per CTA of the row kernels (0: none)
+  int shape_set[3];      // 2-D: which of these the environment or the autotuner has set (SHAPE_*)
   int split[3];          // 2-D: one field per launch (the fields' row bands or columns do not fit
                          // shared memory together, or IBDL_SPLIT_FIELDS=1)
 
