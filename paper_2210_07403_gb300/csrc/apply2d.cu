@@ -555,7 +555,7 @@ static ibdl_status batch_prepare_staged(Batch* B) {
     IBDL_TRY(encode_col_map(g->spec, g->n, g->rows_per_cta[1], g->cols_per_cta[1], spec_fields_fp32(g), &maps[b]));
   }
   IBDL_CUDA(cudaMalloc((void**)&B->tmaps, sizeof(CUtensorMap) * B->count));
-  IBDL_CUDA(cudaMemcpy(B->tmaps, maps.data(), sizeof(CUtensorMap) * B->count, cudaMemcpyHostToDevice));
+  IBDL_CUDA(copy_in(B->tmaps, maps.data(), sizeof(CUtensorMap) * B->count));
   return IBDL_OK;
 }
 
@@ -616,7 +616,7 @@ static ibdl_status batch_prepare_t(Batch* B, const int* kptr /* device &st[b].k,
     if (*dst) cudaFree(*dst);
     *dst = nullptr;
     IBDL_CUDA(cudaMalloc(dst, bytes));
-    IBDL_CUDA(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
+    IBDL_CUDA(copy_in(*dst, src, bytes));
     return IBDL_OK;
   };
   IBDL_TRY(upload(&B->rowp[pi][0], user.data(), sizeof(RowParams<T>) * B->count));

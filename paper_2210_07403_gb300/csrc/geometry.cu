@@ -306,11 +306,12 @@ static ibdl_status dalloc(P** p, size_t bytes) {
 }
 
 // The rows some stencil meets (a point of base row b meets rows b … b + 3, wrapped; in 3-D likewise
-// planes) and the bands that hold such rows, from the cell counts, read back once per geometry.
-static ibdl_status touched_rows(Geometry* g) {
+// planes) and the bands that hold such rows, from the cell counts, read back once per geometry on its stream.
+static ibdl_status touched_rows(Geometry* g, cudaStream_t s) {
   const int n = g->n, Q = n / 8, planes = g->dim == 3 ? n : 1;
   std::vector<int> start(g->ncell + 1);
-  IBDL_CUDA(cudaMemcpy(start.data(), g->cell_start, sizeof(int) * (g->ncell + 1), cudaMemcpyDeviceToHost));
+  IBDL_CUDA(cudaMemcpyAsync(start.data(), g->cell_start, sizeof(int) * (g->ncell + 1), cudaMemcpyDeviceToHost, s));
+  IBDL_CUDA(cudaStreamSynchronize(s));
   // points whose stencils meet the rows [r0, r0 + R) (wrapped) of plane z
   auto points = [&](int z, int r0, int R) {
     int c = 0;
@@ -373,7 +374,7 @@ static ibdl_status touched_rows(Geometry* g) {
   g->row_on = d + bytes;
   g->plane_on = g->row_on + on.size();
   g->nplanes = (int)zs.size();
-  IBDL_CUDA(cudaMemcpy(d, all.data(), all.size(), cudaMemcpyHostToDevice));
+  IBDL_CUDA(copy_in(d, all.data(), all.size(), s));
   return IBDL_OK;
 }
 
@@ -623,7 +624,7 @@ ibdl_status create_geometry(const ibdl_geometry_desc* d, cudaStream_t s, Geometr
     GCUDA(cudaHostAlloc((void**)&g->err_host, sizeof(int), cudaHostAllocMapped));
     *g->err_host = 0;
     GCUDA(cudaHostGetDevicePointer((void**)&g->err_dev, g->err_host, 0));
-    GTRY(touched_rows(g));
+    GTRY(touched_rows(g, s));
     GTRY(dim == 2 ? plan_2d(g) : plan_3d(g));
   }
   g->X64 = dX;  // kept: the near-boundary interpolation decides on the caller's coordinates

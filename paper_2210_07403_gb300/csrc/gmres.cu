@@ -836,7 +836,7 @@ static ibdl_status batch_workspace(Batch* B, int m, const ArnoldiCfg& c) {
     if (*dst) cudaFree(*dst);
     *dst = nullptr;
     IBDL_CUDA(cudaMalloc(dst, bytes));
-    IBDL_CUDA(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
+    IBDL_CUDA(copy_in(*dst, src, bytes));
     return IBDL_OK;
   };
   std::vector<int64_t> off(B->off, B->off + B->count);

@@ -312,6 +312,13 @@ ibdl_status apply_2d_indexed(Geometry* g, int precision, double* V, const int* i
 ibdl_status apply_3d_indexed(Geometry* g, int precision, double* V, const int* idx, int nd, cudaStream_t s,
                              const int* stop, int op = OPK_A);
 
+// host tables to the device, there for every stream when it returns (cudaMemcpy from pageable memory may
+// return while the last part of the copy is still under way, ordered with the legacy stream only)
+inline cudaError_t copy_in(void* dst, const void* src, size_t bytes, cudaStream_t s = nullptr) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(s);
+}
+
 // IBDL_ERR_TIMEOUT (and the flag cleared) if a staged column pass of this geometry gave up waiting
 // for its copies since the last check; the flag lives in mapped host memory, so no copy is needed
 inline ibdl_status take_device_error(Geometry* g) {
