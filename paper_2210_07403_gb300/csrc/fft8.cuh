@@ -398,13 +398,13 @@ __device__ __forceinline__ void f8_fft(cplx<T> (&x)[FL][V][8], cplx<T>* buf, int
 // ------------------------------------------------------------------------------------------
 __host__ __device__ constexpr int ipow(int b, int e) { return e == 0 ? 1 : b * ipow(b, e - 1); }
 
-// Twiddles: NV values per stage S ≥ 1 and k = j mod E^S (E = 2: w; E = 4: w, w², w³, or w, w² in the fused
-// form), then for the tail two per lane j (w of i = j, j + Q); 16-byte values, value c of k at
-// offset(S) + c·E^S + k.
+// Twiddles: NV values per stage S ≥ 1 and k = j mod E^S (E = 2: w; E = 4: w, w², w³), then for the tail two per
+// lane j (w of i = j, j + Q); 16-byte values, value c of k at offset(S) + c·E^S + k.
 template <typename T, int L, int E>
 struct FewLayout {
+  static_assert(E == 2 || !kFused8<T>, "four elements per lane: float-float only (no fused radix-4 stage)");
   static constexpr int LE = E == 2 ? 1 : 2, NS = L / LE, LT = L % LE, Q = (1 << L) / E;
-  static constexpr int NV = E == 2 ? 1 : (kFused8<T> ? 2 : 3), NT = LT ? 2 : 0;
+  static constexpr int NV = E - 1, NT = LT ? 2 : 0;
   __host__ __device__ static constexpr int offset(int S) { return NV * ((ipow(E, S) - E) / (E - 1)); }
   static constexpr int NTW = NV * (NS - 1) + NT;
 };
@@ -453,15 +453,6 @@ __device__ __forceinline__ void few_fft(cplx<T> (&x)[E], cplx<T>* buf, int j, co
         bfly<T, INV>(x[1], x[3], tw.w[(S - 1) * Y::NV + 1]);
       } else if constexpr (S == 0) {
         dft4<T, INV>(x[0], x[1], x[2], x[3]);
-      } else if constexpr (kFused8<T>) {
-        const cplx<T> w1 = tw.w[(S - 1) * Y::NV], w2 = tw.w[(S - 1) * Y::NV + 1];
-        bfly_tan<T, INV, false, true>(x[0], x[2], w2);
-        bfly_tan<T, INV, false, true>(x[1], x[3], w2);
-        bfly_tan<T, INV, false>(x[0], x[1], w1);  // outputs 0, 2
-        bfly_tan<T, INV, true>(x[2], x[3], w1);   // outputs 1, 3
-        const cplx<T> y1 = x[2], y2 = x[1];
-        x[1] = y1;
-        x[2] = y2;
       } else {
 #pragma unroll
         for (int r = 1; r < 4; ++r) x[r] = cmul_tw<T, INV>(x[r], tw.w[(S - 1) * Y::NV + r - 1]);

@@ -173,7 +173,7 @@ template <typename T>
 __global__ void k_twiddles_few(int L, int E, int count, cplx<T>* tw) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= count) return;
-  const int n = 1 << L, NS = E == 2 ? L : L / 2, nv = E == 2 ? 1 : (kFused8<T> ? 2 : 3);
+  const int n = 1 << L, NS = E == 2 ? L : L / 2, nv = E - 1;
   int S = 1, p = E, off = 0;
   while (S < NS && e >= off + nv * p) {
     off += nv * p;
