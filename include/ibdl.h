@@ -40,7 +40,8 @@
  *   IBDL_ARNOLDI_CLUSTER=8   run the Arnoldi step on 8-CTA clusters even where 16 fit;
  *   IBDL_PLAN_R, IBDL_PLAN_C, IBDL_THREADS   2-D launch shape before autotuning (rows per CTA of
  *                            the row kernels, columns per CTA of the column pass, least threads
- *                            per CTA of the row kernels);
+ *                            per CTA of the row kernels); a batch keeps what these or
+ *                            ibdl_autotune set and chooses the rest by its problems' count;
  *   IBDL_PLAN3_R, IBDL_PLAN3_C, IBDL_PLAN3_CZ   the same for the 3-D kernels;
  *   IBDL_BATCH_PERSISTENT=1  batched column passes of the scalar operator on persistent CTAs
  *                            that load the next unit before transforming the current one,

@@ -646,9 +646,12 @@ ibdl_status batch_prepare_2d(Batch* B) {
 }
 
 // ------------------------------------------------------------------------------------------
-// launch shapes. A row kernel's CTA has (R/2)·QT threads and a column kernel's C·QT, with
-// QT = n/8 threads per transform (n/16 at n = 8192); both hold one padded sequence of n + n/8
-// complex values per field and row pair (column) in shared memory.
+// launch shapes. A transform of n = 2^L points runs on QT threads (threads_per_seq_2d): n/8 with one lane of
+// eight elements per thread, half or a quarter of that where a thread holds two or four lanes, n/2 or n/4 on
+// small grids with two or four elements per lane. A row kernel's CTA has (R/2)·QT threads per field group and
+// a column kernel's C·QT, a group of several filling up its last warp (group_threads_2d). Both hold one padded
+// sequence per field and row pair (column) in shared memory: n + n/8 complex values, n + n/16 in the FP32
+// 8192² row kernels (row_pad_2d), plus the shift that col_stride_2d adds where sequences interleave.
 // ------------------------------------------------------------------------------------------
 static int nf_row_max(const Geometry* g) { return g->nf_in > g->nf_out ? g->nf_in : g->nf_out; }
 

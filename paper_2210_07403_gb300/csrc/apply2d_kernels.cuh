@@ -104,7 +104,7 @@ __host__ __device__ constexpr int threads_per_seq_2d(int L, bool f32, int E = 8)
 
 // Elements per lane of a single problem's FP64 and float-float kernels with two-row bands and single
 // columns, where a grid leaves most of the GPU idle (8: the ordinary kernels only). An FP64 warp
-// instruction takes about 64 cycles whatever its active lanes, so the 312 instructions of a 64-point
+// instruction takes 64 to 76 cycles whatever its active lanes, so the 312 instructions of a 64-point
 // column on eight lanes took 10 µs on one sub-partition, three of four idle. Applications back to back
 // with 8 / few elements (µs): FP64 scalar 64² 32.1 / 13.6, 256² 41.3 / 21.9, Stokes 64² 37.0 / 17.4, 256² 49.8 /
 // 37.9; float-float scalar 64² 23.4 / 11.0, 256² 30.1 / 15.9, 512² (four elements) 29.5 / 21.8, Stokes 512² 49.0 /
@@ -453,8 +453,8 @@ __device__ __forceinline__ void spread_rowfft_body(const RowParams<T>& p, int or
       pout[i] = p.jump * pin[i] + (p.aug ? pin[NC * M + i / M] : 0.0);
   __syncthreads();  // the accumulation buffer is cleared
   if (p.aug && ord == 0 && first) {
-    // constraint rows of the completed method: η Σ_i Δs_i Q_{l,i} (Δs = wscale·h^d); the block
-    // size is a power of two (a partial warp below 32 threads), the partial sums go to the
+    // constraint rows of the completed method: η Σ_i Δs_i Q_{l,i} (Δs = wscale·h^d); the block size is a
+    // multiple of 32, or one partial warp of a power of two of threads; the partial sums go to the
     // reduction slots after the sequence buffers
     double* red = reinterpret_cast<double*>(buf + (size_t)NB * half * PN);
     const int wl = blockDim.x < 32 ? blockDim.x : 32;

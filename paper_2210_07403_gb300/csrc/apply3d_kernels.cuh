@@ -113,9 +113,12 @@ constexpr int few_elements_3d(int L) {
 // with the most CTAs sets their time: at 128³ the z pass has 520 CTAs of 256 threads, four on some of 152
 // SMs where the mean is 3.4, and 1040 of 128 threads, seven where it is 6.8. On 32³ and 64³ CTAs of 256
 // threads left SMs without any. The y pass of 128³ divides no better in smaller CTAs and loses
-// coalescing, FP32 kernels wait on latency, and 16³ pays for the narrower accesses. Spheres, back to
-// back, 256 / these threads (µs): FP64 32³ 31.5 / 28.2, 64³ 79.2 / 68.2, 128³ 220.8 / 207.6 (the y pass in 128
-// threads too 231), float-float 128³ 109.3 / 107.5; with 64 threads float-float 16³ 17.7 / 18.7, 64³ 50.7 / 51.3.
+// coalescing, FP32 kernels wait on latency, 16³ pays for the narrower accesses, and 256³ has so many CTAs that
+// no SM is left behind. Spheres, back to back, 256 / these threads (µs): FP64 32³ 31.5 / 28.2, 64³ 79.2 / 68.2,
+// 128³ 220.8 / 207.6 (the y pass in 128 threads too 231, both passes in 64 237), float-float 128³ 109.3 / 107.5.
+// Where 256 stays, 256 / fewer: float-float 16³ 17.7 / 18.7 and 64³ 50.7 / 51.3 (64 threads), FP32 64³ 20.9 / 22.3
+// (128), 256³ FP64 1372 / 1356 and float-float 467 / 483 (128; neither by much, so both keep one size). FP64
+// and float-float share the z pass's rule at 128³ because both measured faster there.
 template <typename T>
 __host__ __device__ constexpr int y_threads3(int L) {
   return std::is_same<T, double>::value && (L == 5 || L == 6) ? 64 : kThreads3;

@@ -339,9 +339,9 @@ static ibdl_status build_cycle_graph(Geometry* g, int prec, int m, int op, cudaG
 // Iterations (application + Arnoldi step) per body of the captured while loop. Inside a body the
 // kernels follow each other with programmatic launch; between bodies the graph waits for the
 // body to finish and re-evaluates the loop condition (about 4 µs), and the slots of the last body
-// after the stop still launch their kernels, which return at once (4 to 8 µs per slot). A mixed
-// solve stops once per refinement sweep, after 3 to 13 iterations, so short bodies pay: mixed solves
-// to 1e−10 with bodies of 2 / 4 / 5 / 8 / 12: 512² Stokes star 1084 / 1046 / 1104 / 1086 / 1052 µs, 64² circle
+// after the stop still launch their kernels, which return at once (4 µs per slot on the 64² circle, 5.5 on the
+// star, 6 to 8 with the six kernels of the 128³ sphere). A mixed solve stops once per refinement sweep, after
+// 3 to 13 iterations, so short bodies pay: mixed solves to 1e−10 with bodies of 2 / 4 / 5 / 8 / 12: 512² Stokes star 1084 / 1046 / 1104 / 1086 / 1052 µs, 64² circle
 // 408 / 402 / 421 / 461 / 511, 32³ sphere 529 / 521 / 532 / 597 / 672, 128³ sphere (two problems) 891, 984 / 919,
 // 1010 / 858, 969 / 909, 1073 / 976, 1147; FP64 solves (8 iterations) 512² circle 526 / 513 / 527 / 511 / 536.
 // IBDL_UNROLL=u (1..16) overrides.

@@ -2,8 +2,8 @@
 
     python -m paper_2210_07403_gb300.profile --workload star512 --precision fp32 --repeat 1
 
-builds the workload's geometry (or batch), autotunes its launch shapes as bench.py does, warms up
-with three applications, then runs `--repeat` applications between cudaProfilerStart and
+builds the workload's geometry (or batch), autotunes its launch shapes as bench.py does (`--shapes default`:
+leaves the library's default ones), warms up with three applications, then runs `--repeat` applications between cudaProfilerStart and
 cudaProfilerStop, so that `ncu --profile-from-start off` captures exactly those kernels.
 
 Workloads (synthetic, seeded, as in ibdl_inputs):
@@ -21,7 +21,7 @@ import sys
 import numpy as np
 
 
-def _build(workload: str, dev):
+def _build(workload: str, dev, tune: bool):
     import torch
 
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -35,7 +35,8 @@ def _build(workload: str, dev):
     if workload == "batch256":
         probs = I.ellipse_batch(256)
         B = Batch(probs)
-        B.autotune()
+        if tune:
+            B.autotune()
         q = torch.from_numpy(np.concatenate([p.Ub.reshape(-1) for p in probs])).to(dev)
         return B, q
     if workload == "star512":
@@ -50,7 +51,8 @@ def _build(workload: str, dev):
     else:
         raise SystemExit(f"unknown workload {workload!r}")
     g = Geometry.from_problem(p)
-    g.autotune()
+    if tune:
+        g.autotune()
     return g, torch.from_numpy(p.Ub.reshape(-1).copy()).to(dev)
 
 
@@ -58,6 +60,7 @@ def main(argv=None):
     ap = argparse.ArgumentParser(description=__doc__, formatter_class=argparse.RawDescriptionHelpFormatter)
     ap.add_argument("--workload", default="star512")
     ap.add_argument("--precision", default="fp32", choices=["fp64", "fp32", "fp32x2"])
+    ap.add_argument("--shapes", default="tuned", choices=["tuned", "default"])
     ap.add_argument("--repeat", type=int, default=1)
     args = ap.parse_args(argv)
     import torch
@@ -68,7 +71,7 @@ def main(argv=None):
     b.build()
     ibdl.load()
     dev = torch.device("cuda", 0)
-    obj, q = _build(args.workload, dev)
+    obj, q = _build(args.workload, dev, args.shapes == "tuned")
     y = torch.empty_like(q)
     for _ in range(3):
         obj.apply(q, y, precision=args.precision)
